@@ -492,12 +492,14 @@ static int side_stream(int device, cudaStream_t caller, SideStream* out)
     return 0;
 }
 
-// Queries per work-list item: the default, or `group` when it is in range
-// (1..128 for the tensor-core screen, whose MMA tile has 128 query rows;
-// 1..group_size for the fp32 tile scan, whose thread layout fixes the most).
+// Queries per work-list item: the default (two MMA tiles of 128 query rows on
+// the tensor-core screen), or `group` when it is in range (1..128 for the
+// screen; 1..group_size for the fp32 tile scan, whose thread layout fixes the
+// most).
 static int item_group(const osann_index* ix, int mode, int group)
 {
-    const int gmax = tc_mode(mode) ? TC_GROUP : group_size(ix->d_pad);
+    if (tc_mode(mode)) return group >= 1 && group <= TC_GROUP ? group : 2 * TC_GROUP;
+    const int gmax = group_size(ix->d_pad);
     return group >= 1 && group <= gmax ? group : gmax;
 }
 
@@ -1372,8 +1374,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                     radius, b, reinterpret_cast<uint32_t*>(w + L.ubits),
                                     reinterpret_cast<uint32_t*>(w + L.scnt), reinterpret_cast<uint32_t*>(w + L.surv),
                                     TC_SURV_CAP, ix->status, ix->diag, ix->xs, Y, P_eff, ix->d, ix->d_pad, k,
-                                    ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms,
-                                    layout);
+                                    ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms);
             }
             if (!rc) {
                 StageScope s(OSANN_STAGE_TC_RERANK, st);

@@ -154,7 +154,7 @@ int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int
 
 // tc_scan.cu: 16-bit tensor-core screening + fp32 rerank.  prec 0 = bf16,
 // 1 = fp16 (with an exact power-of-two scale of the data and queries)
-constexpr int TC_GROUP = 128;
+constexpr int TC_GROUP = 128;  // query rows of an MMA tile; a default work item has two
 constexpr int TC_SURV_CAP = 1024;
 size_t tc_map_bytes();
 int tc_encode_rows_map(void* map_out, const void* x16, int64_t N, int d_pad, int prec);  // d_pad 0: extra block
@@ -169,8 +169,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
-                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
-                   int layout = 0);
+                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms);
 int launch_tc_rerank(const float* xs, int d_pad, const uint32_t* perm, const uint32_t* offsets, uint32_t NC,
                      const float* Y, int d, int64_t Q, const uint32_t* probes, int64_t P_eff, const uint32_t* surv_cnt,
                      const uint32_t* surv, int cap, int k, const int64_t* query_src, int64_t grid_w, int radius,

@@ -124,8 +124,8 @@ size_t bucket_of(const osann_server* s, int64_t n)
 }
 
 // The candidate (path, group, layout) choices of the tuner; the workspace of
-// a slot covers all of them.  The query-tile layout of the screen is a
-// choice only where both exist (d_pad = 128: 64 < d <= 128).
+// a slot covers all of them.  Group 0 is the screen's default, items of two
+// query tiles; smaller groups make more items, for small batches.
 std::vector<Choice> candidates(const osann_server* s, int i)
 {
     int32_t d = 0;
@@ -134,12 +134,8 @@ std::vector<Choice> candidates(const osann_server* s, int i)
     c.push_back({OSANN_PATH_PLAIN, 0, OSANN_LAYOUT_DEFAULT});
     c.push_back({OSANN_PATH_BATCHED, 0, OSANN_LAYOUT_DEFAULT});
     c.push_back({OSANN_PATH_BATCHED, 32, OSANN_LAYOUT_DEFAULT});
-    if (d > 64 && d <= 128) {
-        c.push_back({OSANN_PATH_FP16, 128, OSANN_LAYOUT_TMEM});
-        c.push_back({OSANN_PATH_FP16, 128, OSANN_LAYOUT_SMEM});
-    } else {
-        c.push_back({OSANN_PATH_FP16, 128, OSANN_LAYOUT_DEFAULT});
-    }
+    c.push_back({OSANN_PATH_FP16, 0, OSANN_LAYOUT_DEFAULT});
+    c.push_back({OSANN_PATH_FP16, 128, d > 64 && d <= 128 ? OSANN_LAYOUT_SMEM : OSANN_LAYOUT_DEFAULT});
     c.push_back({OSANN_PATH_FP16, 64, OSANN_LAYOUT_DEFAULT});
     return c;
 }

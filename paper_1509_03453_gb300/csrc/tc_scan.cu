@@ -422,8 +422,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
-                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
-                   int layout)
+                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms)
 {
     TcArgs a{};
     a.perm = perm;
@@ -434,8 +433,6 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
     a.query_src = query_src;
     a.items = b.items;
     a.n_items_dev = b.n_items_dev;
-    a.qcount = b.qcount;
-    a.qoff = b.qoff;
     a.qlist = b.qlist;
     a.counter = b.counters;
     a.Ubits = Ubits;
@@ -452,33 +449,15 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
     a.k = k;
     a.radius = radius;
     a.cap = cap;
-    a.stages = tc_stages(d_pad);
-    a.abufs = tc_abufs(d_pad);
-    if (a.stages > TC_STAGES_MAX || a.abufs > TC_NA_MAX) return -2;  // unsupported shape
-    a.debug = debug;
+    a.prec = prec;
+    a.ksteps = (d + 15) / 16;
     a.cdot2 = cdot2;
     a.Bn = Bn;
     a.cabs = cabs;
     const bool excl = query_src != nullptr;
-    if (d_pad == 128 && !excl && layout != OSANN_LAYOUT_SMEM) {
-        // one CTA per SM with the query tiles in TMEM and five cone-tile stages
-        a.stages = tc_stages_at(d_pad);
-        return launch_tc_scan_tmem(maps, a, k, prec, debug != 0, st, num_sms);
-    }
-    if (debug) return launch_tc_scan_debug(maps, a, k, prec, excl, st, num_sms);
-#define OSANN_TC(KM)                                                                                 \
-    do {                                                                                             \
-        if (prec == 0)                                                                               \
-            return excl ? launch_tc_t<KM, true, 0, false>(maps, a, st, num_sms)                      \
-                        : launch_tc_t<KM, false, 0, false>(maps, a, st, num_sms);                    \
-        return excl ? launch_tc_t<KM, true, 1, false>(maps, a, st, num_sms)                          \
-                    : launch_tc_t<KM, false, 1, false>(maps, a, st, num_sms);                        \
-    } while (0)
-    if (k <= 1) OSANN_TC(1);
-    if (k <= 4) OSANN_TC(4);
-    if (k <= 16) OSANN_TC(16);
-    OSANN_TC(32);
-#undef OSANN_TC
+    if (excl) return launch_tc_scan_excl(maps, a, k, debug != 0, st, num_sms);
+    if (debug) return launch_tc_scan_debug(maps, a, k, st, num_sms);
+    return launch_tc_dp<false, false>(maps, a, k, st, num_sms);
 }
 
 int launch_tc_rerank(const float* xs, int d_pad, const uint32_t* perm, const uint32_t* offsets, uint32_t NC,

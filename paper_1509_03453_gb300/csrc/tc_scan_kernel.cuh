@@ -64,32 +64,45 @@ __device__ __forceinline__ float from16(uint16_t h)
     if (PREC == 0) return __bfloat162float(__ushort_as_bfloat16(h));
     return __half2float(__ushort_as_half(h));
 }
+// the value 16-bit word of a number that the 16-bit type holds exactly, precision at run time
+__device__ __forceinline__ uint16_t to16_exact(int prec, float f)
+{
+    return prec == 0 ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : __half_as_ushort(__float2half_rn(f));
+}
 __device__ __forceinline__ uint32_t pack16(uint16_t lo, uint16_t hi) { return uint32_t(lo) | (uint32_t(hi) << 16); }
 
-__host__ __device__ inline int tc_row_bytes(int d_pad) { return d_pad >= 64 ? 128 : d_pad * 2; }
-__host__ __device__ inline int tc_kblocks(int d_pad) { return d_pad >= 64 ? d_pad / 64 : 1; }
-// tile stages and query buffers per CTA: two CTAs per SM (each with its own
-// MMA issuer) while the shared memory allows, else one.  Two query buffers
-// suffice (a third measured no faster at d = 32); the shared memory they
-// leave buys a third cone-tile stage at d = 64 (6% faster on 4096-query
-// batches), the stage ring being what the producer waits on.
-__host__ inline int tc_stages(int d_pad) { return d_pad <= 16 ? 6 : (d_pad == 32 ? 4 : 3); }
-__host__ inline int tc_abufs(int) { return 2; }
-// (both within TC_STAGES_MAX and TC_NA_MAX, the sizes of the kernel's barrier arrays)
+__host__ __device__ constexpr int tc_row_bytes(int d_pad) { return d_pad >= 64 ? 128 : d_pad * 2; }
+
+// Shared-memory plan of one CTA (one per SM): query-tile slots per query tile,
+// cone-tile stages of TC_N rows, survivors buffered per screening thread.
+// d_pad = 128 has room for one slot per query tile only (36 KB each): the two
+// query tiles then reload in turn, each behind the other's MMAs.
+constexpr int TC_SMEM_MAX = 232448 - 1024;  // 227 KB, less the alignment slack
+constexpr int TC_QT = 2;                    // query tiles per item
+__host__ __device__ constexpr int tc_tile_bytes(int dp) { return TC_M * dp * 2 + TC_M * 32; }
+__host__ __device__ constexpr int tc_slots(int dp) { return dp >= 128 ? 1 : 2; }
+constexpr int TC_SBUF = 4;                  // survivors buffered per screening thread
+constexpr int TC_IQ = 4;                    // items in the queue
+__host__ __device__ constexpr int tc_static_bytes(int dp)  // barriers, queue, constants, survivors: an upper bound
+{
+    return 1024 + TC_QT * tc_slots(dp) * (TC_M * 20 + 16) + TC_QT * TC_M * (TC_SBUF * 8 + TC_IQ * 4);
+}
+__host__ __device__ constexpr int tc_stages(int dp)
+{
+    const int s = (TC_SMEM_MAX - tc_static_bytes(dp) - TC_QT * tc_slots(dp) * tc_tile_bytes(dp)) / tc_tile_bytes(dp);
+    return s > 8 ? 8 : s;
+}
 
 struct TcArgs {
-    const uint32_t* offsets;
     const uint32_t* perm;
     const float4* rowstat;    // per row: ((1-B)|x|^2, |x|, |x|^2, 0); N + TC_N rows
     const uint16_t* Y16;      // Q x d_pad, 16-bit -2 s y
     const float4* qstat;      // per query, scaled: (|q|^2, |q|, -A' (16-bit value, A' >= 2c|q| + Cabs), Cabs |q|)
     const float* tcs;         // (s, s^2, 1/s^2, X): X bounds every row norm (unscaled)
     const int64_t* query_src;
-    const uint4* items;  // (first row, end row, first slot, slot count)
+    const uint4* items;       // (first row, end row, first slot, slot count)
     const uint32_t* n_items_dev;
-    const uint32_t* qcount;
-    const uint32_t* qoff;
-    const uint32_t* qlist;
+    const uint32_t* qlist;    // list entries: query * S (+ position)
     uint32_t* counter;
     uint32_t* Ubits;     // per query: upper bound on the k-th best distance (float bits)
     uint32_t* surv_cnt;  // per query
@@ -100,48 +113,77 @@ struct TcArgs {
     const float* Y;
     int64_t S;
     int64_t grid_w;
-    int d, d_pad, k, radius, cap, stages, abufs, debug;
+    int d, d_pad, k, radius, cap;
+    int prec;     // 0 bf16, 1 fp16
+    int ksteps;   // K steps of 16 columns that hold components: ceil(d / 16); the rest of d_pad is zero
     float cdot2;  // 2c
     float Bn;     // B
     float cabs;   // coefficient of the subnormal rounding terms
 };
 
-// Item descriptor passed from the producer warp to the MMA and epilogue warps.
+// Item descriptor passed from the producer to the loaders.
 struct TcItem {
     uint32_t r0, r1;    // cone rows; r0 == 0xFFFFFFFF marks the end of the work
     uint32_t qbeg, qn;  // slot-list range of the query group
 };
+// What the issuer and the screening warps need of an item, passed with its query tile.
+struct TcWork {
+    uint32_t r0, nrows;  // nrows == 0 marks the end of the work
+    uint32_t t0;         // number of the item's first cone tile (stage t0 mod S)
+};
+// An item's queries [off, off + 128) belong to query tile qt: both tiles of an
+// item of more than 128 queries, else the tiles take the items in turn.
+__device__ __forceinline__ bool tc_used(uint32_t qt, uint32_t it, uint32_t qn)
+{
+    return qn > uint32_t(TC_M) || (it & 1u) == qt;
+}
 
-// Warp roles (256 threads): warp 0 lane 0 fetches items and streams the cone
-// tiles with TMA; warp 1 lane 0 issues the MMAs (warp 1 owns the TMEM
-// allocation); warps 2-3 ("loaders", 64 threads) gather the query tile of each
-// item (asynchronous 16-byte copies of the queries' 16-bit rows straight into
-// the swizzled tile) and write the per-query constants into one of the
-// shared query buffers, ahead of the MMAs; warps 4-7 (128 threads, one per query row and TMEM lane)
-// screen the accumulators.  Hand-offs are mbarriers: item queue (4 slots, the
-// producer one item ahead of its tiles), tile stages (full/empty), query
-// buffers (full/empty), accumulators (2 TMEM buffers of 128 columns,
-// full/empty), so the MMA of one tile overlaps the screening of the previous
-// one and the query loads overlap both.  Every wait is bounded; a timeout
-// sets ST_TIMEOUT and makes all roles drop out.
+// Warp roles (512 threads, one CTA per SM).  An item is a cone and up to 256
+// queries, two query tiles of 128, so that every cone tile brought into shared
+// memory is multiplied twice.  (One tile per item would need 74 to 82 bytes per
+// cycle and SM from L2 at full tensor rate: TMA moved at most 72 in a streaming
+// test, and that with 110 KB in flight.)
+//   warp 0      fetches items and streams the cone tiles with TMA;
+//   warps 1, 2  issue the MMAs of query tile 0 and 1, two accumulators of TC_N
+//               columns each (all 512 TMEM columns);
+//   warp 3      looks up the items' query indices (list entries) for the loaders;
+//   warps 4-7   loaders, two per query tile: gather the queries' 16-bit rows by
+//               16-byte asynchronous copies straight into the swizzled tile, and
+//               the per-query constants;
+//   warps 8-15  screening, four per query tile, a thread per query row = TMEM lane.
+// Hand-offs are mbarriers: item queue (producer to loaders), cone tiles (full /
+// empty, once per query tile), query tiles with their constants (full / empty),
+// accumulators (full / empty).  Every wait is bounded; a timeout sets ST_TIMEOUT
+// and makes all roles drop out.
 //
-// AT (query tiles in tensor memory; one CTA per SM, 384 threads): the query
-// tile of an item is written into TMEM next to the two accumulators (lane m =
-// query row m, 16-bit elements packed two per column) by warps 8-11, one
-// thread per query row, and every MMA takes A from there.  The MMAs then read
-// only the cone tiles from shared memory, and the shared memory of the query
-// tiles holds more cone-tile stages.  Warps 2-3 idle.
-constexpr int TC_ROLE_THREADS = 256;
-constexpr int TC_AT_THREADS = 384;
-constexpr int TC_IQ = 4;
-constexpr int TC_SBUF = 8;  // survivors buffered per thread before a flush
-constexpr int TC_NA_MAX = 2;
+// What bounds the kernel is the chain of hand-offs around each 128 x 128 tile
+// (192 to 576 tensor-core cycles), so that chain is kept short:
+//   - producer and issuers run as whole warps, with template widths, and elect one
+//     lane for the TMA and MMA instructions only: with run-time widths and a
+//     single-lane branch an MMA took 297 cycles to issue per CTA (64 of the
+//     tensor core);
+//   - one commit per tile.  A second one idles the tensor core for 70 to 80
+//     cycles (streaming test, 5 MMAs per tile: 799 against 640 cycles per pair of
+//     tiles), so the screening warps, woken by the commit, pass on that the cone
+//     tile (and after the last one the query tile) is free;
+//   - issuers and screening warps wait on no item queue: the loaders pass the item
+//     on with its query tile;
+//   - an accumulator is released when its values are in registers, before they
+//     are looked at;
+//   - the loaders find the items' query indices in shared memory, put there by
+//     warp 3, so that one global latency and not two lies between a free query
+//     slot and its new tile;
+//   - survivors wait in shared memory across items and are appended a few at a
+//     time: the atomic's round trip held a screening warp for some 1500 cycles
+//     whenever an item left one (9% of a 4096-query batch at d = 64).
+// Measured on 4096-query batches (us): d = 64 1050 -> 706, d = 128 1205 -> 988;
+// d = 32, 10^4 queries 219 -> 166; before: one query tile per CTA, two CTAs per SM
+// (d = 128: one, query tiles in tensor memory).
+constexpr int TC_THREADS = 512;
 constexpr int TC_STAGES_MAX = 8;
-// TMEM accumulators of TC_N columns per CTA (two CTAs share an SM's 512
-// columns; a CTA alone on its SM with four was measured slower)
-constexpr uint32_t TC_NACC = 2;
+constexpr uint32_t TC_NACC = 2;  // accumulators of TC_N columns per query tile
 
-// per-query constants of a query tile, written by the loaders
+// per-query constants of a query row, derived from (|q|^2, A', Cq, U)
 struct TcQConst {
     float qn2;   // |q|^2 (scaled)
     float Uthr;  // s^2 U - (1-B)|q|^2 + Cq (scaled)
@@ -153,46 +195,48 @@ struct TcQConst {
 
 // DEBUG: check every screened value against an fp32 evaluation of the
 // folded product (a separate instantiation, so the check costs nothing when off)
-template <int KMAX, bool EXCL, int PREC, bool DEBUG, bool AT>
-__global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 : 2)
+template <int KMAX, bool EXCL, bool DEBUG, int DP>
+__global__ void __launch_bounds__(TC_THREADS, 1)
     tc_scan_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_x,
                    const TcArgs a)
 {
-    extern __shared__ unsigned char smem_raw[];
-    unsigned char* base =
-        reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t iq_full[TC_IQ], iq_empty[TC_IQ];
-    __shared__ __align__(8) uint64_t bfull[TC_STAGES_MAX], bempty[TC_STAGES_MAX];
-    __shared__ __align__(8) uint64_t afull[TC_NA_MAX], aempty[TC_NA_MAX], accfull[TC_NACC], accempty[TC_NACC];
-    __shared__ TcItem iq[TC_IQ];
-    __shared__ TcQConst qc[TC_NA_MAX][TC_M];
-    __shared__ uint32_t qidx[TC_NA_MAX][TC_M];  // query index, 0xFFFFFFFF for an unused row
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ volatile int abort_sh;
-    __shared__ uint32_t sbuf_row[TC_SBUF * 128];  // survivors buffered per screening thread
-    __shared__ float sbuf_val[TC_SBUF * 128];
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int row_bytes = tc_row_bytes(a.d_pad);
-    const int kblocks = tc_kblocks(a.d_pad);
-    const int epb = row_bytes / 2;
-    const int ksteps_pb = epb / 16;
-    const int mainA = TC_M * a.d_pad * 2, mainB = TC_N * a.d_pad * 2;
-    const int extA = TC_M * 32, extB = TC_N * 32;  // extra K block: 16 bf16 per row
-    const int S = a.stages;
-    const uint32_t NA = uint32_t(a.abufs);
-    constexpr uint32_t NACC = TC_NACC;
-    unsigned char* sA = base;                                       // NA x (mainA + extA); none with AT
-    unsigned char* sB = AT ? base : base + NA * size_t(mainA + extA);  // S x (mainB + extB)
-    // AT: TMEM columns of a query tile (d_pad / 2 packed pairs, then the 8 of the extra block)
-    const uint32_t acols = uint32_t(a.d_pad / 2 + 8);
-    constexpr uint32_t TMEM_COLS = AT ? 512u : NACC * TC_N;
-    const uint32_t idesc = idesc_f16_f32(TC_M, TC_N, PREC == 0 ? 1u : 0u);
-    const uint32_t tx_bytes = uint32_t(mainB + extB);
-    const float sc = a.tcs[0], sc2 = a.tcs[1], inv_sc2 = a.tcs[2], xmax = a.tcs[3];
     // k = 1 without exclusion: the minimum of a full chunk bounds the best
     // candidate directly, and survivors need only their row
     constexpr bool FAST = KMAX == 1 && !EXCL;
+    constexpr int row_bytes = tc_row_bytes(DP);
+    constexpr int kblocks = DP >= 64 ? DP / 64 : 1;
+    constexpr int epb = row_bytes / 2;
+    constexpr int ksteps_pb = epb / 16;
+    constexpr int mainT = TC_M * DP * 2;         // main part of a query or cone tile (TC_M = TC_N rows)
+    constexpr int tileT = tc_tile_bytes(DP);     // with the extra K block: 16 elements per row
+    constexpr int S = tc_stages(DP);
+    constexpr uint32_t NA = uint32_t(tc_slots(DP)), NACC = TC_NACC;
+    constexpr uint32_t TMEM_COLS = TC_QT * NACC * TC_N;
+    static_assert(S >= 2 && S <= TC_STAGES_MAX, "cone-tile stages");
+
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* base =
+        reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    unsigned char* sA = base;                         // [TC_QT][NA] query tiles
+    unsigned char* sB = base + TC_QT * NA * tileT;    // S cone tiles
+    __shared__ __align__(8) uint64_t iq_full[TC_IQ], ix_full[TC_IQ], iq_empty[TC_IQ];
+    __shared__ __align__(8) uint64_t bfull[TC_STAGES_MAX], bempty[TC_STAGES_MAX];
+    __shared__ __align__(8) uint64_t afull_all[TC_QT][NA], aempty_all[TC_QT][NA];
+    __shared__ __align__(8) uint64_t accfull_all[TC_QT][TC_NACC], accempty_all[TC_QT][TC_NACC];
+    __shared__ TcItem iq[TC_IQ];
+    __shared__ uint32_t iq_q[TC_IQ][TC_QT * TC_M];  // the items' query indices, 0xFFFFFFFF past the last
+    __shared__ TcWork work_all[TC_QT][NA];
+    __shared__ float4 qc_all[TC_QT][NA][TC_M];      // per query row (|q|^2, A', Cq, U)
+    __shared__ uint32_t qidx_all[TC_QT][NA][TC_M];  // query index, 0xFFFFFFFF for an unused row
+    __shared__ uint32_t tmem_base_sh;
+    __shared__ volatile int abort_sh;
+    constexpr int SW = TC_QT * TC_M;
+    // survivors buffered per screening thread: (row, query), with EXCL (row, value)
+    __shared__ uint2 sbuf[TC_SBUF * SW];
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t tx_bytes = uint32_t(tileT);
+    const float sc = a.tcs[0], sc2 = a.tcs[1], inv_sc2 = a.tcs[2], xmax = a.tcs[3];
 
     if (warp == 1) {
         tmem_alloc(&tmem_base_sh, TMEM_COLS);
@@ -201,20 +245,22 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
     if (tid == 0) {
         for (int i = 0; i < TC_IQ; ++i) {
             mbar_init(&iq_full[i], 1);
-            // MMA issuer, 64 loader threads (4 loader warps with AT), 4 screening warps
-            mbar_init(&iq_empty[i], AT ? 1 + 4 + 4 : 1 + 64 + 4);
+            mbar_init(&ix_full[i], 1);
+            mbar_init(&iq_empty[i], 4);  // loader warps
         }
         for (int s = 0; s < S; ++s) {
             mbar_init(&bfull[s], 1);
-            mbar_init(&bempty[s], 1);
+            mbar_init(&bempty[s], TC_QT);  // once per query tile
         }
-        for (uint32_t b = 0; b < NA; ++b) {
-            mbar_init(&afull[b], AT ? 4 : 64);
-            mbar_init(&aempty[b], 4);  // one arrival per screening warp
-        }
-        for (uint32_t b = 0; b < NACC; ++b) {
-            mbar_init(&accfull[b], 1);
-            mbar_init(&accempty[b], 4);
+        for (int q = 0; q < TC_QT; ++q) {
+            for (uint32_t b = 0; b < NA; ++b) {
+                mbar_init(&afull_all[q][b], 64);  // the tile's loader threads
+                mbar_init(&aempty_all[q][b], 4);  // one arrival per screening warp
+            }
+            for (uint32_t b = 0; b < NACC; ++b) {
+                mbar_init(&accfull_all[q][b], 1);
+                mbar_init(&accempty_all[q][b], 4);
+            }
         }
         fence_mbar_init();
         abort_sh = 0;
@@ -224,310 +270,366 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
     tc_fence_after();
     const uint32_t tmem = tmem_base_sh;
 
-    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (abort_sh) return false;
-        if (mbar_wait_bounded(bar, parity)) return true;
-        if (!abort_sh) atomicOr(a.status, ST_TIMEOUT);
-        abort_sh = 1;
-        return false;
+    // called by whole warps; the result is the same in every lane, so that the
+    // warp stays converged for its collective instructions after a give-up
+    auto give_up = [&](uint64_t* bar, uint32_t parity) -> bool {
+        bool ok = false;
+        if (!abort_sh) {
+            ok = mbar_wait_bounded(bar, parity);
+            if (!ok) {
+                if (!abort_sh) atomicOr(a.status, ST_TIMEOUT);
+                abort_sh = 1;
+            }
+        }
+        return ok;
     };
-    // per-query constants of a query row from its statistics and bound
-    auto make_qc = [&](const float4& qsv, float Uv) -> TcQConst {
-        TcQConst c;
-        c.qn2 = qsv.x;
-        c.U = Uv;
-        c.Cq = qsv.w;
-        c.Uthr = sc2 * Uv - (1.0f - a.Bn) * qsv.x + qsv.w;
-        c.Aq1 = -qsv.z;
-        c.Uoff = (1.0f + a.Bn) * qsv.x + 2.0f * a.Bn * sc2 * xmax * xmax + 2.0f * c.Aq1 * sc * xmax + qsv.w;
-        return c;
+    auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+        bool ok = mbar_try_wait(bar, parity);
+        if (!ok) ok = give_up(bar, parity);
+        return __all_sync(0xffffffffu, ok);
     };
 
+    // query tile of this warp's role, and its hand-offs
+    const uint32_t qt = warp == 2 || warp == 6 || warp == 7 || warp >= 12 ? 1u : 0u;
+    uint64_t* const afull = afull_all[qt];
+    uint64_t* const aempty = aempty_all[qt];
+    uint64_t* const accfull = accfull_all[qt];
+    uint64_t* const accempty = accempty_all[qt];
+    TcWork* const work = work_all[qt];
+
     if (warp == 0) {
-        // ------------------------------------------------ producer
-        if (lane == 0) {
-            const uint32_t n_items = *a.n_items_dev;
-            uint32_t it = 0, tc = 0, s = 0, s_ph = 0;
-            // the next item's index and descriptor are fetched one publish
-            // ahead, so their latency overlaps the current item's tiles
-            uint32_t pf_item = atomicAdd(a.counter, 1u);
-            uint4 pf = pf_item < n_items ? a.items[pf_item] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
-            auto publish = [&](TcItem& out) -> bool {
-                const int slot = int(it % TC_IQ);
-                if (it >= TC_IQ && !wait(&iq_empty[slot], ((it / TC_IQ) - 1) & 1u)) return false;
-                TcItem d;
-                d.r0 = pf.x;
-                d.r1 = pf.y;
-                d.qbeg = pf.z;
-                d.qn = pf.w;
-                if (d.r0 != 0xFFFFFFFFu) {
-                    pf_item = atomicAdd(a.counter, 1u);
-                    pf = pf_item < n_items ? a.items[pf_item] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
-                }
-                iq[slot] = d;
+        // ------------------------------------------------ producer (whole warp)
+        const uint32_t n_items = *a.n_items_dev;
+        uint32_t it = 0, tc = 0, s = 0, s_ph = 0;
+        // lane 0 fetches the next item's index and descriptor one publish ahead,
+        // so their latency overlaps the current item's tiles
+        uint4 pf = make_uint4(0xFFFFFFFFu, 0, 0, 0);
+        auto fetch = [&]() {
+            const uint32_t i = atomicAdd(a.counter, 1u);
+            pf = i < n_items ? a.items[i] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
+        };
+        if (lane == 0) fetch();
+        auto publish = [&](uint32_t& r0, uint32_t& r1) -> bool {
+            const uint32_t slot = it % TC_IQ;
+            if (it >= TC_IQ && !wait(&iq_empty[slot], ((it / TC_IQ) - 1) & 1u)) return false;
+            r0 = __shfl_sync(0xffffffffu, pf.x, 0);
+            r1 = __shfl_sync(0xffffffffu, pf.y, 0);
+            if (lane == 0) {
+                iq[slot] = TcItem{pf.x, pf.y, pf.z, pf.w};
                 mbar_arrive(&iq_full[slot]);
-                ++it;
-                out = d;
-                return d.r0 != 0xFFFFFFFFu;
-            };
-            TcItem cur, nxt;
-            bool have = publish(cur);
-            while (have && !abort_sh) {
-                const bool have_next = publish(nxt);  // one item ahead of its tiles
-                const int ntiles = int((cur.r1 - cur.r0 + TC_N - 1) / TC_N);
-                for (int t = 0; t < ntiles; ++t, ++tc) {
-                    // stage s = tc mod S, s_ph = (tc / S) & 1: wait for the stage's previous use
-                    if (tc >= uint32_t(S) && !wait(&bempty[s], s_ph ^ 1u)) break;
-                    const int y0 = int(cur.r0) + t * TC_N;
-                    unsigned char* dst = sB + size_t(s) * (mainB + extB);
+                if (r0 != 0xFFFFFFFFu) fetch();
+            }
+            ++it;
+            return r0 != 0xFFFFFFFFu;
+        };
+        uint32_t cr0, cr1, nr0, nr1;
+        bool have = publish(cr0, cr1), ok = true;
+        while (have) {
+            const bool have_next = publish(nr0, nr1);  // one item ahead of its tiles
+            const int ntiles = int((cr1 - cr0 + TC_N - 1) / TC_N);
+            for (int t = 0; t < ntiles; ++t, ++tc) {
+                // stage s = tc mod S, s_ph = (tc / S) & 1: wait for the stage's previous use
+                if (tc >= uint32_t(S) && !wait(&bempty[s], s_ph ^ 1u)) { ok = false; break; }
+                const int y0 = int(cr0) + t * TC_N;
+                unsigned char* dst = sB + s * uint32_t(tileT);
+                if (elect_one()) {
                     mbar_arrive_expect_tx(&bfull[s], tx_bytes);
+#pragma unroll
                     for (int kb = 0; kb < kblocks; ++kb)
-                        tma_load_2d(dst + size_t(kb) * TC_N * row_bytes, &tmap, kb * epb, y0, &bfull[s]);
-                    tma_load_2d(dst + mainB, &tmap_x, 0, y0, &bfull[s]);
-                    if (++s == uint32_t(S)) {
-                        s = 0;
-                        s_ph ^= 1u;
-                    }
+                        tma_load_2d(dst + kb * TC_N * row_bytes, &tmap, kb * epb, y0, &bfull[s]);
+                    tma_load_2d(dst + mainT, &tmap_x, 0, y0, &bfull[s]);
                 }
-                if (abort_sh) break;
-                cur = nxt;
-                have = have_next;
+                if (++s == uint32_t(S)) {
+                    s = 0;
+                    s_ph ^= 1u;
+                }
             }
-            if (abort_sh) {
-                // let the last tile issued into each stage land before shared memory goes away
-                for (uint32_t g = tc > uint32_t(S) ? tc - uint32_t(S) : 0u; g < tc; ++g)
-                    mbar_wait_bounded(&bfull[g % uint32_t(S)], (g / uint32_t(S)) & 1u);
-            }
+            if (!ok) break;
+            cr0 = nr0;
+            cr1 = nr1;
+            have = have_next;
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            const int ksteps = kblocks * ksteps_pb;  // <= 8
-            // descriptors of query buffer 0 and tile stage 0; a buffer, a stage
-            // and a K step add their byte offset / 16 to the 14-bit start-address
-            // field, which never carries (shared memory is below 2^18 bytes)
-            const uint64_t da0 = smem_desc_kmajor(smem_u32(sA), row_bytes);
-            const uint64_t db0 = smem_desc_kmajor(smem_u32(sB), row_bytes);
-            const uint64_t dax0 = smem_desc_kmajor(smem_u32(sA + mainA), 32);
-            const uint64_t dbx0 = smem_desc_kmajor(smem_u32(sB + mainB), 32);
-            const uint32_t a_step = uint32_t(mainA + extA) >> 4, b_step = uint32_t(mainB + extB) >> 4;
-            uint32_t koff[8];
+        if (__any_sync(0xffffffffu, abort_sh != 0)) {
+            // let the last tile issued into each stage land before shared memory goes away
+            for (uint32_t g = tc > uint32_t(S) ? tc - uint32_t(S) : 0u; g < tc; ++g)
+                mbar_wait_bounded(&bfull[g % uint32_t(S)], (g / uint32_t(S)) & 1u);
+        }
+    } else if (warp <= TC_QT) {
+        // ------------------------------------------------ MMA issuer of query tile qt (whole warp)
+        constexpr int KS = kblocks * ksteps_pb;  // <= 8
+        const int ksteps = a.ksteps;             // those that hold components
+        // instruction descriptor: a full tile, or its first 64 rows
+        const uint32_t idesc = idesc_f16_f32(TC_M, TC_N, a.prec == 0 ? 1u : 0u);
+        const uint32_t idesc_h = idesc_f16_f32(TC_M, TC_N / 2, a.prec == 0 ? 1u : 0u);
+        // descriptors of this tile's slot 0 and of stage 0; a slot, a stage and a K step
+        // add their byte offset / 16 to the 14-bit start-address field, which
+        // never carries (shared memory is below 2^18 bytes)
+        unsigned char* sA0 = sA + qt * NA * uint32_t(tileT);
+        const uint64_t da0 = smem_desc_kmajor(smem_u32(sA0), row_bytes);
+        const uint64_t db0 = smem_desc_kmajor(smem_u32(sB), row_bytes);
+        const uint64_t dax0 = smem_desc_kmajor(smem_u32(sA0 + mainT), 32);
+        const uint64_t dbx0 = smem_desc_kmajor(smem_u32(sB + mainT), 32);
+        constexpr uint32_t step = uint32_t(tileT) >> 4;
+        // Every issuer sees every cone tile, in order: one of an item that is not its
+        // query tile's it only waits for and releases, so that no stage's phase
+        // runs ahead of it.
+        uint32_t tc = 0, ab = 0, ab_ph = 0, seen = 0, s = 0, s_ph = 0;
+        for (;;) {
+            if (!wait(&afull[ab], ab_ph)) break;
+            const uint32_t nrows = __shfl_sync(0xffffffffu, work[ab].nrows, 0);
+            const uint32_t t0 = __shfl_sync(0xffffffffu, work[ab].t0, 0);
+            bool ok = true;
+            for (; ok && seen < t0; ++seen) {
+                ok = wait(&bfull[s], s_ph);
+                if (ok && lane == 0) mbar_arrive(&bempty[s]);
+                if (++s == uint32_t(S)) {
+                    s = 0;
+                    s_ph ^= 1u;
+                }
+            }
+            if (!ok || nrows == 0) break;
+            const int ntiles = int((nrows + TC_N - 1) / TC_N);
+            seen += uint32_t(ntiles);
+            const uint64_t da = da0 + ab * step, dax = dax0 + ab * step;
+            for (int t = 0; t < ntiles; ++t, ++tc) {
+                const uint32_t acc = tc % NACC, acc_ph = ((tc / NACC) - 1) & 1u;
+                // the two waits together: their latencies overlap
+                bool rb = mbar_try_wait(&bfull[s], s_ph);
+                bool ra = tc < NACC || mbar_try_wait(&accempty[acc], acc_ph);
+                if (!rb) rb = give_up(&bfull[s], s_ph);
+                if (!ra) ra = give_up(&accempty[acc], acc_ph);
+                if (!__all_sync(0xffffffffu, ra && rb)) { ok = false; break; }
+                tc_fence_after();
+                const uint64_t db = db0 + s * step, dbx = dbx0 + s * step;
+                const uint32_t dt = tmem + (qt * NACC + acc) * TC_N;
+                // the screening reads whole 64-column chunks: a last tile of at
+                // most 64 rows needs only the first
+                const uint32_t id = nrows - uint32_t(t) * TC_N <= TC_N / 2 ? idesc_h : idesc;
+                if (elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk)
-                koff[kk] = uint32_t((kk / ksteps_pb) * TC_M * row_bytes + (kk % ksteps_pb) * 32) >> 4;
-            uint32_t it = 0, tc = 0, s = 0, s_ph = 0, ab = 0, ab_ph = 0;
-            for (;;) {
-                const int slot = int(it % TC_IQ);
-                if (!wait(&iq_full[slot], (it / TC_IQ) & 1u)) break;
-                const TcItem d = iq[slot];
-                if (d.r0 == 0xFFFFFFFFu) break;
-                if (!wait(&afull[ab], ab_ph)) break;
-                const int ntiles = int((d.r1 - d.r0 + TC_N - 1) / TC_N);
-                const uint64_t da = da0 + ab * a_step, dax = dax0 + ab * a_step;
-                const uint32_t ta = tmem + NACC * TC_N + ab * acols;  // AT: the query tile's columns
-                bool ok = true;
-                for (int t = 0; t < ntiles; ++t, ++tc) {
-                    const uint32_t acc = tc % NACC;
-                    if (!wait(&bfull[s], s_ph)) { ok = false; break; }
-                    if (tc >= NACC && !wait(&accempty[acc], ((tc / NACC) - 1) & 1u)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint64_t db = db0 + s * b_step, dbx = dbx0 + s * b_step;
-                    const uint32_t dt = tmem + acc * TC_N;
-                    if (AT) {
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)
-                            if (kk < ksteps) mma_f16_ts(dt, ta + uint32_t(kk) * 8u, db + koff[kk], idesc, kk > 0 ? 1u : 0u);
-                        mma_f16_ts(dt, ta + uint32_t(a.d_pad / 2), dbx, idesc, 1u);
-                    } else {
-#pragma unroll
-                        for (int kk = 0; kk < 8; ++kk)
-                            if (kk < ksteps) mma_bf16_ss(dt, da + koff[kk], db + koff[kk], idesc, kk > 0 ? 1u : 0u);
-                        // extra K block: |x|^2 and |x| terms folded into the product
-                        mma_bf16_ss(dt, dax, dbx, idesc, 1u);
+                    for (int kk = 0; kk < KS; ++kk) {
+                        const uint32_t ko = uint32_t((kk / ksteps_pb) * TC_M * row_bytes + (kk % ksteps_pb) * 32) >> 4;
+                        if (kk < ksteps) mma_bf16_ss(dt, da + ko, db + ko, id, kk > 0 ? 1u : 0u);
                     }
-                    mma_commit(&bempty[s]);
+                    // extra K block: |x|^2 and |x| terms folded into the product
+                    mma_bf16_ss(dt, dax, dbx, id, 1u);
                     mma_commit(&accfull[acc]);
-                    if (++s == uint32_t(S)) {
-                        s = 0;
-                        s_ph ^= 1u;
-                    }
                 }
-                if (!ok) break;
-                mbar_arrive(&iq_empty[slot]);
-                ++it;
-                if (++ab == NA) {
-                    ab = 0;
-                    ab_ph ^= 1u;
+                if (++s == uint32_t(S)) {
+                    s = 0;
+                    s_ph ^= 1u;
                 }
             }
-            if (abort_sh && tc > 0) mbar_wait_bounded(&accfull[(tc - 1) % NACC], ((tc - 1) / NACC) & 1u);
+            if (!ok) break;
+            if (++ab == NA) {
+                ab = 0;
+                ab_ph ^= 1u;
+            }
         }
-    } else if (!AT && warp < 4) {
-        // ------------------------------------------------ query tile loaders
-        // warp 2 gathers query rows 0..63 of the tile, warp 3 rows 64..127;
-        // lane l holds the indices and constants of rows rb + l and rb + 32 + l
-        const int rb = 64 * (warp - 2);
-        const int cpr = a.d_pad / 8;  // 16-byte chunks per 16-bit query row (2, 4, 8 or 16)
-        const int cpr_sh = __ffs(cpr) - 1;
-        const int chunks_sh = __ffs(row_bytes / 16) - 1;  // chunks per row of one K block of the tile
+        if (abort_sh && tc > 0) mbar_wait_bounded(&accfull[(tc - 1) % NACC], ((tc - 1) / NACC) & 1u);
+    } else if (warp == 3) {
+        // ------------------------------------------------ query indices of the items
+        const uint32_t dv = uint32_t(a.S);
         for (uint32_t it = 0;; ++it) {
-            const int slot = int(it % TC_IQ);
+            const uint32_t slot = it % TC_IQ;
             if (!wait(&iq_full[slot], (it / TC_IQ) & 1u)) break;
             const TcItem d = iq[slot];
-            if (d.r0 == 0xFFFFFFFFu) break;
-            const uint32_t ab = it % NA;
-            if (it >= NA && !wait(&aempty[ab], ((it / NA) - 1) & 1u)) break;
-            unsigned char* dstA = sA + size_t(ab) * (mainA + extA);
-            // both rows' query indices; then the warp's 64 16-bit rows as
-            // asynchronous 16-byte copies straight into the swizzled tile, every
-            // chunk in flight at once, consecutive lanes on consecutive chunks of
-            // one row (each instruction reads whole 32-byte sectors); while those
-            // land, both rows' constants
-            uint32_t qr[2];
+            const bool end = d.r0 == 0xFFFFFFFFu;
+            constexpr int E = TC_QT * TC_M / 32;
+            uint32_t e[E];
+#pragma unroll
+            for (int i = 0; i < E; ++i) e[i] = !end && uint32_t(lane + 32 * i) < d.qn ? a.qlist[d.qbeg + lane + 32 * i] : 0u;
+#pragma unroll
+            for (int i = 0; i < E; ++i)
+                iq_q[slot][lane + 32 * i] =
+                    !end && uint32_t(lane + 32 * i) < d.qn ? (dv == 1u ? e[i] : e[i] / dv) : 0xFFFFFFFFu;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&ix_full[slot]);
+            if (end) break;
+        }
+    } else if (warp >= 4 && warp < 8) {
+        // ------------------------------------------------ query tile loaders
+        // per query tile, one warp gathers rows 0..63 and one rows 64..127; lane l
+        // holds the indices and constants of rows rb + l and rb + 32 + l
+        const int rb = 64 * (warp & 1);
+        constexpr int cpr = DP / 8;          // 16-byte chunks per 16-bit query row (2, 4, 8 or 16)
+        constexpr int cpb = row_bytes / 16;  // chunks per row of one K block of the tile
+        uint32_t t0 = 0, nl = 0;
+        for (uint32_t it = 0;; ++it) {
+            const uint32_t slot = it % TC_IQ;
+            if (!wait(&ix_full[slot], (it / TC_IQ) & 1u)) break;
+            const TcItem d = iq[slot];
+            // nrows = 0: the end mark
+            const uint32_t nrows = d.r0 == 0xFFFFFFFFu ? 0u : d.r1 - d.r0;
+            const bool mine = nrows == 0 || tc_used(qt, it, d.qn);
+            const uint32_t off = (d.qn > uint32_t(TC_M) ? qt * TC_M : 0u) + rb + lane;
+            const uint32_t qr[2] = {iq_q[slot][off], iq_q[slot][off + 32]};
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&iq_empty[slot]);
+            const uint32_t first = t0;
+            t0 += (nrows + TC_N - 1) / TC_N;
+            if (!mine) continue;
+            const uint32_t ab = nl % NA;
+            if (nl >= NA && !wait(&aempty[ab], ((nl / NA) - 1) & 1u)) break;
+            ++nl;
             float4 qs[2];
             float Ur[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int r = rb + lane + 32 * h;
-                qr[h] = uint32_t(r) < d.qn ? a.qlist[d.qbeg + r] / uint32_t(a.S) : 0xFFFFFFFFu;
-            }
-            for (int j = 0; j < 2 * cpr; ++j) {
-                const int i = lane + 32 * j;  // chunk of the warp's rows
-                const int rl = i >> cpr_sh, ch = i & (cpr - 1);
-                // rl < 32 for all lanes or for none: the source register is uniform
-                const uint32_t qs_src = __shfl_sync(0xffffffffu, j < cpr ? qr[0] : qr[1], rl & 31);
-                unsigned char* dst = dstA + size_t(ch >> chunks_sh) * TC_M * row_bytes +
-                                     swz_offset(rb + rl, ch & ((1 << chunks_sh) - 1), row_bytes);
-                if (qs_src != 0xFFFFFFFFu)
-                    cp_async16(dst, reinterpret_cast<const uint4*>(a.Y16 + int64_t(qs_src) * a.d_pad) + ch);
-                else
-                    *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
-            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 qs[h] = make_float4(0.f, 0.f, 0.f, 0.f);
                 Ur[h] = INFINITY;
                 if (qr[h] != 0xFFFFFFFFu) {
                     qs[h] = a.qstat[qr[h]];
-                    Ur[h] = __uint_as_float(a.Ubits[qr[h]]);
+                    Ur[h] = __uint_as_float(__ldcg(a.Ubits + qr[h]));
+                }
+            }
+            unsigned char* dstA = sA + (qt * NA + ab) * uint32_t(tileT);
+            if (lane == 0 && rb == 0) work[ab] = TcWork{d.r0, nrows, first};
+            if (nrows != 0) {
+                // the warp's 64 16-bit rows as asynchronous 16-byte copies, every chunk
+                // in flight at once, consecutive lanes on consecutive chunks of one row
+                // (each instruction reads whole 32-byte sectors)
+#pragma unroll
+                for (int j = 0; j < 2 * cpr; ++j) {
+                    const int i = lane + 32 * j;  // chunk of the warp's rows
+                    const int rl = i / cpr, ch = i % cpr;
+                    // rl < 32 for all lanes or for none: the source register is uniform
+                    const uint32_t qs_src = __shfl_sync(0xffffffffu, j < cpr ? qr[0] : qr[1], rl & 31);
+                    unsigned char* dst = dstA + (ch / cpb) * TC_M * row_bytes + swz_offset(rb + rl, ch % cpb, row_bytes);
+                    if (qs_src != 0xFFFFFFFFu)
+                        cp_async16(dst, reinterpret_cast<const uint4*>(a.Y16 + int64_t(qs_src) * DP) + ch);
+                    else
+                        *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
                 }
             }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int r = rb + lane + 32 * h;
-                const bool active = qr[h] != 0xFFFFFFFFu;
                 // extra block: (1, 1, -A', -A', 0, ...) against (|x|^2 hi, lo, |x| hi, lo, 0, ...)
                 uint4 e0 = make_uint4(0, 0, 0, 0);
-                if (active) {
-                    const uint16_t one = to16_rn<PREC>(1.0f), na = to16_rn<PREC>(qs[h].z);  // exact
+                if (qr[h] != 0xFFFFFFFFu) {
+                    const uint16_t one = to16_exact(a.prec, 1.0f), na = to16_exact(a.prec, qs[h].z);
                     e0.x = pack16(one, one);
                     e0.y = pack16(na, na);
                 }
-                *reinterpret_cast<uint4*>(dstA + mainA + swz_offset(r, 0, 32)) = e0;
-                *reinterpret_cast<uint4*>(dstA + mainA + swz_offset(r, 1, 32)) = make_uint4(0, 0, 0, 0);
-                qc[ab][r] = make_qc(qs[h], Ur[h]);
-                qidx[ab][r] = qr[h];
+                qc_all[qt][ab][r] = make_float4(qs[h].x, -qs[h].z, qs[h].w, Ur[h]);
+                qidx_all[qt][ab][r] = qr[h];
+                *reinterpret_cast<uint4*>(dstA + mainT + swz_offset(r, 0, 32)) = e0;
+                *reinterpret_cast<uint4*>(dstA + mainT + swz_offset(r, 1, 32)) = make_uint4(0, 0, 0, 0);
             }
             // this thread's copies have landed; make them and the stores above
             // visible to the tensor core (async proxy)
             cp_async_wait_all();
             fence_proxy_async_smem();
             mbar_arrive(&afull[ab]);
-            mbar_arrive(&iq_empty[slot]);
+            if (nrows == 0) break;
         }
-    } else if (warp >= 4 && warp < 8) {
-        // ------------------------------------------------ screening
-        const int er = 32 * (warp & 3) + lane;  // query row of the group = TMEM lane
-        const uint32_t tl = tmem + (uint32_t(32 * (warp & 3)) << 16);
-        for (uint32_t it = 0, tc = 0;; ++it) {
-            const int slot = int(it % TC_IQ);
-            if (!wait(&iq_full[slot], (it / TC_IQ) & 1u)) break;
-            const TcItem dc = iq[slot];
-            if (dc.r0 == 0xFFFFFFFFu) break;
+        cp_async_wait_all();
+    } else if (warp >= 8) {
+        // ------------------------------------------------ screening of query tile qt
+        const int er = 32 * (warp & 3) + lane;  // query row of the tile = TMEM lane
+        const int sr = int(qt) * TC_M + er;     // this thread's column of the survivor buffer
+        const uint32_t tl = tmem + (uint32_t(32 * (warp & 3)) << 16) + qt * NACC * TC_N;
+        uint32_t tc = 0;
+        int nb = 0;  // survivors buffered by this thread
+        // append the buffered survivors to their queries' lists (the atomics in
+        // flight together)
+        auto flush = [&]() {
+            uint2 e[TC_SBUF];
+            uint32_t pos[TC_SBUF];
+#pragma unroll
+            for (int i = 0; i < TC_SBUF; ++i)
+                if (i < nb) {
+                    e[i] = sbuf[i * SW + sr];
+                    pos[i] = atomicAdd(a.surv_cnt + e[i].y, 1u);
+                }
+#pragma unroll
+            for (int i = 0; i < TC_SBUF; ++i)
+                if (i < nb && pos[i] < uint32_t(a.cap)) a.surv[int64_t(e[i].y) * a.cap + pos[i]] = e[i].x;
+            nb = 0;
+        };
+        for (uint32_t it = 0;; ++it) {
             const uint32_t ab = it % NA;
             if (!wait(&afull[ab], (it / NA) & 1u)) break;
-            TcQConst cur = qc[ab][er];
+            const TcWork wk = work[ab];
+            if (wk.nrows == 0) break;
+            const float4 q4 = qc_all[qt][ab][er];
+            const uint32_t qi = qidx_all[qt][ab][er];
+            const int ntiles = int((wk.nrows + TC_N - 1) / TC_N);
+            uint32_t s = wk.t0 % uint32_t(S);
+            TcQConst cur;
+            cur.qn2 = q4.x;
+            cur.Aq1 = q4.y;
+            cur.Cq = q4.z;
+            cur.U = q4.w;
+            cur.Uthr = sc2 * q4.w - (1.0f - a.Bn) * q4.x + q4.z;
+            cur.Uoff = (1.0f + a.Bn) * q4.x + 2.0f * a.Bn * sc2 * xmax * xmax + 2.0f * q4.y * sc * xmax + q4.z;
             const float U0 = cur.U;
-            const uint32_t qi = qidx[ab][er];
             const bool active = qi != 0xFFFFFFFFu;
             const int64_t q = active ? int64_t(qi) : 0;
             const int64_t src = EXCL && active ? a.query_src[q] : -1;
-            const int ntiles = int((dc.r1 - dc.r0 + TC_N - 1) / TC_N);
             float ubl[KMAX];  // k smallest upper bounds seen for this query in this item
 #pragma unroll
             for (int u = 0; u < KMAX; ++u) ubl[u] = INFINITY;
-            int nb = 0;  // survivors buffered in shared memory by this thread
-            // append the buffered survivors (minus excluded rows) to the query's
-            // list, then tighten U with their upper bounds (deferred: a stale U
-            // only admits more rows)
-            auto flush = [&]() {
-                if (FAST) {
-                    if (nb > 0) {
-                        const uint32_t pos = atomicAdd(a.surv_cnt + q, uint32_t(nb));
-                        for (int i = 0; i < nb; ++i)
-                            if (pos + uint32_t(i) < uint32_t(a.cap)) a.surv[q * a.cap + pos + i] = sbuf_row[i * 128 + er];
+            auto bound = [&](float ub) {  // an upper bound on a candidate's distance
+                if (ub < ubl[KMAX - 1]) {
+#pragma unroll
+                    for (int u = KMAX - 1; u > 0; --u) {
+                        const float pu = ubl[u - 1];
+                        if (pu > ub) ubl[u] = pu;
+                        else if (ubl[u] > ub) ubl[u] = ub;
                     }
-                    nb = 0;
-                    return;
+                    if (ubl[0] > ub) ubl[0] = ub;
                 }
-                int keep = 0;
+                // the k-th smallest bound of k distinct candidates bounds the k-th best
+                float kth = INFINITY;
+#pragma unroll
+                for (int u = 0; u < KMAX; ++u)
+                    if (u == a.k - 1) kth = ubl[u];
+                if (kth < cur.U) {
+                    cur.U = kth;
+                    cur.Uthr = sc2 * cur.U - (1.0f - a.Bn) * cur.qn2 + cur.Cq;
+                }
+            };
+            // EXCL: append the buffered survivors, minus the excluded rows, to the
+            // query's list, and tighten U with the others' upper bounds (deferred: a
+            // stale U only admits more rows)
+            auto flush_excl = [&]() {
                 for (int i = 0; i < nb; ++i) {
-                    const uint32_t row = sbuf_row[i * 128 + er];
-                    if (EXCL && src >= 0) {
-                        const int64_t id = int64_t(__ldg(a.perm + row));
-                        int64_t dr = id / a.grid_w - src / a.grid_w, dcc = id % a.grid_w - src % a.grid_w;
-                        dr = dr < 0 ? -dr : dr;
-                        dcc = dcc < 0 ? -dcc : dcc;
-                        if ((dr > dcc ? dr : dcc) <= a.radius) continue;
-                    }
-                    sbuf_row[keep * 128 + er] = row;
-                    sbuf_val[keep * 128 + er] = sbuf_val[i * 128 + er];
-                    ++keep;
-                }
-                if (keep > 0) {
-                    const uint32_t pos = atomicAdd(a.surv_cnt + q, uint32_t(keep));
-                    for (int i = 0; i < keep; ++i) {
-                        const uint32_t row = sbuf_row[i * 128 + er];
-                        const float D = sbuf_val[i * 128 + er];
-                        if (pos + uint32_t(i) < uint32_t(a.cap)) a.surv[q * a.cap + pos + i] = row;
-                        // d~ + E <= D + (1+B)|q|^2 + 2B|x|^2 + 2A'|x| + Cq (scaled units)
-                        const float4 rs = __ldg(a.rowstat + row);
-                        const float ubs = (D + (1.0f + a.Bn) * cur.qn2 + 2.0f * a.Bn * sc2 * rs.z +
-                                           2.0f * cur.Aq1 * sc * rs.y + cur.Cq) * (1.0f + 1e-6f);
-                        const float ub = fmaxf(ubs * inv_sc2, 0.0f);
-                        if (ub < ubl[KMAX - 1]) {
-#pragma unroll
-                            for (int u = KMAX - 1; u > 0; --u) {
-                                const float pu = ubl[u - 1];
-                                if (pu > ub) ubl[u] = pu;
-                                else if (ubl[u] > ub) ubl[u] = ub;
-                            }
-                            if (ubl[0] > ub) ubl[0] = ub;
-                        }
-                    }
-                    // the k-th smallest bound of k distinct candidates bounds the k-th best
-                    float kth = INFINITY;
-#pragma unroll
-                    for (int u = 0; u < KMAX; ++u)
-                        if (u == a.k - 1) kth = ubl[u];
-                    if (kth < cur.U) {
-                        cur.U = kth;
-                        cur.Uthr = sc2 * cur.U - (1.0f - a.Bn) * cur.qn2 + cur.Cq;
-                    }
+                    const uint32_t row = sbuf[i * SW + sr].x;
+                    const int64_t id = int64_t(__ldg(a.perm + row));
+                    int64_t dr = id / a.grid_w - src / a.grid_w, dcc = id % a.grid_w - src % a.grid_w;
+                    dr = dr < 0 ? -dr : dr;
+                    dcc = dcc < 0 ? -dcc : dcc;
+                    if (src >= 0 && (dr > dcc ? dr : dcc) <= a.radius) continue;
+                    const uint32_t pos = atomicAdd(a.surv_cnt + q, 1u);
+                    if (pos < uint32_t(a.cap)) a.surv[q * a.cap + pos] = row;
+                    bound(fmaxf((__uint_as_float(sbuf[i * SW + sr].y) + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
                 }
                 nb = 0;
             };
             bool ok = true;
             for (int t = 0; t < ntiles; ++t, ++tc) {
-                const int acc = int(tc % NACC);
+                const uint32_t acc = tc % NACC;
                 if (!wait(&accfull[acc], (tc / NACC) & 1u)) { ok = false; break; }
+                if (lane == 0) {
+                    // the tile's MMAs have completed: its operands are free
+                    if ((warp & 3) == 0) mbar_arrive(&bempty[s]);
+                    if (t == ntiles - 1) mbar_arrive(&aempty[ab]);
+                }
+                if (++s == uint32_t(S)) s = 0;
                 tc_fence_after();
-                const int y0 = int(dc.r0) + t * TC_N;
-                const int nvalid = min(TC_N, int(dc.r1) - y0);
+                const int y0 = int(wk.r0) + t * TC_N;
+                const int nvalid = min(TC_N, int(wk.nrows) - t * TC_N);
                 for (int c0 = 0; c0 < nvalid; c0 += 64) {
                     float v[64], m[2];
                     tmem_ld32x2_min(tl + uint32_t(acc * TC_N + c0), v, m[0], m[1]);
+                    if (c0 + 64 >= nvalid) {
+                        // the accumulator's values are in registers: one arrival per warp
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&accempty[acc]);
+                    }
                     const float vmin = fminf(m[0], m[1]);
                     const int lim = nvalid - c0;
                     // columns past the item's rows (the next cone's, in the last
@@ -544,6 +646,7 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
                         }
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
+                            if (m[h] > cur.Uthr) continue;
                             uint32_t mask = 0;
 #pragma unroll
                             for (int j = 0; j < 32; ++j) mask |= (v[32 * h + j] <= cur.Uthr ? 1u : 0u) << j;
@@ -553,14 +656,20 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
                             while (mask) {
                                 const int j = __ffs(int(mask)) - 1;
                                 mask &= mask - 1u;
-                                if (nb == TC_SBUF) flush();
-                                sbuf_row[nb * 128 + er] = uint32_t(y0 + c0 + 32 * h + j);
+                                if (nb == TC_SBUF) {
+                                    if (EXCL) flush_excl();
+                                    else flush();
+                                }
+                                float val = 0.f;
                                 if (!FAST) {
-                                    float val = v[32 * h];
+                                    val = v[32 * h];
 #pragma unroll
                                     for (int u = 1; u < 32; ++u) val = u == j ? v[32 * h + u] : val;
-                                    sbuf_val[nb * 128 + er] = val;
                                 }
+                                // d~ + E <= D + Uoff (scaled units)
+                                if (!FAST && !EXCL) bound(fmaxf((val + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
+                                sbuf[nb * SW + sr] =
+                                    make_uint2(uint32_t(y0 + c0 + 32 * h + j), EXCL ? __float_as_uint(val) : qi);
                                 ++nb;
                             }
                         }
@@ -570,7 +679,7 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
                         const int col = lane + 32 * (c0 / 64 % 2);
                         if (col < lim) {
                             const int row = y0 + c0 + col;
-                            const float* xr = a.xs + size_t(row) * a.d_pad;
+                            const float* xr = a.xs + size_t(row) * DP;
                             const float* yr = a.Y + q * int64_t(a.d);
                             float dot = 0.f;
                             for (int i = 0; i < a.d; ++i) dot = fmaf(xr[i], yr[i], dot);
@@ -591,115 +700,63 @@ __global__ void __launch_bounds__(AT ? TC_AT_THREADS : TC_ROLE_THREADS, AT ? 1 :
                         }
                     }
                 }
-                // every lane's loads of this accumulator are complete: one arrival per warp
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&accempty[acc]);
             }
             if (!ok) break;
-            if (active) {
+            if (EXCL) {
+                flush_excl();
+            } else if (__any_sync(0xffffffffu, nb > TC_SBUF / 2)) {
                 flush();
+            }
+            if (active) {
                 if (cur.U < U0) atomicMin(a.Ubits + q, __float_as_uint(fmaxf(cur.U, 0.0f)));
             }
-            // the warp has read its query constants and the item descriptor
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&aempty[ab]);
-                mbar_arrive(&iq_empty[slot]);
-            }
         }
-    } else if (AT && warp >= 8) {
-        // ------------------------------------------------ query tiles into TMEM (AT, d_pad = 128)
-        const int r = 32 * (warp & 3) + lane;  // query row of the tile = TMEM lane
-        const uint32_t tl = tmem + (uint32_t(32 * (warp & 3)) << 16);
-        const int cpr = a.d_pad / 8;  // 16-byte chunks of a 16-bit query row (16)
-        for (uint32_t it = 0;; ++it) {
-            const int slot = int(it % TC_IQ);
-            if (!wait(&iq_full[slot], (it / TC_IQ) & 1u)) break;
-            const TcItem d = iq[slot];
-            if (d.r0 == 0xFFFFFFFFu) break;
-            const uint32_t ab = it % NA;
-            if (it >= NA && !wait(&aempty[ab], ((it / NA) - 1) & 1u)) break;
-            // the MMAs that read this buffer's columns have completed
-            tc_fence_after();
-            const uint32_t qr = uint32_t(r) < d.qn ? a.qlist[d.qbeg + r] / uint32_t(a.S) : 0xFFFFFFFFu;
-            const bool active = qr != 0xFFFFFFFFu;
-            const uint4* src = reinterpret_cast<const uint4*>(a.Y16 + int64_t(active ? qr : 0u) * a.d_pad);
-            uint4 row[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) row[c] = active && c < cpr ? __ldg(src + c) : make_uint4(0, 0, 0, 0);
-            float4 qs = make_float4(0.f, 0.f, 0.f, 0.f);
-            float Ur = INFINITY;
-            uint4 e0 = make_uint4(0, 0, 0, 0);
-            if (active) {
-                qs = a.qstat[qr];
-                Ur = __uint_as_float(a.Ubits[qr]);
-                // extra block: (1, 1, -A', -A', 0, ...) against (|x|^2 hi, lo, |x| hi, lo, 0, ...)
-                const uint16_t one = to16_rn<PREC>(1.0f), na = to16_rn<PREC>(qs.z);  // exact
-                e0.x = pack16(one, one);
-                e0.y = pack16(na, na);
-            }
-            qc[ab][r] = make_qc(qs, Ur);
-            qidx[ab][r] = qr;
-            const uint32_t tcol = tl + NACC * TC_N + ab * acols;
-            tmem_st64(tcol, row);
-            tmem_st8(tcol + uint32_t(a.d_pad / 2), e0, make_uint4(0, 0, 0, 0));
-            // the tile's columns are written; order them before the MMAs
-            tmem_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&afull[ab]);
-                mbar_arrive(&iq_empty[slot]);
-            }
-        }
+        if (!EXCL) flush();
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-// AT: cone-tile stages in the shared memory the query tiles leave (d_pad = 128:
-// five of 36 KB)
-__host__ inline int tc_stages_at(int d_pad) { return d_pad == 128 ? 5 : tc_stages(d_pad); }
-
-inline size_t tc_smem_bytes(int d_pad, bool at)
-{
-    const size_t tileA = size_t(TC_M) * d_pad * 2 + TC_M * 32, tileB = size_t(TC_N) * d_pad * 2 + TC_N * 32;
-    if (at) return 1024 + size_t(tc_stages_at(d_pad)) * tileB;
-    const size_t need = 1024 + size_t(tc_abufs(d_pad)) * tileA + size_t(tc_stages(d_pad)) * tileB;
-    // at least 80 KB so that at most two CTAs (2 x 256 TMEM columns) share an SM
-    return need < 80u * 1024u ? 80u * 1024u : need;
-}
-
-template <int KMAX, bool EXCL, int PREC, bool DEBUG, bool AT = false>
+template <int KMAX, bool EXCL, bool DEBUG, int DP>
 static int launch_tc_t(const void* maps, const TcArgs& a, cudaStream_t st, int num_sms)
 {
-    const size_t smem = tc_smem_bytes(a.d_pad, AT);
-    auto kern = tc_scan_kernel<KMAX, EXCL, PREC, DEBUG, AT>;
-    constexpr int threads = AT ? TC_AT_THREADS : TC_ROLE_THREADS;
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    // resident CTAs per SM: registers, shared memory (228 KB per SM, 1 KB
-    // reserved per CTA) and TMEM (512 columns: 256 per CTA, all of them with AT)
-    cudaFuncAttributes fa{};
-    cudaFuncGetAttributes(&fa, kern);
-    const int regs = fa.numRegs > 0 ? fa.numRegs : 255;
-    const int by_regs = 65536 / (regs * threads);
-    const int by_smem = int((228u * 1024u) / (smem + 1024u + size_t(fa.sharedSizeBytes)));
-    int occ = by_regs < by_smem ? by_regs : by_smem;
-    if (occ > (AT ? 1 : 2)) occ = AT ? 1 : 2;
-    if (occ < 1) occ = 1;
+    constexpr int need = 1024 + (TC_QT * tc_slots(DP) + tc_stages(DP)) * tc_tile_bytes(DP);
+    // over half of an SM's shared memory: a CTA takes all of its TMEM columns
+    constexpr int smem = need < 116 * 1024 ? 116 * 1024 : need;
+    auto kern = tc_scan_kernel<KMAX, EXCL, DEBUG, DP>;
+    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaGetLastError();
     const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
-    kern<<<unsigned(num_sms * occ), threads, smem, st>>>(m[0], m[1], a);
+    kern<<<unsigned(num_sms), TC_THREADS, smem, st>>>(m[0], m[1], a);
     return count_launch();
 }
 
-// tc_scan_tmem.cu: the launches with the query tiles in TMEM (d_pad = 128,
-// no exclusion), bound check on or off
-int launch_tc_scan_tmem(const void* maps, const TcArgs& a, int k, int prec, bool debug, cudaStream_t st, int num_sms);
+// Launch of one (exclusion, check) class over k and the padded widths.
+template <bool EXCL, bool DEBUG, int DP>
+static int launch_tc_k(const void* maps, const TcArgs& a, int k, cudaStream_t st, int num_sms)
+{
+    if (k <= 1) return launch_tc_t<1, EXCL, DEBUG, DP>(maps, a, st, num_sms);
+    if (k <= 4) return launch_tc_t<4, EXCL, DEBUG, DP>(maps, a, st, num_sms);
+    if (k <= 16) return launch_tc_t<16, EXCL, DEBUG, DP>(maps, a, st, num_sms);
+    return launch_tc_t<32, EXCL, DEBUG, DP>(maps, a, st, num_sms);
+}
+template <bool EXCL, bool DEBUG>
+static int launch_tc_dp(const void* maps, const TcArgs& a, int k, cudaStream_t st, int num_sms)
+{
+    switch (a.d_pad) {
+    case 16: return launch_tc_k<EXCL, DEBUG, 16>(maps, a, k, st, num_sms);
+    case 32: return launch_tc_k<EXCL, DEBUG, 32>(maps, a, k, st, num_sms);
+    case 64: return launch_tc_k<EXCL, DEBUG, 64>(maps, a, k, st, num_sms);
+    case 128: return launch_tc_k<EXCL, DEBUG, 128>(maps, a, k, st, num_sms);
+    }
+    return -2;
+}
 
-// tc_scan_debug.cu: the same launch with the bound check compiled in
-int launch_tc_scan_debug(const void* maps, const TcArgs& a, int k, int prec, bool excl, cudaStream_t st, int num_sms);
+// One translation unit per launch class (they compile in parallel):
+// tc_scan_excl.cu: exclusion radius, bound check on or off
+int launch_tc_scan_excl(const void* maps, const TcArgs& a, int k, bool debug, cudaStream_t st, int num_sms);
+// tc_scan_debug.cu: the plain launch with the bound check compiled in
+int launch_tc_scan_debug(const void* maps, const TcArgs& a, int k, cudaStream_t st, int num_sms);
 
 }  // namespace osann
