@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(256) data_keys_row_kernel(const float* __restr
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
         // nonnegative floats order like their bits
-        if (lane == 0 && nmax > 0.0f && finite_f(nmax)) atomicMax(maxn2_bits, __float_as_uint(nmax));
+        // (+inf: a norm past the fp32 range, or a non-finite row, which is reported)
+        if (lane == 0 && nmax > 0.0f) atomicMax(maxn2_bits, __float_as_uint(nmax));
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, ST_NONFINITE_DATA);
 }
@@ -329,7 +330,8 @@ __global__ void __launch_bounds__(256) data_keys_kernel(const float* __restrict_
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) nmax = fmaxf(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
         // nonnegative floats order like their bits
-        if (lane == 0 && nmax > 0.0f && finite_f(nmax)) atomicMax(maxn2_bits, __float_as_uint(nmax));
+        // (+inf: a norm past the fp32 range, or a non-finite row, which is reported)
+        if (lane == 0 && nmax > 0.0f) atomicMax(maxn2_bits, __float_as_uint(nmax));
     }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(status, ST_NONFINITE_DATA);
 }
@@ -436,7 +438,7 @@ __global__ void __launch_bounds__(256) row_norm_max_kernel(const float* __restri
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if ((threadIdx.x & 31) == 0 && best > 0.0f && finite_f(best)) atomicMax(maxn2_bits, __float_as_uint(best));
+    if ((threadIdx.x & 31) == 0 && best > 0.0f) atomicMax(maxn2_bits, __float_as_uint(best));
 }
 
 int launch_row_norm_max(const float* X, int64_t n, int d, uint32_t* maxn2_bits, cudaStream_t st, int num_sms)

@@ -1348,7 +1348,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                 rc = cuda_fail(cudaGetLastError(), "osann_search: fork");
             if (!rc) {
                 StageScope s(OSANN_STAGE_TC_PREP, side.st);
-                rc = launch_tc_query_prep(prec, Y, Q, ix->d, ix->d_pad, probes, P_eff, ix->offsets, uint32_t(ix->NC),
+                rc = launch_tc_query_prep(prec, Y, Q, ix->d, ix->d_pad, probes, P_eff, ix->N, ix->offsets, uint32_t(ix->NC),
                                           ix->xs, k, ix->cdot2[prec], ix->cabs[prec], ix->tcs + 4 * prec, ix->perm,
                                           src, grid_w, radius, TC_SURV_CAP, w + L.yb,
                                           reinterpret_cast<float4*>(w + L.qstat),

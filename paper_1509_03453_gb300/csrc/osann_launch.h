@@ -160,11 +160,12 @@ size_t tc_map_bytes();
 int tc_encode_rows_map(void* map_out, const void* x16, int64_t N, int d_pad, int prec);  // d_pad 0: extra block
 int launch_tc_rows(int prec, const float* xs, const float4* rowstat, int64_t N, int d_pad, const uint32_t* maxn2_bits,
                    float* tcs, void* x16, void* xe16, cudaStream_t st, int num_sms);
+// probes null: the seed is spread over all N rows; seed_rows 0: by batch size and k
 int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, const uint32_t* probes,
-                         int64_t P_eff, const uint32_t* offsets, uint32_t NC, const float* xs, int k, float cdot2,
-                         float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src, int64_t grid_w,
-                         int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits, uint32_t* surv_cnt,
-                         cudaStream_t st);
+                         int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
+                         float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
+                         int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
+                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows = 0);
 int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float4* rowstat, const void* Y16,
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,

@@ -8,13 +8,28 @@ namespace osann {
 
 // ---------------------------------------------------------------- query prep
 
-// One warp per query: 16-bit copy of -2 s y, scaled norms and A', survivor
-// counter reset, and the initial upper bound U: the k-th smallest canonical
-// fp32 distance over the rows of the first probed cones (in probe order,
-// excluded rows skipped, at least `seed_rows` rows when the cones hold them),
-// inflated by the fp32 error bound; +inf if fewer than k rows.  A query too large for the 16-bit range is left to the
-// rerank's full scan (its survivor count is set above the capacity).
+// 16-bit copy of -2 s y, scaled norms and A', survivor counter reset, and the
+// initial upper bound U of each query: the k-th smallest canonical fp32 distance
+// over a seed of rows (excluded rows skipped), inflated by the fp32 error bound;
+// +inf if the seed holds fewer than k.  The seed is the rows of the first probed
+// cones, in probe order, up to `seed_rows` (probes non-null), or `seed_rows` rows
+// spread evenly over all N (probes null: linear search).  A query too large for
+// the 16-bit range is left to an exact scan (its survivor count is set above the
+// capacity), and so is every query when a row norm passed the fp32 range
+// (tcs[3] = inf).
+//
+// The rows are read at random, so what bounds the kernel is the latency of the
+// chain list entry -> cone offsets -> rows.  From PREP_SMALL_Q queries up, a warp
+// per query hides it behind the other warps and takes a cone at a time.  A small
+// batch leaves the chip idle instead: there, PREP_SMALL warps share a query; 32
+// probes are looked up at once (a lane each), the next 32 while these ones' rows
+// are read, and a warp scan of the cone sizes lays thin cones end to end, so that
+// every warp has TC_SEED_ILP row groups in flight.  Measured: 77 queries at
+// d = 64, 132 -> 31 us; one query at d = 32, 49 -> 17 us; 4096 queries at d = 64,
+// one warp each 28, the lookup of 32 cones 36 us.
 constexpr int TC_SEED_ILP = 8;  // row groups loaded per iteration
+constexpr int PREP_SMALL = 8;   // warps per query of a small batch
+constexpr int PREP_SMALL_Q = 1024;
 
 // Rows scanned exactly for a query's initial bound.  A large batch keeps
 // tightening its bounds as items finish, so a short seed suffices (64 rows
@@ -33,23 +48,44 @@ static int tc_seed_rows(int64_t Q, int k)
     return int(r < 64 ? 64 : (r > 1024 ? 1024 : r));
 }
 
+struct PrepArgs {
+    const float* Y;
+    int64_t Q;
+    int d, d_pad;
+    const uint32_t* probes;  // null: the seed is spread over all N rows
+    int64_t P_eff, N;
+    const uint32_t* offsets;
+    uint32_t NC;
+    const float* xs;
+    int k;
+    float cdot2, cabs;
+    const float* tcs;
+    const uint32_t* perm;
+    const int64_t* query_src;
+    int64_t grid_w;
+    int radius, cap, seed_rows;
+    uint16_t* Y16;
+    float4* qstat;
+    uint32_t* Ubits;
+    uint32_t* surv_cnt;
+};
+
 template <int F, int PREC, int KMAX>
-__global__ void __launch_bounds__(128) tc_query_prep_kernel(const float* __restrict__ Y, int64_t Q, int d, int d_pad,
-                                                            const uint32_t* __restrict__ probes, int64_t P_eff,
-                                                            const uint32_t* __restrict__ offsets, uint32_t NC,
-                                                            const float* __restrict__ xs, int k, float cdot2,
-                                                            float cabs, const float* __restrict__ tcs,
-                                                            const uint32_t* __restrict__ perm,
-                                                            const int64_t* __restrict__ query_src, int64_t grid_w,
-                                                            int radius, int cap, uint16_t* __restrict__ Y16,
-                                                            float4* __restrict__ qstat, uint32_t* __restrict__ Ubits,
-                                                            uint32_t* __restrict__ surv_cnt, int seed_rows)
+__global__ void __launch_bounds__(128)
+    tc_query_prep_kernel(const PrepArgs a)
 {
+    const float* const Y = a.Y;
+    const int d = a.d, d_pad = a.d_pad, k = a.k, cap = a.cap, radius = a.radius, seed_rows = a.seed_rows;
+    const int64_t Q = a.Q, P_eff = a.P_eff, grid_w = a.grid_w;
+    const uint32_t* __restrict__ const probes = a.probes;
+    const uint32_t* __restrict__ const offsets = a.offsets;
+    const float* __restrict__ const xs = a.xs;
+    const uint32_t NC = a.NC;
     const int lane = threadIdx.x & 31;
     const int64_t q = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (q >= Q) return;  // whole warp
     const float* y = Y + q * int64_t(d);
-    const float sc = tcs[0];
+    const float sc = a.tcs[0];
     float s = 0.f, amax = 0.f;
     for (int c = lane * 4; c < d_pad; c += 128) {
         float4 v;
@@ -62,7 +98,7 @@ __global__ void __launch_bounds__(128) tc_query_prep_kernel(const float* __restr
         uint2 pk;
         pk.x = pack16(to16_rn<PREC>(-2.f * sc * v.x), to16_rn<PREC>(-2.f * sc * v.y));
         pk.y = pack16(to16_rn<PREC>(-2.f * sc * v.z), to16_rn<PREC>(-2.f * sc * v.w));
-        *reinterpret_cast<uint2*>(Y16 + q * int64_t(d_pad) + c) = pk;
+        *reinterpret_cast<uint2*>(a.Y16 + q * int64_t(d_pad) + c) = pk;
         s = fmaf(v.x, v.x, s);
         s = fmaf(v.y, v.y, s);
         s = fmaf(v.z, v.z, s);
@@ -90,7 +126,7 @@ __global__ void __launch_bounds__(128) tc_query_prep_kernel(const float* __restr
         qv[f].z = c + 2 < d ? y[c + 2] : 0.f;
         qv[f].w = c + 3 < d ? y[c + 3] : 0.f;
     }
-    const int64_t src = query_src ? query_src[q] : -1;
+    const int64_t src = a.query_src ? a.query_src[q] : -1;
     uint64_t list[KMAX];
     topk_init<KMAX>(list, k);
     int scanned = 0;
@@ -119,7 +155,7 @@ __global__ void __launch_bounds__(128) tc_query_prep_kernel(const float* __restr
                 bool usable = rr[u] < o1;
                 if (usable && src >= 0) {
                     // an excluded row is not a candidate and cannot seed the bound
-                    const int64_t id = int64_t(perm[rr[u]]);
+                    const int64_t id = int64_t(a.perm[rr[u]]);
                     int64_t dr = id / grid_w - src / grid_w, dc = id % grid_w - src % grid_w;
                     dr = dr < 0 ? -dr : dr;
                     dc = dc < 0 ? -dc : dc;
@@ -153,11 +189,197 @@ __global__ void __launch_bounds__(128) tc_query_prep_kernel(const float* __restr
         // scaled units: |q'| = s |q|; A' = 2c|q'| + Cabs, inflated by 2^-14
         // (16-bit hi/lo split of |x|) and rounded up to the 16-bit format
         const float qn = sc * sc * s, qnorm = sc * sqrtf(s);
-        const float A = (cdot2 * qnorm + cabs) * (1.0f + 6.1035156e-5f);
+        const float A = (a.cdot2 * qnorm + a.cabs) * (1.0f + 6.1035156e-5f);
         const float Ap = from16<PREC>(to16_ru<PREC>(A));
-        qstat[q] = make_float4(qn, qnorm, -Ap, cabs * qnorm);
-        Ubits[q] = __float_as_uint(U);
-        surv_cnt[q] = unscreenable ? uint32_t(cap) + 1u : 0u;
+        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm);
+        a.Ubits[q] = __float_as_uint(U);
+        a.surv_cnt[q] = unscreenable || a.tcs[3] > 3.4e38f ? uint32_t(cap) + 1u : 0u;
+    }
+}
+
+// The same for a small batch (a block per query), and for a seed spread over all
+// rows (probes null).
+template <int F, int PREC, int KMAX>
+__global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(const PrepArgs a)
+{
+    constexpr int WPQ = PREP_SMALL;
+    const int lane = threadIdx.x & 31, wq = int(threadIdx.x >> 5);  // warp of the query
+    const int64_t q = blockIdx.x;
+    const float* y = a.Y + q * int64_t(a.d);
+    const float sc = a.tcs[0];
+
+    // seed rows: TPR lanes per row (canonical distance, as in the rerank)
+    const int n4 = a.d_pad >> 2;
+    const int TPR = n4 / F, CPP = 32 / TPR;
+    const int g = lane / TPR, sub = lane % TPR;
+    float4 qv[F];
+#pragma unroll
+    for (int f = 0; f < F; ++f) {
+        const int c = 4 * (sub * F + f);
+        qv[f].x = c + 0 < a.d ? y[c + 0] : 0.f;
+        qv[f].y = c + 1 < a.d ? y[c + 1] : 0.f;
+        qv[f].z = c + 2 < a.d ? y[c + 2] : 0.f;
+        qv[f].w = c + 3 < a.d ? y[c + 3] : 0.f;
+    }
+    const int64_t src = a.query_src ? a.query_src[q] : -1;
+    uint64_t list[KMAX];
+    topk_init<KMAX>(list, a.k);
+    // the rows t0 + u * CPP + g (u < TC_SEED_ILP) below `end`, row_of(t) -> row
+    auto scan = [&](int t0, int end, auto row_of) {
+        float4 xv[TC_SEED_ILP][F];
+        uint32_t rr[TC_SEED_ILP];
+        bool live[TC_SEED_ILP];
+#pragma unroll
+        for (int u = 0; u < TC_SEED_ILP; ++u) {
+            const int t = t0 + u * CPP + g;
+            live[u] = t < end;
+            rr[u] = row_of(live[u] ? t : end - 1);
+        }
+#pragma unroll
+        for (int u = 0; u < TC_SEED_ILP; ++u) {
+            const float4* xr = reinterpret_cast<const float4*>(a.xs + size_t(rr[u]) * a.d_pad) + sub * F;
+#pragma unroll
+            for (int f = 0; f < F; ++f) xv[u][f] = xr[f];
+        }
+#pragma unroll
+        for (int u = 0; u < TC_SEED_ILP; ++u) {
+            float cpart[F];
+#pragma unroll
+            for (int f = 0; f < F; ++f) cpart[f] = sq4(xv[u][f], qv[f]);
+            const float dist = lane_tree(pair_tree<F>(cpart), TPR);
+            bool usable = live[u];
+            if (usable && src >= 0) {
+                // an excluded row is not a candidate and cannot seed the bound
+                const int64_t id = int64_t(a.perm[rr[u]]);
+                int64_t dr = id / a.grid_w - src / a.grid_w, dc = id % a.grid_w - src % a.grid_w;
+                dr = dr < 0 ? -dr : dr;
+                dc = dc < 0 ? -dc : dc;
+                usable = (dr > dc ? dr : dc) > a.radius;
+            }
+            if (sub == 0 && usable) {
+                const uint64_t v = pack_di(dist, rr[u]);
+                if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
+            }
+        }
+    };
+    const int step = WPQ * TC_SEED_ILP * CPP;
+    if (!a.probes) {
+        for (int t0 = wq * TC_SEED_ILP * CPP; t0 < a.seed_rows; t0 += step)
+            scan(t0, a.seed_rows, [&](int t) { return uint32_t(int64_t(t) * a.N / a.seed_rows); });
+    } else {
+        const uint32_t* pl = a.probes + q * a.P_eff;
+        auto probe = [&](int64_t p) -> uint32_t { return p < a.P_eff ? pl[p] : 0xFFFFFFFFu; };
+        uint32_t st = 0, sz = 0, b1 = probe(32 + lane);
+        auto cone = [&](uint32_t b, uint32_t& s0, uint32_t& n) {
+            s0 = 0;
+            n = 0;
+            if (b < a.NC) {
+                s0 = a.offsets[b];
+                n = a.offsets[b + 1] - s0;
+            }
+        };
+        cone(probe(lane), st, sz);
+        int scanned = 0;
+        for (int64_t p0 = 0; p0 < a.P_eff && scanned < a.seed_rows; p0 += 32) {
+            // the next 32 cones, and the probes after them
+            uint32_t st1, sz1;
+            cone(b1, st1, sz1);
+            b1 = probe(p0 + 64 + lane);
+            // no more rows of a cone than the seed still needs
+            const uint32_t need = uint32_t(a.seed_rows - scanned);
+            sz = sz < need ? sz : need;
+            uint32_t incl = sz;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const uint32_t all = __shfl_sync(0xffffffffu, incl, 31);
+            const int total = int(all < need ? all : need);
+            for (int t0 = wq * TC_SEED_ILP * CPP; t0 < total; t0 += step)
+                scan(t0, total, [&](int t) {
+                    // the first cone whose inclusive sum passes t
+                    int c = 0;
+#pragma unroll
+                    for (int w = 16; w > 0; w >>= 1)
+                        if (__shfl_sync(0xffffffffu, incl, c + w - 1) <= uint32_t(t)) c += w;
+                    return __shfl_sync(0xffffffffu, st, c) + uint32_t(t) -
+                           (__shfl_sync(0xffffffffu, incl, c) - __shfl_sync(0xffffffffu, sz, c));
+                });
+            scanned += total;
+            st = st1;
+            sz = sz1;
+        }
+    }
+    // k-th smallest: k rounds of warp minimum over each warp's lists, then over the
+    // warps' k best, gathered in shared memory
+    __shared__ uint64_t best_sh[WPQ * KMAX];
+    float U = INFINITY;
+    {
+        float kth = INFINITY;
+        int found = 0;
+        auto rounds = [&](uint64_t* keep) {
+            for (int j = 0; j < a.k; ++j) {
+                const uint64_t head = topk_head<KMAX>(list, a.k);
+                const uint64_t best = warp_min_u64(head);
+                if (keep && lane == 0) keep[j] = best;
+                if (best == EMPTY_DI) {
+                    if (keep) continue;
+                    break;
+                }
+                if (head == best) topk_remove<KMAX>(list, a.k, best);
+                kth = di_dist(best);
+                ++found;
+            }
+        };
+        rounds(best_sh + wq * KMAX);
+        __syncthreads();
+        if (wq != 0) return;
+        topk_init<KMAX>(list, a.k);
+        for (int i = lane; i < WPQ * a.k; i += 32) {
+            const uint64_t v = best_sh[(i / a.k) * KMAX + i % a.k];
+            if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
+        }
+        found = 0;
+        rounds(nullptr);
+        // the canonical fp32 distance is within 6.6e-7 relative of the exact one
+        if (found == a.k) U = kth * (1.0f + 2e-6f) + 1e-30f;
+    }
+    float s = 0.f, amax = 0.f;
+    for (int c = lane * 4; c < a.d_pad; c += 128) {
+        float4 v;
+        v.x = c + 0 < a.d ? y[c + 0] : 0.f;
+        v.y = c + 1 < a.d ? y[c + 1] : 0.f;
+        v.z = c + 2 < a.d ? y[c + 2] : 0.f;
+        v.w = c + 3 < a.d ? y[c + 3] : 0.f;
+        // -2 s y: the factor is a power of two, so the 16-bit value is exact
+        // up to the 16-bit rounding of s y itself
+        uint2 pk;
+        pk.x = pack16(to16_rn<PREC>(-2.f * sc * v.x), to16_rn<PREC>(-2.f * sc * v.y));
+        pk.y = pack16(to16_rn<PREC>(-2.f * sc * v.z), to16_rn<PREC>(-2.f * sc * v.w));
+        *reinterpret_cast<uint2*>(a.Y16 + q * int64_t(a.d_pad) + c) = pk;
+        s = fmaf(v.x, v.x, s);
+        s = fmaf(v.y, v.y, s);
+        s = fmaf(v.z, v.z, s);
+        s = fmaf(v.w, v.w, s);
+        amax = fmaxf(amax, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+    }
+    // fp16 holds |v| < 65504; keep 2 |s y| and the norm terms well inside
+    const bool unscreenable = PREC == 1 && (2.f * sc * amax > 16384.f || sc * sc * s > 32768.f);
+    if (lane == 0) {
+        // scaled units: |q'| = s |q|; A' = 2c|q'| + Cabs, inflated by 2^-14
+        // (16-bit hi/lo split of |x|) and rounded up to the 16-bit format
+        const float qn = sc * sc * s, qnorm = sc * sqrtf(s);
+        const float A = (a.cdot2 * qnorm + a.cabs) * (1.0f + 6.1035156e-5f);
+        const float Ap = from16<PREC>(to16_ru<PREC>(A));
+        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm);
+        a.Ubits[q] = __float_as_uint(U);
+        a.surv_cnt[q] = unscreenable || a.tcs[3] > 3.4e38f ? uint32_t(a.cap) + 1u : 0u;
     }
 }
 
@@ -170,8 +392,8 @@ __global__ void tc_scale_kernel(const uint32_t* __restrict__ maxn2_bits, float* 
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int e = 0;
-    const float m = __uint_as_float(*maxn2_bits);
-    if (PREC == 1 && m > 0.0f) {
+    const float m = __uint_as_float(*maxn2_bits);  // +inf: a row's norm passed the fp32 range (nothing is screened)
+    if (PREC == 1 && m > 0.0f && m < INFINITY) {
         int x;
         frexpf(m, &x);  // m < 2^x
         const int t = 14 - x;
@@ -388,31 +610,51 @@ int tc_encode_rows_map(void* map_out, const void* x16, int64_t N, int d_pad, int
 size_t tc_map_bytes() { return 2 * sizeof(CUtensorMap); }
 
 int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, const uint32_t* probes,
-                         int64_t P_eff, const uint32_t* offsets, uint32_t NC, const float* xs, int k, float cdot2,
-                         float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src, int64_t grid_w,
-                         int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits, uint32_t* surv_cnt,
-                         cudaStream_t st)
+                         int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
+                         float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
+                         int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
+                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows)
 {
     if (Q == 0) return 0;
-    const unsigned blocks = unsigned((Q * 32 + 127) / 128);
-    uint16_t* y16 = static_cast<uint16_t*>(Y16);
-    const int seed_rows = tc_seed_rows(Q, k);
-#define OSANN_PREP(F, PR, KM)                                                                                       \
-    tc_query_prep_kernel<F, PR, KM><<<blocks, 128, 0, st>>>(Y, Q, d, d_pad, probes, P_eff, offsets, NC, xs, k, cdot2, \
-                                                            cabs, tcs, perm, query_src, grid_w, radius, cap, y16,    \
-                                                            qstat, Ubits, surv_cnt, seed_rows)
-#define OSANN_PREP_K(F, PR)             \
-    if (k <= 1) OSANN_PREP(F, PR, 1);      \
-    else if (k <= 4) OSANN_PREP(F, PR, 4); \
-    else if (k <= 16) OSANN_PREP(F, PR, 16); \
-    else OSANN_PREP(F, PR, 32);
-    if (d_pad <= 128) {
-        if (prec == 0) { OSANN_PREP_K(1, 0) }
-        else { OSANN_PREP_K(1, 1) }
-    } else {
-        if (prec == 0) { OSANN_PREP_K(2, 0) }
-        else { OSANN_PREP_K(2, 1) }
-    }
+    PrepArgs a{};
+    a.Y = Y;
+    a.Q = Q;
+    a.d = d;
+    a.d_pad = d_pad;
+    a.probes = probes;
+    a.P_eff = P_eff;
+    a.N = N;
+    a.offsets = offsets;
+    a.NC = NC;
+    a.xs = xs;
+    a.k = k;
+    a.cdot2 = cdot2;
+    a.cabs = cabs;
+    a.tcs = tcs;
+    a.perm = perm;
+    a.query_src = query_src;
+    a.grid_w = grid_w;
+    a.radius = radius;
+    a.cap = cap;
+    a.seed_rows = seed_rows > 0 ? seed_rows : tc_seed_rows(Q, k);
+    a.Y16 = static_cast<uint16_t*>(Y16);
+    a.qstat = qstat;
+    a.Ubits = Ubits;
+    a.surv_cnt = surv_cnt;
+    // d_pad <= 128: one float4 piece per lane
+    const bool small = Q < PREP_SMALL_Q || !probes;
+#define OSANN_PREP(PR, KM)                                                                              \
+    do {                                                                                                \
+        if (small) tc_query_prep_block_kernel<1, PR, KM><<<unsigned(Q), 32 * PREP_SMALL, 0, st>>>(a);   \
+        else tc_query_prep_kernel<1, PR, KM><<<unsigned((Q * 32 + 127) / 128), 128, 0, st>>>(a);        \
+    } while (0)
+#define OSANN_PREP_K(PR)             \
+    if (k <= 1) OSANN_PREP(PR, 1);      \
+    else if (k <= 4) OSANN_PREP(PR, 4); \
+    else if (k <= 16) OSANN_PREP(PR, 16); \
+    else OSANN_PREP(PR, 32);
+    if (prec == 0) { OSANN_PREP_K(0) }
+    else { OSANN_PREP_K(1) }
 #undef OSANN_PREP_K
 #undef OSANN_PREP
     return count_launch();
