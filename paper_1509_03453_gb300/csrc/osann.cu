@@ -1544,10 +1544,40 @@ int osann_screen_stats(const osann_index* ix, void* stream, int64_t* out4)
     return OSANN_OK;
 }
 
+// Linear search through the fp16 screen from this many rows up (the seed alone
+// reads 512): below, the fp32 tile scan.
+constexpr int64_t DENSE_MIN_ROWS = 8192;
+// Queries per pass: a query's survivor list and constants take 4 KB.
+constexpr int64_t DENSE_MAX_Q = 16384;
+static bool linear_dense(const osann_index* ix) { return ix->tc_ready[1] && ix->N >= DENSE_MIN_ROWS; }
+
+static DenseIndex dense_index(const osann_index* ix)
+{
+    DenseIndex di{};
+    di.maps = ix->tmap[1];
+    di.perm = ix->perm;
+    di.offsets = ix->offsets;
+    di.rowstat = ix->rowstat;
+    di.tcs = ix->tcs + 4;
+    di.xs = ix->xs;
+    di.N = ix->N;
+    di.NC = uint32_t(ix->NC);
+    di.d = ix->d;
+    di.d_pad = ix->d_pad;
+    di.cdot2 = ix->cdot2[1];
+    di.Bn = ix->Bn;
+    di.cabs = ix->cabs[1];
+    di.status = ix->status;
+    di.diag = ix->diag;
+    return di;
+}
+
 size_t osann_bruteforce_workspace_size(const osann_index* ix, int64_t Q, int32_t k)
 {
     if (!ix || Q < 0 || k < 1 || k > MAX_K) return 0;
-    return al256(bruteforce_ws_bytes(ix->N, ix->d_pad, Q, k)) + 256;
+    if (!linear_dense(ix)) return al256(bruteforce_ws_bytes(ix->N, ix->d_pad, Q, k)) + 256;
+    if (Q > DENSE_MAX_Q) Q = DENSE_MAX_Q;
+    return al256(bruteforce_ws_bytes(ix->N, ix->d_pad, Q, k)) + al256(dense_ws_bytes(Q, ix->d_pad, k)) + 256;
 }
 
 int osann_bruteforce(const osann_index* ix, const float* d_queries, const int64_t* d_query_src, int64_t Q, int32_t k,
@@ -1581,8 +1611,27 @@ int osann_bruteforce(const osann_index* ix, const float* d_queries, const int64_
     int rc;
     {
         StageScope s(OSANN_STAGE_BRUTEFORCE, st);
-        rc = launch_bruteforce_rows(ix->xs, ix->perm, ix->N, ix->d_pad, d_queries, ix->d, Q, k, d_query_src, grid_w,
-                                    radius, w, counter, d_ids, d_sqdists, ix->status, st, ix->num_sms);
+        // the 16-bit screen over all rows; the queries it leaves (a survivor list
+        // overflowed, or a vector out of the 16-bit range) take the fp32 scan
+        rc = 0;
+        const bool dense = linear_dense(ix);
+        const int64_t step = dense && Q > DENSE_MAX_Q ? DENSE_MAX_Q : Q;
+        for (int64_t q0 = 0; q0 < Q && !rc; q0 += step) {
+            const int64_t n = Q - q0 < step ? Q - q0 : step;
+            const float* y = d_queries + q0 * ix->d;
+            const int64_t* src = d_query_src ? d_query_src + q0 : nullptr;
+            const uint32_t* left = nullptr;
+            if (dense) {
+                char* dw = w + al256(bruteforce_ws_bytes(ix->N, ix->d_pad, step, k));
+                left = dense_ovf(dw, n, ix->d_pad, k);
+                rc = launch_dense(dense_index(ix), y, n, k, src, grid_w, radius, nullptr, dw, d_ids + q0 * k,
+                                  d_sqdists + q0 * k, debug_checks(), st, ix->num_sms);
+            }
+            if (!rc)
+                rc = launch_bruteforce_rows(ix->xs, ix->perm, ix->N, ix->d_pad, y, ix->d, n, k, src, grid_w, radius, w,
+                                            counter, d_ids + q0 * k, d_sqdists + q0 * k, ix->status, st, ix->num_sms,
+                                            left);
+        }
     }
     if (owned) dev_free(owned, need, st);
     return rc;

@@ -145,12 +145,13 @@ int launch_tile_scan(const float* xs, const uint32_t* offsets, const uint32_t* p
 int launch_merge(const uint64_t* partial, int64_t Q, int64_t slots, int k, const uint32_t* perm_or_null,
                  int64_t* out_ids, float* out_d, cudaStream_t st);
 
-// linear search (scan_batched.cu): dense tile scan over all rows of xs
+// linear search (scan_batched.cu): dense tile scan over all rows of xs.  qsel
+// (nullable): device list [count, q_0, ...] of the queries to search
 size_t bruteforce_ws_bytes(int64_t N, int d_pad, int64_t Q, int k);
 int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int d_pad, const float* Y, int d,
                            int64_t Q, int k, const int64_t* query_src, int64_t grid_w, int radius, void* ws,
                            uint32_t* counter, int64_t* out_ids, float* out_d, uint32_t* status, cudaStream_t st,
-                           int num_sms);
+                           int num_sms, const uint32_t* qsel = nullptr);
 
 // tc_scan.cu: 16-bit tensor-core screening + fp32 rerank.  prec 0 = bf16,
 // 1 = fp16 (with an exact power-of-two scale of the data and queries)
@@ -166,16 +167,60 @@ int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, 
                          float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
                          int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
                          uint32_t* surv_cnt, cudaStream_t st, int seed_rows = 0);
+// Work items of a dense phase (linear search, or a search whose cones are screened
+// together): tile chunks x groups of 256 queries.  The phase's 128-row tiles are
+// mul * (0, 1, 2, ...), or with `skip` mul * (the numbers not divisible by 8);
+// chunk c takes every `chunks`-th of them from c on.
+struct TcDense {
+    uint32_t N, Q, tiles, chunks, groups, mul, n_items;
+    int skip;
+};
+// dense (non-null): its items instead of b's list, and no tightening of U
 int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float4* rowstat, const void* Y16,
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
-                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms);
+                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
+                   const TcDense* dense = nullptr);
 int launch_tc_rerank(const float* xs, int d_pad, const uint32_t* perm, const uint32_t* offsets, uint32_t NC,
                      const float* Y, int d, int64_t Q, const uint32_t* probes, int64_t P_eff, const uint32_t* surv_cnt,
                      const uint32_t* surv, int cap, int k, const int64_t* query_src, int64_t grid_w, int radius,
                      unsigned long long* diag, uint32_t* ovf, int64_t* out_ids, float* out_d, cudaStream_t st);
 // ovf: device list [count, q_0, ...] of the queries whose survivor list
 // overflowed (Q + 1 words); they are left to the plain scan
+
+// tc_dense.cu: dense screening of every row for every query, in phases: after each
+// one the survivors are evaluated exactly and the bounds tightened.  Linear
+// search, or (member non-null) only the rows of the cones that a query probes
+// count.  The seed: rows spread over the index, or the first probed cones'.
+struct DenseMember {
+    const uint8_t* qorder;  // Q x dk magnitude orders
+    const uint32_t* qsign;
+    const uint32_t* keys;   // cone id per point
+    const uint64_t* binom;
+    int dk, L;
+    int64_t P_eff;
+    const uint32_t* seed_probes;  // Q x seed_P first probed cones
+    int64_t seed_P;
+};
+struct DenseIndex {
+    const void* maps;
+    const uint32_t *perm, *offsets;
+    const float4* rowstat;
+    const float *tcs, *xs;
+    int64_t N;
+    uint32_t NC;
+    int d, d_pad;
+    float cdot2, Bn, cabs;
+    uint32_t* status;
+    unsigned long long* diag;
+};
+size_t dense_ws_bytes(int64_t Q, int d_pad, int k);
+// the device list [count, q_0, ...] of the queries left to an exact scan (survivor
+// list overflowed, or out of the 16-bit range), inside the workspace
+uint32_t* dense_ovf(void* ws, int64_t Q, int d_pad, int k);
+int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const int64_t* query_src, int64_t grid_w,
+                 int radius, const DenseMember* member, void* ws, int64_t* out_ids, float* out_d, int debug,
+                 cudaStream_t st, int num_sms);
 
 }  // namespace osann

@@ -562,7 +562,8 @@ struct TileArgs {
     int64_t S;                 // slots per query
     int64_t grid_w;
     int64_t N, Q;              // dense mode sizes
-    int64_t n_groups, n_items_dense;
+    int64_t n_chunks;
+    const uint32_t* qsel;      // dense mode: device list [count, q_0, ...] of the queries (null: all Q)
     int d_pad, d, k, radius;
     int dense;                 // 1: linear search items
 };
@@ -573,17 +574,26 @@ struct ItemDesc {
     uint32_t chunk;       // dense: chunk index = slot offset
 };
 
-__device__ __forceinline__ ItemDesc load_item(const TileArgs& a, uint32_t item, int G)
+// queries of a dense pass
+__device__ __forceinline__ int64_t dense_queries(const TileArgs& a)
+{
+    if (!a.qsel) return a.Q;
+    const int64_t n = int64_t(a.qsel[0]);
+    return n < a.Q ? n : a.Q;
+}
+
+__device__ __forceinline__ ItemDesc load_item(const TileArgs& a, uint32_t item, int G, int64_t nq)
 {
     ItemDesc it;
     if (a.dense) {
-        const uint32_t c = item / uint32_t(a.n_groups), g = item % uint32_t(a.n_groups);
+        const uint32_t n_groups = uint32_t((nq + G - 1) / G);
+        const uint32_t c = item / n_groups, g = item % n_groups;
         it.row0 = c * BF_CHUNK_ROWS;
         const int64_t e = int64_t(it.row0) + BF_CHUNK_ROWS;
         it.row1 = uint32_t(e < a.N ? e : a.N);
         it.qbeg = g * uint32_t(G);
         const int64_t qe = int64_t(it.qbeg) + G;
-        it.qn = uint32_t((qe < a.Q ? qe : a.Q) - it.qbeg);
+        it.qn = uint32_t((qe < nq ? qe : nq) - it.qbeg);
         it.chunk = c;
     } else {
         const uint4 d = a.items[item];
@@ -610,7 +620,8 @@ __global__ void __launch_bounds__(TILE_THREADS) tile_scan_kernel(const TileArgs 
     const int G = TILE_THREADS / TPR;
     const int RPC = TILE_STAGE_FLOATS / a.d_pad;
     const int qs = tid / TPR, sub = tid % TPR;
-    const uint32_t n_items = a.dense ? uint32_t(a.n_items_dense) : *a.n_items_dev;
+    const int64_t nq = a.dense ? dense_queries(a) : 0;
+    const uint32_t n_items = a.dense ? uint32_t(a.n_chunks * ((nq + G - 1) / G)) : *a.n_items_dev;
 
     // producer state (thread 0 only)
     bool done = false;
@@ -623,7 +634,7 @@ __global__ void __launch_bounds__(TILE_THREADS) tile_scan_kernel(const TileArgs 
                 done = true;
                 break;
             }
-            const ItemDesc d = load_item(a, it, G);
+            const ItemDesc d = load_item(a, it, G, nq);
             cur_item = int(it);
             cur = d.row0;
             cur_end = d.row1;
@@ -665,12 +676,13 @@ __global__ void __launch_bounds__(TILE_THREADS) tile_scan_kernel(const TileArgs 
         if (m.z != item) {
             // first chunk of a new item: load this thread's query slice
             item = m.z;
-            const ItemDesc d = load_item(a, uint32_t(item), G);
+            const ItemDesc d = load_item(a, uint32_t(item), G, nq);
             active = uint32_t(qs) < d.qn;
             int64_t q = 0;
             if (active) {
                 if (a.dense) {
                     q = int64_t(d.qbeg) + qs;
+                    if (a.qsel) q = int64_t(a.qsel[1 + q]);
                     slot = q * a.S + d.chunk;
                 } else {
                     slot = int64_t(a.qlist[d.qbeg + qs]);
@@ -821,11 +833,16 @@ int launch_tile_scan(const float* xs, const uint32_t* offsets, const uint32_t* p
 
 template <int KMAX>
 __global__ void __launch_bounds__(128) merge_kernel(const uint64_t* __restrict__ partial, int64_t Q, int64_t S, int k,
-                                                    int64_t* __restrict__ out_ids, float* __restrict__ out_d)
+                                                    int64_t* __restrict__ out_ids, float* __restrict__ out_d,
+                                                    const uint32_t* __restrict__ qsel)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t q = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    int64_t q = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (q >= Q) return;
+    if (qsel) {  // the listed queries only
+        if (q >= int64_t(qsel[0])) return;
+        q = int64_t(qsel[1 + q]);
+    }
     const uint64_t* p = partial + q * S * k;
     const int64_t n = S * k;
     // each lane keeps the k best of its share, then k rounds of warp minimum
@@ -847,17 +864,23 @@ __global__ void __launch_bounds__(128) merge_kernel(const uint64_t* __restrict__
     }
 }
 
+static int launch_merge_sel(const uint64_t* partial, int64_t Q, int64_t S, int k, int64_t* out_ids, float* out_d,
+                            const uint32_t* qsel, cudaStream_t st)
+{
+    if (Q == 0) return 0;
+    const unsigned blocks = unsigned((Q * 32 + 127) / 128);
+    if (k <= 1) merge_kernel<1><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d, qsel);
+    else if (k <= 4) merge_kernel<4><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d, qsel);
+    else if (k <= 16) merge_kernel<16><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d, qsel);
+    else merge_kernel<32><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d, qsel);
+    return count_launch();
+}
+
 int launch_merge(const uint64_t* partial, int64_t Q, int64_t S, int k, const uint32_t* perm_or_null, int64_t* out_ids,
                  float* out_d, cudaStream_t st)
 {
     (void)perm_or_null;
-    if (Q == 0) return 0;
-    const unsigned blocks = unsigned((Q * 32 + 127) / 128);
-    if (k <= 1) merge_kernel<1><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d);
-    else if (k <= 4) merge_kernel<4><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d);
-    else if (k <= 16) merge_kernel<16><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d);
-    else merge_kernel<32><<<blocks, 128, 0, st>>>(partial, Q, S, k, out_ids, out_d);
-    return count_launch();
+    return launch_merge_sel(partial, Q, S, k, out_ids, out_d, nullptr, st);
 }
 
 // ---------------------------------------------------------------- linear search
@@ -869,8 +892,9 @@ size_t bruteforce_ws_bytes(int64_t N, int d_pad, int64_t Q, int k)
     return size_t(Q) * size_t(S) * size_t(k) * 8 + 256;
 }
 
-__global__ void fill_u64_kernel(uint64_t* __restrict__ p, int64_t n, uint64_t v)
+__global__ void fill_u64_kernel(uint64_t* __restrict__ p, int64_t n, uint64_t v, const uint32_t* __restrict__ qsel)
 {
+    if (qsel && qsel[0] == 0) return;  // no query listed
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
         p[i] = v;
 }
@@ -878,7 +902,7 @@ __global__ void fill_u64_kernel(uint64_t* __restrict__ p, int64_t n, uint64_t v)
 int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int d_pad, const float* Y, int d,
                            int64_t Q, int k, const int64_t* query_src, int64_t grid_w, int radius, void* ws,
                            uint32_t* counter, int64_t* out_ids, float* out_d, uint32_t* status, cudaStream_t st,
-                           int num_sms)
+                           int num_sms, const uint32_t* qsel)
 {
     if (Q == 0) return 0;
     const int64_t S = (N + BF_CHUNK_ROWS - 1) / BF_CHUNK_ROWS;
@@ -887,12 +911,10 @@ int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int
     int64_t fb = (np + 255) / 256;
     if (fb > 8 * num_sms) fb = 8 * num_sms;
     if (fb < 1) fb = 1;
-    fill_u64_kernel<<<unsigned(fb), 256, 0, st>>>(partial, np, EMPTY_DI);
+    fill_u64_kernel<<<unsigned(fb), 256, 0, st>>>(partial, np, EMPTY_DI, qsel);
     int rc = count_launch();
     if (rc) return rc;
     if (N > 0) {
-        const int DPT = d_pad == 16 ? 16 : 32;
-        const int G = TILE_THREADS / (d_pad / DPT);
         cudaMemsetAsync(counter, 0, 4, st);
         TileArgs a{};
         a.xs = xs;
@@ -906,8 +928,8 @@ int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int
         a.grid_w = grid_w;
         a.N = N;
         a.Q = Q;
-        a.n_groups = (Q + G - 1) / G;
-        a.n_items_dense = S * a.n_groups;
+        a.n_chunks = S;
+        a.qsel = qsel;
         a.d_pad = d_pad;
         a.d = d;
         a.k = k;
@@ -915,7 +937,7 @@ int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int
         a.dense = 1;
         if ((rc = launch_tile_any(a, st, num_sms))) return rc;
     }
-    return launch_merge(partial, Q, S, k, nullptr, out_ids, out_d, st);
+    return launch_merge_sel(partial, Q, S, k, out_ids, out_d, qsel, st);
 }
 
 }  // namespace osann

@@ -664,7 +664,8 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
-                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms)
+                   int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
+                   const TcDense* dense)
 {
     TcArgs a{};
     a.perm = perm;
@@ -674,6 +675,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
     a.tcs = tcs;
     a.query_src = query_src;
     a.items = b.items;
+    if (dense) a.dense = *dense;
     a.n_items_dev = b.n_items_dev;
     a.qlist = b.qlist;
     a.counter = b.counters;
@@ -697,6 +699,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
     a.Bn = Bn;
     a.cabs = cabs;
     const bool excl = query_src != nullptr;
+    if (dense) return launch_tc_scan_dense(maps, a, debug != 0, st, num_sms);
     if (excl) return launch_tc_scan_excl(maps, a, k, debug != 0, st, num_sms);
     if (debug) return launch_tc_scan_debug(maps, a, k, st, num_sms);
     return launch_tc_dp<false, false>(maps, a, k, st, num_sms);

@@ -103,6 +103,7 @@ struct TcArgs {
     const uint4* items;       // (first row, end row, first slot, slot count)
     const uint32_t* n_items_dev;
     const uint32_t* qlist;    // list entries: query * S (+ position)
+    TcDense dense;
     uint32_t* counter;
     uint32_t* Ubits;     // per query: upper bound on the k-th best distance (float bits)
     uint32_t* surv_cnt;  // per query
@@ -131,6 +132,12 @@ struct TcWork {
     uint32_t r0, nrows;  // nrows == 0 marks the end of the work
     uint32_t t0;         // number of the item's first cone tile (stage t0 mod S)
 };
+// First row of the t-th tile of chunk c of a dense phase.
+__device__ __forceinline__ uint32_t dense_row(const TcDense& d, uint32_t c, uint32_t t)
+{
+    const uint32_t p = c + t * d.chunks;
+    return (d.skip ? p + p / 7u + 1u : p) * d.mul * uint32_t(TC_N);
+}
 // An item's queries [off, off + 128) belong to query tile qt: both tiles of an
 // item of more than 128 queries, else the tiles take the items in turn.
 __device__ __forceinline__ bool tc_used(uint32_t qt, uint32_t it, uint32_t qn)
@@ -195,7 +202,9 @@ struct TcQConst {
 
 // DEBUG: check every screened value against an fp32 evaluation of the
 // folded product (a separate instantiation, so the check costs nothing when off)
-template <int KMAX, bool EXCL, bool DEBUG, int DP>
+// DENSE: the items of a.dense (k = 1 class, whatever the search's k: the bounds
+// are left to the phases' exact updates).
+template <int KMAX, bool EXCL, bool DEBUG, int DP, bool DENSE>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_scan_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmap_x,
                    const TcArgs a)
@@ -299,14 +308,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 
     if (warp == 0) {
         // ------------------------------------------------ producer (whole warp)
-        const uint32_t n_items = *a.n_items_dev;
+        const uint32_t n_items = DENSE ? a.dense.n_items : *a.n_items_dev;
         uint32_t it = 0, tc = 0, s = 0, s_ph = 0;
         // lane 0 fetches the next item's index and descriptor one publish ahead,
         // so their latency overlaps the current item's tiles
         uint4 pf = make_uint4(0xFFFFFFFFu, 0, 0, 0);
         auto fetch = [&]() {
             const uint32_t i = atomicAdd(a.counter, 1u);
-            pf = i < n_items ? a.items[i] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
+            if (i >= n_items) {
+                pf = make_uint4(0xFFFFFFFFu, 0, 0, 0);
+            } else if (!DENSE) {
+                pf = a.items[i];
+            } else {
+                // tile chunk (of this phase) and query group, the groups of a chunk in turn
+                const uint32_t c = i / a.dense.groups, q0 = (i - c * a.dense.groups) * uint32_t(TC_QT * TC_M);
+                const uint32_t n = a.dense.Q - q0;
+                const uint32_t nt = (a.dense.tiles - c + a.dense.chunks - 1) / a.dense.chunks;
+                pf = make_uint4(c, c + nt * TC_N, q0, n < uint32_t(TC_QT * TC_M) ? n : uint32_t(TC_QT * TC_M));
+            }
         };
         if (lane == 0) fetch();
         auto publish = [&](uint32_t& r0, uint32_t& r1) -> bool {
@@ -330,7 +349,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             for (int t = 0; t < ntiles; ++t, ++tc) {
                 // stage s = tc mod S, s_ph = (tc / S) & 1: wait for the stage's previous use
                 if (tc >= uint32_t(S) && !wait(&bempty[s], s_ph ^ 1u)) { ok = false; break; }
-                const int y0 = int(cr0) + t * TC_N;
+                const int y0 = DENSE ? int(dense_row(a.dense, cr0, uint32_t(t))) : int(cr0) + t * TC_N;
                 unsigned char* dst = sB + s * uint32_t(tileT);
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&bfull[s], tx_bytes);
@@ -438,7 +457,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             constexpr int E = TC_QT * TC_M / 32;
             uint32_t e[E];
 #pragma unroll
-            for (int i = 0; i < E; ++i) e[i] = !end && uint32_t(lane + 32 * i) < d.qn ? a.qlist[d.qbeg + lane + 32 * i] : 0u;
+            for (int i = 0; i < E; ++i) {
+                const uint32_t j = d.qbeg + uint32_t(lane + 32 * i);
+                e[i] = !end && uint32_t(lane + 32 * i) < d.qn ? (DENSE ? j : a.qlist[j]) : 0u;
+            }
 #pragma unroll
             for (int i = 0; i < E; ++i)
                 iq_q[slot][lane + 32 * i] =
@@ -619,8 +641,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
                 if (++s == uint32_t(S)) s = 0;
                 tc_fence_after();
-                const int y0 = int(wk.r0) + t * TC_N;
-                const int nvalid = min(TC_N, int(wk.nrows) - t * TC_N);
+                const int y0 = DENSE ? int(dense_row(a.dense, wk.r0, uint32_t(t))) : int(wk.r0) + t * TC_N;
+                const int nvalid = min(TC_N, DENSE ? int(a.dense.N) - y0 : int(wk.nrows) - t * TC_N);
                 for (int c0 = 0; c0 < nvalid; c0 += 64) {
                     float v[64], m[2];
                     tmem_ld32x2_min(tl + uint32_t(acc * TC_N + c0), v, m[0], m[1]);
@@ -635,7 +657,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     // columns past the item's rows (the next cone's, in the last
                     // tile) can only lower the minimum: the exact mask below drops them
                     if (active && vmin <= cur.Uthr) {
-                        if (FAST && lim >= 64) {
+                        if (FAST && !DENSE && lim >= 64) {
                             // every column is a row of the item's cone, so the row at
                             // the minimum is a candidate within this bound
                             const float ub = fmaxf((vmin + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f);
@@ -718,13 +740,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <int KMAX, bool EXCL, bool DEBUG, int DP>
+template <int KMAX, bool EXCL, bool DEBUG, int DP, bool DENSE = false>
 static int launch_tc_t(const void* maps, const TcArgs& a, cudaStream_t st, int num_sms)
 {
     constexpr int need = 1024 + (TC_QT * tc_slots(DP) + tc_stages(DP)) * tc_tile_bytes(DP);
     // over half of an SM's shared memory: a CTA takes all of its TMEM columns
     constexpr int smem = need < 116 * 1024 ? 116 * 1024 : need;
-    auto kern = tc_scan_kernel<KMAX, EXCL, DEBUG, DP>;
+    auto kern = tc_scan_kernel<KMAX, EXCL, DEBUG, DP, DENSE>;
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaGetLastError();
     const CUtensorMap* m = static_cast<const CUtensorMap*>(maps);
@@ -753,9 +775,24 @@ static int launch_tc_dp(const void* maps, const TcArgs& a, int k, cudaStream_t s
     return -2;
 }
 
+// Launch of a dense phase.
+template <bool DEBUG>
+static int launch_tc_dense_dp(const void* maps, const TcArgs& a, cudaStream_t st, int num_sms)
+{
+    switch (a.d_pad) {
+    case 16: return launch_tc_t<1, false, DEBUG, 16, true>(maps, a, st, num_sms);
+    case 32: return launch_tc_t<1, false, DEBUG, 32, true>(maps, a, st, num_sms);
+    case 64: return launch_tc_t<1, false, DEBUG, 64, true>(maps, a, st, num_sms);
+    case 128: return launch_tc_t<1, false, DEBUG, 128, true>(maps, a, st, num_sms);
+    }
+    return -2;
+}
+
 // One translation unit per launch class (they compile in parallel):
 // tc_scan_excl.cu: exclusion radius, bound check on or off
 int launch_tc_scan_excl(const void* maps, const TcArgs& a, int k, bool debug, cudaStream_t st, int num_sms);
+// tc_dense.cu: a dense phase
+int launch_tc_scan_dense(const void* maps, const TcArgs& a, bool debug, cudaStream_t st, int num_sms);
 // tc_scan_debug.cu: the plain launch with the bound check compiled in
 int launch_tc_scan_debug(const void* maps, const TcArgs& a, int k, cudaStream_t st, int num_sms);
 
