@@ -415,11 +415,14 @@ struct WsLayout {
     size_t qorder, qsign, probes, partial, qcount, qoff, fill, nitems, item_off, qlist, items, counters, scan_temp;
     size_t yb, qstat, ubits, scnt, surv, ovf, hbuf, yrot, vcl, ptab;
     size_t qset;  // query sets of the tensor-core work list, or SIZE_MAX
+    size_t dense;  // dense screen: its workspace
     size_t total;
     int64_t max_items;
 };
 
-enum SearchMode { MODE_PLAIN = 0, MODE_BATCHED = 1, MODE_BF16 = 2, MODE_FP16 = 3 };
+// MODE_DENSE: every row screened for every query (tc_dense.cu), chosen by
+// OSANN_PATH_AUTO only
+enum SearchMode { MODE_PLAIN = 0, MODE_BATCHED = 1, MODE_BF16 = 2, MODE_FP16 = 3, MODE_DENSE = 4 };
 
 static bool tc_mode(int mode) { return mode == MODE_BF16 || mode == MODE_FP16; }
 
@@ -522,7 +525,9 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
     w.qsign = take(size_t(Qv) * (MAX_D / 32) * 4);
     w.probes = take(size_t(Q) * P_eff * 4);
     w.ptab = take(probe_table_bytes(P_eff));
-    if (mode != MODE_PLAIN) {
+    if (mode == MODE_DENSE) {
+        w.dense = take(dense_ws_bytes(Q, ix->d_pad, k));
+    } else if (mode != MODE_PLAIN) {
         const int G = item_group(ix, mode, group);
         const int64_t n = Q * P_eff;
         int64_t mi = n / G + ix->NC + 1;
@@ -554,7 +559,54 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
     return w;
 }
 
-static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int path)
+// Whether screening every row beats the mode that would be taken otherwise.  All
+// in microseconds on this chip, from these measurements:
+//   dense screen: N / 128 row tiles per 128 queries, 64 cycles per 16 columns at
+//   about 0.8 of the tensor rate; 250 for the phases and updates;
+//   seed rows, read at random: 2.4 TB/s (2800 for 10^4 x 1024 rows of 512 bytes,
+//   28 for 4096 x 64 of 256);
+//   cone by cone, an item (a cone and up to 256 queries) costs its tiles, but at
+//   least DENSE_ITEM_CYCLES however few its rows (5200 measured at d = 128, cones
+//   of 6 rows, 3800 with cones of 25); its work list 10 ps per (query, probe), above
+//   12288 cones (global atomics) 45 ps (5400 for 1.2*10^8); seed and list side by side;
+//   per-query scan of thin cones: 2 TB/s of rows.
+// Only for the set key with a direct table and L <= 4, whose list positions the
+// dense screen recomputes for a survivor's cone.
+constexpr double DENSE_ITEM_CYCLES = 4000.0;
+static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, double cones, int mode)
+{
+    if (!ix->tc_ready[1] || ix->hashed || ix->K || ix->key_mode != OSANN_KEY_SET || ix->L > 4 || ix->N < 8192 ||
+        Q > 65536)
+        return false;
+    const double sm_us = ix->num_sms * 2000.0;  // SM cycles per microsecond of the chip
+    const double row = 4.0 * ix->d_pad, seed_rate = 2.4e6;
+    const double tile = 80.0 * double((ix->d + 15) / 16 + 1);
+    const double dense_us = double((ix->N + 127) / 128) * double((Q + 127) / 128) * tile / sm_us + 250.0 +
+                            double(Q) * 256.0 * row / seed_rate;
+    const double probes = double(Q) * double(P_eff);
+    const double rows = double(ix->N) / cones;  // of an occupied cone
+    // A phase holds eight times the rows before it, so it leaves about 8 k N / M
+    // survivors per query (M its candidates; fewer where the probed cones hold
+    // nearer rows than the others): past the list's capacity the exact scan would
+    // have the work.  (2240 by this count, 85 found, on the descriptor search; 8200
+    // and mostly overflows on a two-basis Gaussian one, 2950 us against 2080.)
+    if (8.0 * k * double(ix->N) > 2500.0 * rows * double(P_eff)) return false;
+    double other;
+    if (mode == MODE_PLAIN) {
+        other = probes * rows * row / 2.0e6 + 20.0;
+    } else {
+        const double hit = probes < cones ? probes : cones;  // cones with work
+        const double groups = std::ceil(probes / hit / 256.0);
+        const double work = 2.0 * std::ceil(rows / 128.0) * tile;
+        const double seed = double(Q) * tc_seed_rows(Q, k) * row / seed_rate;
+        const double list = ix->NC > 12288 ? 150.0 + probes * 45e-6 : 40.0 + probes * 10e-6;
+        other = hit * groups * (work > DENSE_ITEM_CYCLES ? work : DENSE_ITEM_CYCLES) / sm_us +
+                (seed > list ? seed : list) + 60.0;
+    }
+    return dense_us < 0.8 * other;
+}
+
+static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path)
 {
     if (path == OSANN_PATH_PLAIN) return MODE_PLAIN;
     if (path == OSANN_PATH_BATCHED) return MODE_BATCHED;
@@ -571,8 +623,33 @@ static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int path
     const double per_cone = double(Q) * double(P_eff) / cones;
     const double per_query = double(P_eff) * double(ix->N) / double(ix->NC);
     const bool big_queries = per_query >= 16384.0;
-    if (ix->tc_ready[1] && (per_cone >= 8.0 || big_queries)) return MODE_FP16;
-    return per_cone >= 16.0 || big_queries ? MODE_BATCHED : MODE_PLAIN;
+    int mode = per_cone >= 16.0 || big_queries ? MODE_BATCHED : MODE_PLAIN;
+    if (ix->tc_ready[1] && (per_cone >= 8.0 || big_queries)) mode = MODE_FP16;
+    return dense_pays(ix, Q, P_eff, k, cones, mode) ? MODE_DENSE : mode;
+}
+
+// Probed cones looked up for the dense screen's seed (it stops at its rows).
+constexpr int64_t DENSE_SEED_CONES = 512;
+
+static DenseIndex dense_index(const osann_index* ix)
+{
+    DenseIndex di{};
+    di.maps = ix->tmap[1];
+    di.perm = ix->perm;
+    di.offsets = ix->offsets;
+    di.rowstat = ix->rowstat;
+    di.tcs = ix->tcs + 4;
+    di.xs = ix->xs;
+    di.N = ix->N;
+    di.NC = uint32_t(ix->NC);
+    di.d = ix->d;
+    di.d_pad = ix->d_pad;
+    di.cdot2 = ix->cdot2[1];
+    di.Bn = ix->Bn;
+    di.cabs = ix->cabs[1];
+    di.status = ix->status;
+    di.diag = ix->diag;
+    return di;
 }
 
 // ---------------------------------------------------------------- C ABI
@@ -1144,7 +1221,7 @@ size_t osann_search_workspace_size_group(const osann_index* ix, int64_t Q, int32
     if (!ix || Q < 0 || P < 1 || k < 1 || k > MAX_K) return 0;
     if (path < 0 || path > OSANN_PATH_FP16 || group < 0) return 0;
     const int64_t P_eff = p_eff(ix, P);
-    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, path), group).total;
+    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, k, path), group).total;
 }
 
 size_t osann_search_clusters_workspace_size(const osann_index* ix, int64_t Q, int32_t M, int32_t P, int32_t k,
@@ -1154,7 +1231,7 @@ size_t osann_search_clusters_workspace_size(const osann_index* ix, int64_t Q, in
     if (path < 0 || path > OSANN_PATH_FP16) return 0;
     const int Mv = clusters_of(ix, M);
     const int64_t P_eff = Mv * p_eff(ix, P);
-    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, path), 0, Mv).total;
+    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, k, path), 0, Mv).total;
 }
 
 size_t osann_search_workspace_size(const osann_index* ix, int64_t Q, int32_t P, int32_t k, int32_t path)
@@ -1165,13 +1242,15 @@ size_t osann_search_workspace_size(const osann_index* ix, int64_t Q, int32_t P, 
 // Query keys and probe lists.  P_per: positions per key row; Mv: key rows
 // per query (its Mv nearest clusters with ROSANNA+, else 1); the probe list
 // of query q is rows q * Mv .. q * Mv + Mv - 1 in turn (Mv * P_per slots).
+// qsel (nullable): device list [count, q_0, ...] of the queries whose lists are
+// made, their orders already in the workspace.
 static int query_front(const osann_index* ix, const float* Y, int64_t Q, int64_t P_per, int Mv, const WsLayout& L,
-                       char* w, bool init_partial, int k, cudaStream_t st)
+                       char* w, bool init_partial, int k, cudaStream_t st, const uint32_t* qsel = nullptr)
 {
     int rc = 0;
     const int64_t Qv = Q * Mv;
     uint32_t* vcl = ix->K ? reinterpret_cast<uint32_t*>(w + L.vcl) : nullptr;
-    {
+    if (!qsel) {
         StageScope s(OSANN_STAGE_QUERY_ORDER, st);
         // on a rotated basis the magnitude order is that of the query's coordinates there
         const float* Yk = Y;
@@ -1194,6 +1273,7 @@ static int query_front(const osann_index* ix, const float* Y, int64_t Q, int64_t
     if (rc) return rc;
     StageScope s(OSANN_STAGE_PROBES, st);
     ProbeMap pm{};
+    pm.qsel = qsel;
     pm.ordered = ix->key_mode == OSANN_KEY_ORDERED;
     if (ix->hashed) {
         pm.binom_w = ix->binom_w;
@@ -1281,13 +1361,13 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         return OSANN_ERR_UNSUPPORTED;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int mode = choose_mode(ix, Q, P_eff, path);
+    const int mode = choose_mode(ix, Q, P_eff, k, path);
     const int prec = mode == MODE_FP16 ? 1 : 0;
     if (tc_mode(mode)) {
         int trc = ensure_tc(const_cast<osann_index*>(ix), prec, st);
         if (trc) return trc;
     }
-    const bool batched = mode != MODE_PLAIN;
+    const bool batched = mode != MODE_PLAIN && mode != MODE_DENSE;
     const WsLayout L = ws_layout(ix, Q, P_eff, k, mode, group, Mv);
     // the query-side steps read neither the rows, nor a second-level table,
     // nor a basis or centroids of the index only with a plain direct table
@@ -1314,7 +1394,9 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         return OSANN_ERR_INVALID;
     }
     char* w = static_cast<char*>(d_ws);
-    int rc = query_front(ix, Y, Q, P_per, Mv, L, w, mode == MODE_BATCHED, k, fst);
+    // the dense screen needs the first cones only (its seed)
+    const int64_t P_front = mode == MODE_DENSE && P_per > DENSE_SEED_CONES ? DENSE_SEED_CONES : P_per;
+    int rc = query_front(ix, Y, Q, P_front, Mv, L, w, mode == MODE_BATCHED, k, fst);
     if (front.st) {
         // join (also after an error, so that the side stream's work stays ordered before the caller's)
         if (cudaEventRecord(front.join, front.st) != cudaSuccess || cudaStreamWaitEvent(st, front.join, 0) != cudaSuccess)
@@ -1399,6 +1481,32 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                 StageScope s(OSANN_STAGE_MERGE, st);
                 rc = launch_merge(partial, Q, P_eff, k, nullptr, ids, dists, st);
             }
+        }
+    } else if (!rc && mode == MODE_DENSE) {
+        uint32_t* probes = reinterpret_cast<uint32_t*>(w + L.probes);
+        DenseMember m{};
+        m.qorder = reinterpret_cast<const uint8_t*>(w + L.qorder);
+        m.qsign = reinterpret_cast<const uint32_t*>(w + L.qsign);
+        m.keys = ix->keys;
+        m.binom = ix->binom;
+        m.dk = ix->dk;
+        m.L = ix->L;
+        m.P_eff = P_eff;
+        m.seed_probes = probes;
+        m.seed_P = P_front;
+        const uint32_t* left = dense_ovf(w + L.dense, Q, ix->d_pad, k);
+        {
+            StageScope s(OSANN_STAGE_TC_SCAN, st);
+            rc = launch_dense(dense_index(ix), Y, Q, k, src, grid_w, radius, &m, w + L.dense, ids, dists, debug_checks(),
+                              st, ix->num_sms);
+        }
+        // the queries it leaves: their whole probe lists, and the exact scan
+        if (!rc) {
+            if (P_front < P_eff) rc = query_front(ix, Y, Q, P_eff, 1, L, w, false, k, st, left);
+            if (!rc)
+                rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff,
+                                       uint32_t(ix->NC), k, src, grid_w, radius, left, ix->num_sms, ids, dists,
+                                       ix->status, st);
         }
     } else if (!rc) {
         StageScope s(OSANN_STAGE_PLAIN_SCAN, st);
@@ -1547,30 +1655,9 @@ int osann_screen_stats(const osann_index* ix, void* stream, int64_t* out4)
 // Linear search through the fp16 screen from this many rows up (the seed alone
 // reads 512): below, the fp32 tile scan.
 constexpr int64_t DENSE_MIN_ROWS = 8192;
-// Queries per pass: a query's survivor list and constants take 4 KB.
+// Queries per pass: a query's survivor list and constants take 8 KB.
 constexpr int64_t DENSE_MAX_Q = 16384;
 static bool linear_dense(const osann_index* ix) { return ix->tc_ready[1] && ix->N >= DENSE_MIN_ROWS; }
-
-static DenseIndex dense_index(const osann_index* ix)
-{
-    DenseIndex di{};
-    di.maps = ix->tmap[1];
-    di.perm = ix->perm;
-    di.offsets = ix->offsets;
-    di.rowstat = ix->rowstat;
-    di.tcs = ix->tcs + 4;
-    di.xs = ix->xs;
-    di.N = ix->N;
-    di.NC = uint32_t(ix->NC);
-    di.d = ix->d;
-    di.d_pad = ix->d_pad;
-    di.cdot2 = ix->cdot2[1];
-    di.Bn = ix->Bn;
-    di.cabs = ix->cabs[1];
-    di.status = ix->status;
-    di.diag = ix->diag;
-    return di;
-}
 
 size_t osann_bruteforce_workspace_size(const osann_index* ix, int64_t Q, int32_t k)
 {

@@ -83,6 +83,7 @@ struct ProbeMap {
     int M = 1;
     const uint32_t* vcl = nullptr;
     uint64_t ncc_lo = 0, ncc_hi = 0;
+    const uint32_t* qsel = nullptr;  // device list [count, q_0, ...]: only these rows' lists (no clusters)
 };
 // tab: scratch of probe_table_bytes(P_eff) for the per-position ranks and flips
 size_t probe_table_bytes(int64_t P_eff);
@@ -156,12 +157,14 @@ int launch_bruteforce_rows(const float* xs, const uint32_t* perm, int64_t N, int
 // tc_scan.cu: 16-bit tensor-core screening + fp32 rerank.  prec 0 = bf16,
 // 1 = fp16 (with an exact power-of-two scale of the data and queries)
 constexpr int TC_GROUP = 128;  // query rows of an MMA tile; a default work item has two
-constexpr int TC_SURV_CAP = 1024;
+constexpr int TC_SURV_CAP = 1024;   // survivors per query, cone by cone
+constexpr int DENSE_SURV_CAP = 2048;  // and per phase of the dense screen
 size_t tc_map_bytes();
 int tc_encode_rows_map(void* map_out, const void* x16, int64_t N, int d_pad, int prec);  // d_pad 0: extra block
 int launch_tc_rows(int prec, const float* xs, const float4* rowstat, int64_t N, int d_pad, const uint32_t* maxn2_bits,
                    float* tcs, void* x16, void* xe16, cudaStream_t st, int num_sms);
-// probes null: the seed is spread over all N rows; seed_rows 0: by batch size and k
+int tc_seed_rows(int64_t Q, int k);  // rows of a query's seed, by batch size and k
+// probes null: the seed is spread over all N rows; seed_rows 0: tc_seed_rows
 int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, const uint32_t* probes,
                          int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
                          float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,

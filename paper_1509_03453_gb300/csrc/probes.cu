@@ -216,7 +216,11 @@ __global__ void __launch_bounds__(256) probes_kernel(const uint8_t* __restrict__
     if (LC > 0) L = LC;
     __shared__ uint8_t ord[MAX_D];
     __shared__ uint32_t sg[MAX_D / 32];
-    const int64_t q = blockIdx.x;  // row of qorder/qsign
+    int64_t q = blockIdx.x;  // row of qorder/qsign
+    if (pm.qsel) {
+        if (q >= int64_t(pm.qsel[0])) return;
+        q = int64_t(pm.qsel[1 + q]);
+    }
     for (int i = threadIdx.x; i < d; i += blockDim.x) ord[i] = qorder[q * int64_t(d) + i];
     if (threadIdx.x < MAX_D / 32) sg[threadIdx.x] = qsign[q * (MAX_D / 32) + threadIdx.x];
     __syncthreads();

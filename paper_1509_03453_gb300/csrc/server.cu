@@ -328,7 +328,9 @@ int osann_server_create(const osann_index* const* indexes, int32_t n_indexes, co
     // server may run at the largest bucket, plus query and result buffers
     size_t ws = 0;
     for (int i = 0; i < n_indexes; ++i) {
-        ws = std::max(ws, osann_search_workspace_size_group(s->idx[i], max_batch, P[i], k[i], OSANN_PATH_AUTO, 0));
+        // the automatic path differs by batch size, and with it the workspace
+        for (int64_t b : s->buckets)
+            ws = std::max(ws, osann_search_workspace_size_group(s->idx[i], b, P[i], k[i], OSANN_PATH_AUTO, 0));
         for (const Choice& c : candidates(s, i))
             ws = std::max(ws, osann_search_workspace_size_group(s->idx[i], max_batch, P[i], k[i], c.path, c.group));
     }

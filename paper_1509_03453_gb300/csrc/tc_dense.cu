@@ -302,7 +302,7 @@ Ws ws_of(int64_t Q, int d_pad, int k)
     w.qstat = take(size_t(Q) * 16);
     w.ubits = take(size_t(Q) * 4);
     w.scnt = take(size_t(Q) * 4);
-    w.surv = take(size_t(Q) * TC_SURV_CAP * 4);
+    w.surv = take(size_t(Q) * DENSE_SURV_CAP * 4);
     w.best = take(size_t(Q) * k * 8);
     w.ovf = take(size_t(Q + 1) * 4);
     w.counter = take(256);
@@ -353,10 +353,10 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
     uint32_t* surv = reinterpret_cast<uint32_t*>(w + L.surv);
     uint32_t* ovf = reinterpret_cast<uint32_t*>(w + L.ovf);
     uint32_t* counter = reinterpret_cast<uint32_t*>(w + L.counter);
-    const int64_t seed = member ? 2 * DENSE_SEED : DENSE_SEED;
+    const int64_t seed = DENSE_SEED;
     int rc = launch_tc_query_prep(1, Y, Q, ix.d, ix.d_pad, member ? member->seed_probes : nullptr,
                                   member ? member->seed_P : 0, ix.N, ix.offsets, ix.NC, ix.xs, k, ix.cdot2, ix.cabs,
-                                  ix.tcs, ix.perm, query_src, grid_w, radius, TC_SURV_CAP, w + L.yb,
+                                  ix.tcs, ix.perm, query_src, grid_w, radius, DENSE_SURV_CAP, w + L.yb,
                                   reinterpret_cast<float4*>(w + L.qstat), Ubits, scnt, st, int(seed));
     if (rc) return rc;
     cudaMemsetAsync(ovf, 0, 4, st);
@@ -373,7 +373,7 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
     u.d = ix.d;
     u.d_pad = ix.d_pad;
     u.k = k;
-    u.cap = TC_SURV_CAP;
+    u.cap = DENSE_SURV_CAP;
     u.radius = radius;
     u.Q = Q;
     u.grid_w = grid_w;
@@ -410,7 +410,7 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
         dn.n_items = uint32_t(chunks * groups);
         if (dn.n_items > 0) {
             rc = launch_tc_scan(1, ix.maps, ix.perm, ix.rowstat, w + L.yb, reinterpret_cast<float4*>(w + L.qstat), ix.tcs,
-                                nullptr, 0, 0, b, Ubits, scnt, surv, TC_SURV_CAP, ix.status, ix.diag, ix.xs, Y, 1, ix.d,
+                                nullptr, 0, 0, b, Ubits, scnt, surv, DENSE_SURV_CAP, ix.status, ix.diag, ix.xs, Y, 1, ix.d,
                                 ix.d_pad, 1, ix.cdot2, ix.Bn, ix.cabs, debug, st, num_sms, &dn);
             if (rc) return rc;
         }

@@ -41,7 +41,7 @@ constexpr int PREP_SMALL_Q = 1024;
 // seed leaves loose: 1024 rows (on the thin-cone descriptor search, k = 10,
 // Q = 10^4, this cut the survivors from 9.7 to 2.0 million and removed the
 // overflow rescans: 26.2 -> 21.5 ms).
-static int tc_seed_rows(int64_t Q, int k)
+int tc_seed_rows(int64_t Q, int k)
 {
     if (k > 4) return 1024;
     const int64_t r = Q > 0 ? (int64_t(262144) + Q - 1) / Q : 1024;

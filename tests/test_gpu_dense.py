@@ -71,3 +71,48 @@ def test_linear_ranges(osann):
     big = X.copy()
     big[17] = 1e19   # its squared norm passes the fp32 range
     check(osann, big, Y, (3,))
+
+
+# L, d, P (up to past all unflipped profiles), Q: sizes at which the automatic
+# path screens every row and keeps the survivors of probed cones
+@pytest.mark.parametrize("L,d,m,P,Q", [(3, 32, 0, 1500, 1700), (3, 32, 0, 6000, 700), (2, 100, 0, 2600, 1501),
+                                       (2, 100, 0, 9000, 513), (4, 20, 0, 9000, 700), (1, 128, 0, 140, 4500),
+                                       (3, 64, 40, 11_000, 600)])
+def test_thin_cones_match_scan(osann, L, d, m, P, Q):
+    rng = np.random.default_rng(L * 1000 + d + P)
+    N = 30_011 if L > 1 else 9_001
+    X = rng.standard_normal((N, d)).astype(np.float32)
+    X[:, : d // 2] = np.abs(X[:, : d // 2])
+    Y = rng.standard_normal((Q, d)).astype(np.float32)
+    Y[5] *= 1e9          # left to the exact scan
+    Y[6] = 0
+    kw = {}
+    if m:
+        q, _ = np.linalg.qr(rng.standard_normal((d, d)))
+        kw = dict(rot=to_dev(q[:m].astype(np.float32)), rot_offset=to_dev(q[:m].sum(1).astype(np.float32)))
+    idx = osann.Index(to_dev(X), L, **kw)
+    Yd = to_dev(Y)
+    src = to_dev(rng.integers(0, N, Q))
+    for k in (1, 10):
+        if L > 1:  # the dense route: neither the per-query scan nor the cone-major list
+            sizes = {p: idx.workspace_size(Q, P, k, p) for p in ("auto", "plain", "fp16")}
+            assert sizes["auto"] not in (sizes["plain"], sizes["fp16"])
+        same(idx.search(Yd, P, k), idx.search(Yd, P, k, path="plain"))
+        ex = dict(query_src=src, grid_w=173, radius=6)
+        same(idx.search(Yd, P, k, **ex), idx.search(Yd, P, k, path="plain", **ex))
+    assert idx.status() == 0
+    idx.close()
+
+
+def test_thin_cones_overflow(osann):
+    rng = np.random.default_rng(11)
+    base = np.round(3 * rng.standard_normal((300, 32))).astype(np.float32)
+    X = rng.standard_normal((30_000, 32)).astype(np.float32)
+    X[:20_000] = base[rng.integers(0, 6, 20_000)]   # thousands of equal rows: lists overflow
+    Y = np.concatenate([X[:300], rng.standard_normal((1400, 32))]).astype(np.float32)
+    idx = osann.Index(to_dev(X), 3)
+    Yd = to_dev(Y)
+    idx.screen_stats()
+    same(idx.search(Yd, 1500, 4), idx.search(Yd, 1500, 4, path="plain"))
+    assert idx.status() == 0
+    idx.close()
