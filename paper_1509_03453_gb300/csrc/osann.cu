@@ -569,10 +569,15 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
 //   least DENSE_ITEM_CYCLES however few its rows (5200 measured at d = 128, cones
 //   of 6 rows, 3800 with cones of 25); its work list 10 ps per (query, probe), above
 //   12288 cones (global atomics) 45 ps (5400 for 1.2*10^8); seed and list side by side;
-//   per-query scan of thin cones: 2 TB/s of rows.
+//   per-query scan: 6 TB/s of rows.
 // Only for the set key with a direct table and L <= 4, whose list positions the
 // dense screen recomputes for a survivor's cone.
 constexpr double DENSE_ITEM_CYCLES = 4000.0;
+// rows of an occupied cone (of a cone, while the occupied ones are not counted)
+static double rows_per_cone(const osann_index* ix)
+{
+    return double(ix->N) / (ix->occupied > 0 ? double(ix->occupied) : double(ix->NC));
+}
 static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, double cones, int mode)
 {
     if (!ix->tc_ready[1] || ix->hashed || ix->K || ix->key_mode != OSANN_KEY_SET || ix->L > 4 || ix->N < 8192 ||
@@ -584,7 +589,7 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
     const double dense_us = double((ix->N + 127) / 128) * double((Q + 127) / 128) * tile / sm_us + 250.0 +
                             double(Q) * 256.0 * row / seed_rate;
     const double probes = double(Q) * double(P_eff);
-    const double rows = double(ix->N) / cones;  // of an occupied cone
+    const double rows = rows_per_cone(ix);
     // A phase holds eight times the rows before it, so it leaves about 8 k N / M
     // survivors per query (M its candidates; fewer where the probed cones hold
     // nearer rows than the others): past the list's capacity the exact scan would
@@ -593,12 +598,12 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
     if (8.0 * k * double(ix->N) > 2500.0 * rows * double(P_eff)) return false;
     double other;
     if (mode == MODE_PLAIN) {
-        other = probes * rows * row / 2.0e6 + 20.0;
+        other = probes * rows * row / 6.0e6 + 20.0;
     } else {
         const double hit = probes < cones ? probes : cones;  // cones with work
         const double groups = std::ceil(probes / hit / 256.0);
         const double work = 2.0 * std::ceil(rows / 128.0) * tile;
-        const double seed = double(Q) * tc_seed_rows(Q, k) * row / seed_rate;
+        const double seed = double(Q) * tc_seed_rows(Q, k, rows * double(P_eff)) * row / seed_rate;
         const double list = ix->NC > 12288 ? 150.0 + probes * 45e-6 : 40.0 + probes * 10e-6;
         other = hit * groups * (work > DENSE_ITEM_CYCLES ? work : DENSE_ITEM_CYCLES) / sm_us +
                 (seed > list ? seed : list) + 60.0;
@@ -628,6 +633,9 @@ static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
     return dense_pays(ix, Q, P_eff, k, cones, mode) ? MODE_DENSE : mode;
 }
 
+// Rows of an occupied cone, on average, below which a query's warps take cones each
+// in the per-query scan instead of sharing every cone's rows.
+constexpr double THIN_ROWS = 24.0;
 // Probed cones looked up for the dense screen's seed (it stops at its rows).
 constexpr int64_t DENSE_SEED_CONES = 512;
 
@@ -1435,7 +1443,8 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                           src, grid_w, radius, TC_SURV_CAP, w + L.yb,
                                           reinterpret_cast<float4*>(w + L.qstat),
                                           reinterpret_cast<uint32_t*>(w + L.ubits),
-                                          reinterpret_cast<uint32_t*>(w + L.scnt), side.st);
+                                          reinterpret_cast<uint32_t*>(w + L.scnt), side.st,
+                                          tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)));
             }
         }
         if (!rc) {
@@ -1510,7 +1519,13 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         }
     } else if (!rc) {
         StageScope s(OSANN_STAGE_PLAIN_SCAN, st);
-        rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q,
+        // (a shortened wait budget, a test hook, is the staged scan's)
+        if (!plain_wait_budget_set())
+            rc = launch_query_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q,
+                                   reinterpret_cast<uint32_t*>(w + L.probes), P_eff, uint32_t(ix->NC), k, src, grid_w,
+                                   radius, rows_per_cone(ix) >= THIN_ROWS, ids, dists, st);
+        else
+            rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q,
                                reinterpret_cast<uint32_t*>(w + L.probes), P_eff, uint32_t(ix->NC), k, src, grid_w,
                                radius, nullptr, ix->num_sms, ids, dists, ix->status, st);
     }

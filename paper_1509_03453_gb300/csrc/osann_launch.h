@@ -103,13 +103,20 @@ int launch_composite_keys(const uint32_t* asg, int64_t N, uint64_t ncc_lo, uint6
                           uint4* wkeys, cudaStream_t st, int num_sms);
 
 // scan_plain.cu
-// clock budget of the plain scan's stage waits (0: the default, about a second)
+// clock budget of the staged scan's waits (0: the default, about a second)
 void set_plain_wait_budget(long long cycles);
+bool plain_wait_budget_set();
 int launch_plain_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad,
                       const float* Y, int d, int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k,
                       const int64_t* query_src, int64_t grid_w, int radius, const uint32_t* qlist, int num_sms,
                       int64_t* out_ids, float* out_d, uint32_t* status, cudaStream_t st);
 // qlist (nullable): device list [count, q_0, ...] of the queries to scan
+
+// scan_query.cu: the per-query scan, one to sixteen warps per query.  share: fat
+// cones (a query's warps share their rows instead of taking cones each)
+int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
+                     int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
+                     int64_t grid_w, int radius, bool share, int64_t* out_ids, float* out_d, cudaStream_t st);
 
 // scan_batched.cu
 struct BatchedBuffers {
@@ -163,13 +170,14 @@ size_t tc_map_bytes();
 int tc_encode_rows_map(void* map_out, const void* x16, int64_t N, int d_pad, int prec);  // d_pad 0: extra block
 int launch_tc_rows(int prec, const float* xs, const float4* rowstat, int64_t N, int d_pad, const uint32_t* maxn2_bits,
                    float* tcs, void* x16, void* xe16, cudaStream_t st, int num_sms);
-int tc_seed_rows(int64_t Q, int k);  // rows of a query's seed, by batch size and k
-// probes null: the seed is spread over all N rows; seed_rows 0: tc_seed_rows
+// rows of a query's seed, by batch size, k and the candidates M of a query
+int tc_seed_rows(int64_t Q, int k, double M);
+// probes null: the seed is spread over all N rows
 int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, const uint32_t* probes,
                          int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
                          float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
                          int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
-                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows = 0);
+                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows);
 // Work items of a dense phase (linear search, or a search whose cones are screened
 // together): tile chunks x groups of 256 queries.  The phase's 128-row tiles are
 // mul * (0, 1, 2, ...), or with `skip` mul * (the numbers not divisible by 8);

@@ -1,4 +1,6 @@
-// Plain per-query candidate scan (Algorithm 1 with one basis): for each
+// Staged per-query candidate scan (Algorithm 1 with one basis), for the few
+// queries that a screen left to an exact scan, on a device list whose length the
+// host does not know (scan_query.cu is the scan of whole batches): for each
 // query, visit its probed cones in order and compute the exact squared
 // Euclidean distance (Eq. 1) to every point of every visited cone, keeping
 // the k nearest by (distance, id).  Distances are fp32 direct differences.
@@ -44,6 +46,7 @@ constexpr int PLAIN_BAR = 1;              // named barrier of the consumer warps
 static long long g_plain_wait_budget = WAIT_BUDGET_CYCLES;
 
 void set_plain_wait_budget(long long cycles) { g_plain_wait_budget = cycles > 0 ? cycles : WAIT_BUDGET_CYCLES; }
+bool plain_wait_budget_set() { return g_plain_wait_budget != WAIT_BUDGET_CYCLES; }
 
 __device__ __forceinline__ bool excluded_pair(uint32_t id, int64_t src, int64_t grid_w, int radius)
 {

@@ -1,0 +1,256 @@
+// Per-query candidate scan (Algorithm 1 with one basis): for each query, the exact
+// squared Euclidean distance (Eq. 1, fp32) to every point of every probed cone, the
+// k nearest by (distance, id).  One to sixteen warps per query, rows straight from
+// global memory.
+//
+// The staged scan (scan_plain.cu) streams a query's rows through shared memory, one
+// bulk copy per cone; its producer, its per-row shuffles and its single-lane lists
+// bounded it (cones of six rows: 22% of DRAM, 47% of the issue slots, 17 warps per
+// SM).  Here nothing is staged: a lane looks up a probed cone, a warp scan lays 32
+// cones' rows end to end, and eight row loads per lane are in flight at once.  Per
+// batch of eight loads the distances are summed across lanes by halving -- a lane
+// passes on half of its partial sums and keeps the other half, so a batch costs 7
+// to 9 shuffles instead of 40, in the canonical order of additions
+// (osann_device.cuh; only operands of an addition change sides).  The k best are a
+// sorted list over the lanes, so an insertion is a ballot and a shift.  What bounds
+// it now is the rows' reads (6.9 TB/s on thin cones).
+// Measured (us, staged -> this): 10^4 queries, 128 cones of 5.9 rows of d = 128,
+// k = 10, 2070 -> 556; 20000 queries, 64 cones of image patches, d = 64, k = 4, near
+// matches excluded, 3400 -> 601; cones of 500 rows: d = 32, 10^4 queries, 16 cones,
+// k = 10 4880 -> 841, k = 1 1563 -> 828; 20 queries, 20 cones 77 -> 27; d = 64, 300
+// queries, 20 cones, k = 4 192 -> 132; d = 128, 3000 queries 4180 -> 2050.
+#include "osann_device.cuh"
+#include "osann_launch.h"
+
+namespace osann {
+
+namespace {
+
+constexpr int U = 8;  // row loads in flight per lane
+
+struct QueryScanArgs {
+    const float *xs, *Y;
+    const uint32_t *offsets, *perm, *probes;
+    const int64_t* query_src;
+    int64_t Q, P_eff, grid_w;
+    int d, d_pad, k, radius;
+    int share;  // W > 1: the warps share every 32 cones' rows, instead of taking 32 cones each
+    uint32_t NC;
+    int64_t* out_ids;
+    float* out_d;
+};
+
+// TPR lanes per row, F float4 pieces each; W warps per query.
+template <int TPR, int F, bool EXCL, int W>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const QueryScanArgs a)
+{
+    constexpr int CPP = 32 / TPR;     // rows per load instruction
+    constexpr int B = U * CPP;        // rows per batch: 8 .. 64
+    constexpr int RL = B > 32 ? 2 : 1;  // batch rows looked up per lane
+    constexpr int NV = TPR >= U ? 1 : U / TPR;  // row sums a lane ends with
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wq = W == 1 ? 0 : int(threadIdx.x >> 5);
+    const int64_t q = W == 1 ? int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5) : int64_t(blockIdx.x);
+    if (q >= a.Q) return;  // W > 1: never
+    const int g = lane / TPR, sub = lane % TPR;
+    float4 qv[F];
+    {
+        const float* y = a.Y + q * int64_t(a.d);
+#pragma unroll
+        for (int f = 0; f < F; ++f) {
+            const int c = 4 * (sub * F + f);
+            qv[f].x = c + 0 < a.d ? y[c + 0] : 0.f;
+            qv[f].y = c + 1 < a.d ? y[c + 1] : 0.f;
+            qv[f].z = c + 2 < a.d ? y[c + 2] : 0.f;
+            qv[f].w = c + 3 < a.d ? y[c + 3] : 0.f;
+        }
+    }
+    const int64_t src = EXCL ? a.query_src[q] : -1;
+    // the best found, ascending over the lanes (k <= 32); thr: the k-th
+    uint64_t list = EMPTY_DI, thr = EMPTY_DI;
+    auto insert = [&](uint64_t v) {  // v uniform
+        if (v >= thr) return;
+        const int pos = __popc(__ballot_sync(FULL, list < v));
+        const uint32_t lo = __shfl_up_sync(FULL, uint32_t(list), 1), hi = __shfl_up_sync(FULL, uint32_t(list >> 32), 1);
+        if (lane == pos) list = v;
+        else if (lane > pos) list = (uint64_t(hi) << 32) | lo;
+        thr = (uint64_t(__shfl_sync(FULL, uint32_t(list >> 32), a.k - 1)) << 32) |
+              __shfl_sync(FULL, uint32_t(list), a.k - 1);
+    };
+    // the row index, inside its load group, whose sum this lane ends with (its
+    // lowest for TPR < U), from the halving steps below: the top bit first
+    int u0 = 0;
+#pragma unroll
+    for (int s = 0; (1 << s) < (TPR < U ? TPR : U); ++s) u0 |= ((lane >> s) & 1) << (2 - s);
+    const bool primary = sub < U;  // (lanes that share a sum: one of them speaks)
+
+    const uint32_t* pl = a.probes + q * a.P_eff;
+    auto cone = [&](int64_t p, uint32_t& s0, uint32_t& n) {
+        s0 = 0;
+        n = 0;
+        if (p < a.P_eff) {
+            const uint32_t b = __ldg(pl + p);
+            if (b < a.NC) {  // never produced by the probe kernel otherwise; guards the offsets read
+                s0 = __ldg(a.offsets + b);
+                n = __ldg(a.offsets + b + 1) - s0;
+            }
+        }
+    };
+    const bool share = W > 1 && a.share;
+    const int64_t pstep = share ? 32 : 32 * W;
+    const uint32_t tbeg = share ? uint32_t(wq * B) : 0u, tstep = share ? uint32_t(W * B) : uint32_t(B);
+    uint32_t st, sz;
+    cone((share ? 0 : 32 * wq) + lane, st, sz);
+    for (int64_t p0 = share ? 0 : 32 * wq; p0 < a.P_eff; p0 += pstep) {
+        uint32_t st1, sz1;
+        cone(p0 + pstep + lane, st1, sz1);  // the next 32 cones, behind these ones' rows
+        uint32_t incl = sz;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += v;
+        }
+        const uint32_t total = __shfl_sync(FULL, incl, 31);
+        for (uint32_t t0 = tbeg; t0 < total; t0 += tstep) {
+            // rows of the batch: lane l looks up rows l (and l + 32)
+            uint32_t row[RL], id[RL];
+#pragma unroll
+            for (int h = 0; h < RL; ++h) {
+                const uint32_t t = t0 + uint32_t(32 * h + lane);
+                int c = 0;  // the first cone whose inclusive sum passes t
+#pragma unroll
+                for (int w = 16; w > 0; w >>= 1)
+                    if (__shfl_sync(FULL, incl, c + w - 1) <= t) c += w;
+                const uint32_t r = __shfl_sync(FULL, st, c) + t -
+                                   (__shfl_sync(FULL, incl, c) - __shfl_sync(FULL, sz, c));
+                const bool live = t < total && (B >= 32 || lane < B);
+                row[h] = live ? r : 0u;
+                id[h] = live ? __ldg(a.perm + r) : 0u;
+            }
+            float4 xv[U][F];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = u * CPP + g;
+                const uint32_t r = __shfl_sync(FULL, row[RL == 2 && u * CPP >= 32 ? RL - 1 : 0], e & 31);
+                const float4* xr = reinterpret_cast<const float4*>(a.xs + size_t(r) * a.d_pad) + sub * F;
+#pragma unroll
+                for (int f = 0; f < F; ++f) xv[u][f] = __ldg(xr + f);
+            }
+            float v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                float cp[F];
+#pragma unroll
+                for (int f = 0; f < F; ++f) cp[f] = sq4(xv[u][f], qv[f]);
+                v[u] = pair_tree<F>(cp);
+            }
+            // pairwise tree across the TPR lanes: halving while a lane holds several sums
+#pragma unroll
+            for (int s = 0; (1 << s) < TPR; ++s) {
+                const int m = 1 << s;
+                const int half = U >> (s + 1);
+                if (half >= 1) {
+                    const bool up = (lane >> s) & 1;
+#pragma unroll
+                    for (int i = 0; i < half; ++i) {
+                        const float keep = up ? v[i + half] : v[i], give = up ? v[i] : v[i + half];
+                        v[i] = keep + __shfl_xor_sync(FULL, give, m);
+                    }
+                } else {
+                    v[0] += __shfl_xor_sync(FULL, v[0], m);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                const int e = (u0 + i) * CPP + g;
+                const uint32_t lo = __shfl_sync(FULL, id[0], e & 31);
+                const uint32_t hi = RL == 2 ? __shfl_sync(FULL, id[RL - 1], e & 31) : 0u;
+                const uint32_t cid = RL == 2 && e >= 32 ? hi : lo;
+                bool ok = primary && t0 + uint32_t(e) < total && v[i] <= di_dist(thr);
+                if (EXCL && ok && src >= 0) {
+                    int64_t dr = int64_t(cid) / a.grid_w - src / a.grid_w;
+                    int64_t dc = int64_t(cid) % a.grid_w - src % a.grid_w;
+                    dr = dr < 0 ? -dr : dr;
+                    dc = dc < 0 ? -dc : dc;
+                    ok = (dr > dc ? dr : dc) > a.radius;
+                }
+                unsigned m = __ballot_sync(FULL, ok);
+                while (m) {
+                    const int s = __ffs(int(m)) - 1;
+                    m &= m - 1u;
+                    insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)));
+                }
+            }
+        }
+        st = st1;
+        sz = sz1;
+    }
+    if (W > 1) {
+        __shared__ uint64_t sh[W * 32];
+        if (lane < a.k) sh[wq * 32 + lane] = list;
+        __syncthreads();
+        if (wq != 0) return;
+        for (int w = 1; w < W; ++w)
+            for (int j = 0; j < a.k; ++j) insert(sh[w * 32 + j]);
+    }
+    if (lane < a.k) {
+        const uint32_t id = di_id(list);
+        a.out_ids[q * a.k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
+        a.out_d[q * a.k + lane] = di_dist(list);
+    }
+}
+
+template <int TPR, int F, bool EXCL>
+int launch_w(const QueryScanArgs& a, cudaStream_t st)
+{
+    // enough warps for the chip (some 3600 resident): over thin cones one per query
+    // from 2048 queries up and four from 256; over fat ones, whose queries have more
+    // rows, from 4096 and 608 (1000 queries, 20 cones of 504 rows: four 157, sixteen
+    // 180 us; 300 queries: 139 and 49)
+    if (a.Q >= (a.share ? 4096 : 2048)) query_scan_kernel<TPR, F, EXCL, 1><<<unsigned((a.Q + 3) / 4), 128, 0, st>>>(a);
+    else if (a.Q >= (a.share ? 608 : 256)) query_scan_kernel<TPR, F, EXCL, 4><<<unsigned(a.Q), 128, 0, st>>>(a);
+    else query_scan_kernel<TPR, F, EXCL, 16><<<unsigned(a.Q), 512, 0, st>>>(a);
+    return count_launch();
+}
+
+template <bool EXCL>
+int launch_d(const QueryScanArgs& a, cudaStream_t st)
+{
+    switch (a.d_pad) {
+    case 16: return launch_w<4, 1, EXCL>(a, st);
+    case 32: return launch_w<8, 1, EXCL>(a, st);
+    case 64: return launch_w<16, 1, EXCL>(a, st);
+    case 128: return launch_w<32, 1, EXCL>(a, st);
+    }
+    return launch_w<32, 2, EXCL>(a, st);
+}
+
+}  // namespace
+
+int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
+                     int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
+                     int64_t grid_w, int radius, bool share, int64_t* out_ids, float* out_d, cudaStream_t st)
+{
+    if (Q == 0) return 0;
+    QueryScanArgs a{};
+    a.share = share ? 1 : 0;
+    a.xs = xs;
+    a.Y = Y;
+    a.offsets = offsets;
+    a.perm = perm;
+    a.probes = probes;
+    a.query_src = query_src;
+    a.Q = Q;
+    a.P_eff = P_eff;
+    a.grid_w = grid_w;
+    a.d = d;
+    a.d_pad = d_pad;
+    a.k = k;
+    a.radius = radius;
+    a.NC = NC;
+    a.out_ids = out_ids;
+    a.out_d = out_d;
+    return query_src ? launch_d<true>(a, st) : launch_d<false>(a, st);
+}
+
+}  // namespace osann

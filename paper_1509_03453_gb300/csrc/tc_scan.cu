@@ -37,15 +37,17 @@ constexpr int PREP_SMALL_Q = 1024;
 // 64 rows halve this kernel's time and cost the screen and rerank less than
 // that); in a small batch every item runs at once on the first bound, which
 // must then be tighter (up to 1024 rows, a few cones): about 2^18 / Q rows,
-// clamped.  For k > 4 the bound is the k-th best of the seed, which a short
-// seed leaves loose: 1024 rows (on the thin-cone descriptor search, k = 10,
-// Q = 10^4, this cut the survivors from 9.7 to 2.0 million and removed the
-// overflow rescans: 26.2 -> 21.5 ms).
-int tc_seed_rows(int64_t Q, int k)
+// clamped.  For k > 4 the bound is the k-th best of the seed, and items of few
+// rows hardly tighten it: k M / 64 rows, M the query's candidates, so that a few
+// hundred of them stay below it, 64 to 1024 rows.  (1024 rows always, on
+// two bases of 96 cones of 25 rows, k = 5, Q = 3001, took 650 us per basis beside
+// a 280 us screen; on the thin-cone descriptor search, M = 72000, k = 10, 64 rows
+// left 9.7 instead of 2.0 million survivors and overflowed lists.)
+int tc_seed_rows(int64_t Q, int k, double M)
 {
-    if (k > 4) return 1024;
-    const int64_t r = Q > 0 ? (int64_t(262144) + Q - 1) / Q : 1024;
-    return int(r < 64 ? 64 : (r > 1024 ? 1024 : r));
+    const double r = k > 4 ? k * M / 64.0 : 0.0, q = Q > 0 ? (262144.0 + double(Q) - 1.0) / double(Q) : 1024.0;
+    const double n = r > q ? r : q;
+    return n < 64.0 ? 64 : (n > 1024.0 ? 1024 : int(n));
 }
 
 struct PrepArgs {
@@ -636,7 +638,7 @@ int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, 
     a.grid_w = grid_w;
     a.radius = radius;
     a.cap = cap;
-    a.seed_rows = seed_rows > 0 ? seed_rows : tc_seed_rows(Q, k);
+    a.seed_rows = seed_rows;
     a.Y16 = static_cast<uint16_t*>(Y16);
     a.qstat = qstat;
     a.Ubits = Ubits;
