@@ -636,6 +636,19 @@ static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
 // Rows of an occupied cone, on average, below which a query's warps take cones each
 // in the per-query scan instead of sharing every cone's rows.
 constexpr double THIN_ROWS = 24.0;
+// The per-query scan of the probed cones (sel: of the listed queries).  A shortened
+// wait budget, a test hook, takes the staged form, whose waits it is for.
+static int exact_scan(const osann_index* ix, const float* Y, int64_t Q, const uint32_t* probes, int64_t P_eff, int k,
+                      const int64_t* src, int64_t grid_w, int radius, const uint32_t* sel, int64_t* ids, float* dists,
+                      cudaStream_t st)
+{
+    if (plain_wait_budget_set())
+        return launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff, uint32_t(ix->NC),
+                                 k, src, grid_w, radius, sel, ix->num_sms, ids, dists, ix->status, st);
+    return launch_query_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff, uint32_t(ix->NC), k,
+                             src, grid_w, radius, rows_per_cone(ix) >= THIN_ROWS, sel, ix->num_sms, ids, dists, st);
+}
+
 // Probed cones looked up for the dense screen's seed (it stops at its rows).
 constexpr int64_t DENSE_SEED_CONES = 512;
 
@@ -1475,10 +1488,8 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                       ix->diag, reinterpret_cast<uint32_t*>(w + L.ovf), ids, dists, st);
                 // queries whose survivor list overflowed: exact scan of their probed cones
                 if (!rc)
-                    rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff,
-                                           uint32_t(ix->NC), k, src, grid_w, radius,
-                                           reinterpret_cast<const uint32_t*>(w + L.ovf), ix->num_sms, ids, dists,
-                                           ix->status, st);
+                    rc = exact_scan(ix, Y, Q, probes, P_eff, k, src, grid_w, radius,
+                                    reinterpret_cast<const uint32_t*>(w + L.ovf), ids, dists, st);
             }
         } else if (!rc) {
             {
@@ -1513,21 +1524,12 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         if (!rc) {
             if (P_front < P_eff) rc = query_front(ix, Y, Q, P_eff, 1, L, w, false, k, st, left);
             if (!rc)
-                rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff,
-                                       uint32_t(ix->NC), k, src, grid_w, radius, left, ix->num_sms, ids, dists,
-                                       ix->status, st);
+                rc = exact_scan(ix, Y, Q, probes, P_eff, k, src, grid_w, radius, left, ids, dists, st);
         }
     } else if (!rc) {
         StageScope s(OSANN_STAGE_PLAIN_SCAN, st);
-        // (a shortened wait budget, a test hook, is the staged scan's)
-        if (!plain_wait_budget_set())
-            rc = launch_query_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q,
-                                   reinterpret_cast<uint32_t*>(w + L.probes), P_eff, uint32_t(ix->NC), k, src, grid_w,
-                                   radius, rows_per_cone(ix) >= THIN_ROWS, ids, dists, st);
-        else
-            rc = launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q,
-                               reinterpret_cast<uint32_t*>(w + L.probes), P_eff, uint32_t(ix->NC), k, src, grid_w,
-                               radius, nullptr, ix->num_sms, ids, dists, ix->status, st);
+        rc = exact_scan(ix, Y, Q, reinterpret_cast<uint32_t*>(w + L.probes), P_eff, k, src, grid_w, radius, nullptr, ids,
+                        dists, st);
     }
     if (owned) dev_free(owned, L.total, st);
     return rc;

@@ -149,6 +149,37 @@ __device__ __forceinline__ void topk_remove(uint64_t (&list)[KMAX], int k, uint6
         if (j >= KMAX - k && list[j] == v) list[j] = EMPTY_DI;
 }
 
+// The same over a warp, k <= 32: entry j in lane j, ascending; thr is the k-th.  An
+// insertion is a ballot and a shift whatever k (a register list of 32 costs 32 steps
+// in every lane that inserts, and a warp's lanes insert at different times).
+struct WarpTopk {
+    uint64_t list = EMPTY_DI, thr = EMPTY_DI;
+    // v: the same in all lanes, all of them here
+    __device__ __forceinline__ void insert(uint64_t v, int k, int lane)
+    {
+        if (v >= thr) return;
+        const int pos = __popc(__ballot_sync(0xffffffffu, list < v));
+        const uint32_t lo = __shfl_up_sync(0xffffffffu, uint32_t(list), 1);
+        const uint32_t hi = __shfl_up_sync(0xffffffffu, uint32_t(list >> 32), 1);
+        if (lane == pos) list = v;
+        else if (lane > pos) list = (uint64_t(hi) << 32) | lo;
+        thr = (uint64_t(__shfl_sync(0xffffffffu, uint32_t(list >> 32), k - 1)) << 32) |
+              __shfl_sync(0xffffffffu, uint32_t(list), k - 1);
+    }
+    // every lane's v where ok, all lanes here
+    __device__ __forceinline__ void offer(bool ok, uint64_t v, int k, int lane)
+    {
+        unsigned m = __ballot_sync(0xffffffffu, ok && v < thr);
+        while (m) {
+            const int s = __ffs(int(m)) - 1;
+            m &= m - 1u;
+            insert((uint64_t(__shfl_sync(0xffffffffu, uint32_t(v >> 32), s)) << 32) |
+                       __shfl_sync(0xffffffffu, uint32_t(v), s),
+                   k, lane);
+        }
+    }
+};
+
 // Canonical fp32 squared distance.  The padded vector is cut into float4
 // pieces j = 0 .. d_pad/4-1; piece j contributes
 //     c_j = fma(t3,t3, fma(t2,t2, fma(t1,t1, t0*t0))),  t = x - y,

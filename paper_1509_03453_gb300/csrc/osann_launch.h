@@ -112,11 +112,13 @@ int launch_plain_scan(const float* xs, const uint32_t* offsets, const uint32_t* 
                       int64_t* out_ids, float* out_d, uint32_t* status, cudaStream_t st);
 // qlist (nullable): device list [count, q_0, ...] of the queries to scan
 
-// scan_query.cu: the per-query scan, one to sixteen warps per query.  share: fat
-// cones (a query's warps share their rows instead of taking cones each)
+// scan_query.cu: the per-query scan, one to 128 warps per query.  fat: fat cones (a
+// query's warps share their rows instead of taking cones each); sel (nullable): device
+// list [count, q_0, ...] of the queries to scan
 int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
                      int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
-                     int64_t grid_w, int radius, bool share, int64_t* out_ids, float* out_d, cudaStream_t st);
+                     int64_t grid_w, int radius, bool fat, const uint32_t* sel, int num_sms, int64_t* out_ids,
+                     float* out_d, cudaStream_t st);
 
 // scan_batched.cu
 struct BatchedBuffers {

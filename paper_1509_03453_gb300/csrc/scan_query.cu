@@ -1,7 +1,7 @@
 // Per-query candidate scan (Algorithm 1 with one basis): for each query, the exact
 // squared Euclidean distance (Eq. 1, fp32) to every point of every probed cone, the
-// k nearest by (distance, id).  One to sixteen warps per query, rows straight from
-// global memory.
+// k nearest by (distance, id).  One warp to eight blocks of sixteen per query, rows
+// straight from global memory.
 //
 // The staged scan (scan_plain.cu) streams a query's rows through shared memory, one
 // bulk copy per cone; its producer, its per-row shuffles and its single-lane lists
@@ -19,6 +19,8 @@
 // matches excluded, 3400 -> 601; cones of 500 rows: d = 32, 10^4 queries, 16 cones,
 // k = 10 4880 -> 841, k = 1 1563 -> 828; 20 queries, 20 cones 77 -> 27; d = 64, 300
 // queries, 20 cones, k = 4 192 -> 132; d = 128, 3000 queries 4180 -> 2050.
+#include <cooperative_groups.h>
+
 #include "osann_device.cuh"
 #include "osann_launch.h"
 
@@ -34,14 +36,19 @@ struct QueryScanArgs {
     const int64_t* query_src;
     int64_t Q, P_eff, grid_w;
     int d, d_pad, k, radius;
-    int share;  // W > 1: the warps share every 32 cones' rows, instead of taking 32 cones each
+    const uint32_t* sel;  // LISTED: [count, q_0, ...]
+    int team;     // warps that share the rows of 32 cones: a power of two that divides the query's warps
+    int cluster;  // blocks per query
     uint32_t NC;
     int64_t* out_ids;
     float* out_d;
 };
 
-// TPR lanes per row, F float4 pieces each; W warps per query.
-template <int TPR, int F, bool EXCL, int W>
+// TPR lanes per row, F float4 pieces each; W warps per block.  W = 1: a query per
+// warp, four per block; otherwise a cluster of a.cluster blocks per query, in teams
+// of a.team warps: a team takes 32 cones at a time, its warps those cones' rows by turns.
+// LISTED: the clusters take the queries of a list made on the device by turns.
+template <int TPR, int F, bool EXCL, int W, bool LISTED = false>
 __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const QueryScanArgs a)
 {
     constexpr int CPP = 32 / TPR;     // rows per load instruction
@@ -49,9 +56,14 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
     constexpr int RL = B > 32 ? 2 : 1;  // batch rows looked up per lane
     constexpr int NV = TPR >= U ? 1 : U / TPR;  // row sums a lane ends with
     const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, wq = W == 1 ? 0 : int(threadIdx.x >> 5);
-    const int64_t q = W == 1 ? int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5) : int64_t(blockIdx.x);
-    if (q >= a.Q) return;  // W > 1: never
+    const int lane = threadIdx.x & 31, wb = W == 1 ? 0 : int(threadIdx.x >> 5);
+    const unsigned blocks = W == 1 ? 1u : unsigned(a.cluster), rank = W == 1 ? 0u : blockIdx.x % blocks;
+    const int wq = int(rank) * W + wb;  // warp of the query
+    const int64_t first =
+        W == 1 ? int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5) : int64_t(blockIdx.x / blocks);
+    const int64_t count = LISTED ? int64_t(a.sel[0]) : a.Q;
+    for (int64_t at = first; at < count; at += LISTED ? int64_t(gridDim.x / blocks) : count) {
+    const int64_t q = LISTED ? int64_t(a.sel[1 + at]) : at;
     const int g = lane / TPR, sub = lane % TPR;
     float4 qv[F];
     {
@@ -66,17 +78,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
         }
     }
     const int64_t src = EXCL ? a.query_src[q] : -1;
-    // the best found, ascending over the lanes (k <= 32); thr: the k-th
-    uint64_t list = EMPTY_DI, thr = EMPTY_DI;
-    auto insert = [&](uint64_t v) {  // v uniform
-        if (v >= thr) return;
-        const int pos = __popc(__ballot_sync(FULL, list < v));
-        const uint32_t lo = __shfl_up_sync(FULL, uint32_t(list), 1), hi = __shfl_up_sync(FULL, uint32_t(list >> 32), 1);
-        if (lane == pos) list = v;
-        else if (lane > pos) list = (uint64_t(hi) << 32) | lo;
-        thr = (uint64_t(__shfl_sync(FULL, uint32_t(list >> 32), a.k - 1)) << 32) |
-              __shfl_sync(FULL, uint32_t(list), a.k - 1);
-    };
+    WarpTopk best;
     // the row index, inside its load group, whose sum this lane ends with (its
     // lowest for TPR < U), from the halving steps below: the top bit first
     int u0 = 0;
@@ -96,12 +98,12 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
             }
         }
     };
-    const bool share = W > 1 && a.share;
-    const int64_t pstep = share ? 32 : 32 * W;
-    const uint32_t tbeg = share ? uint32_t(wq * B) : 0u, tstep = share ? uint32_t(W * B) : uint32_t(B);
+    const int team = W == 1 ? 1 : a.team;
+    const int64_t pbeg = W == 1 ? 0 : 32 * (wq / team), pstep = W == 1 ? 32 : 32 * (int(blocks) * W / team);
+    const uint32_t tbeg = W == 1 ? 0u : uint32_t(wq % team * B), tstep = uint32_t(team * B);
     uint32_t st, sz;
-    cone((share ? 0 : 32 * wq) + lane, st, sz);
-    for (int64_t p0 = share ? 0 : 32 * wq; p0 < a.P_eff; p0 += pstep) {
+    cone(pbeg + lane, st, sz);
+    for (int64_t p0 = pbeg; p0 < a.P_eff; p0 += pstep) {
         uint32_t st1, sz1;
         cone(p0 + pstep + lane, st1, sz1);  // the next 32 cones, behind these ones' rows
         uint32_t incl = sz;
@@ -166,7 +168,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
                 const uint32_t lo = __shfl_sync(FULL, id[0], e & 31);
                 const uint32_t hi = RL == 2 ? __shfl_sync(FULL, id[RL - 1], e & 31) : 0u;
                 const uint32_t cid = RL == 2 && e >= 32 ? hi : lo;
-                bool ok = primary && t0 + uint32_t(e) < total && v[i] <= di_dist(thr);
+                bool ok = primary && t0 + uint32_t(e) < total && v[i] <= di_dist(best.thr);
                 if (EXCL && ok && src >= 0) {
                     int64_t dr = int64_t(cid) / a.grid_w - src / a.grid_w;
                     int64_t dc = int64_t(cid) % a.grid_w - src % a.grid_w;
@@ -178,7 +180,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
                 while (m) {
                     const int s = __ffs(int(m)) - 1;
                     m &= m - 1u;
-                    insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)));
+                    best.insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)), a.k, lane);
                 }
             }
         }
@@ -187,53 +189,134 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
     }
     if (W > 1) {
         __shared__ uint64_t sh[W * 32];
-        if (lane < a.k) sh[wq * 32 + lane] = list;
+        if (lane < a.k) sh[wb * 32 + lane] = best.list;
         __syncthreads();
-        if (wq != 0) return;
-        for (int w = 1; w < W; ++w)
-            for (int j = 0; j < a.k; ++j) insert(sh[w * 32 + j]);
+        if (wb == 0)
+            for (int w = 1; w < W; ++w)
+                for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
+        if (blocks > 1) {
+            // the blocks' lists, through the first one's shared memory
+            namespace cg = cooperative_groups;
+            cg::cluster_group cl = cg::this_cluster();
+            if (wb == 0 && lane < a.k) sh[lane] = best.list;
+            cl.sync();
+            if (rank == 0 && wb == 0)
+                for (unsigned r = 1; r < blocks; ++r) {
+                    const uint64_t* rs = cl.map_shared_rank(sh, r);
+                    best.offer(lane < a.k, lane < a.k ? rs[lane] : EMPTY_DI, a.k, lane);
+                }
+            cl.sync();  // no block leaves, or goes on, while its list is read
+        } else if (LISTED) {
+            __syncthreads();
+        }
     }
-    if (lane < a.k) {
-        const uint32_t id = di_id(list);
+    if (rank == 0 && wb == 0 && lane < a.k) {
+        const uint32_t id = di_id(best.list);
         a.out_ids[q * a.k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
-        a.out_d[q * a.k + lane] = di_dist(list);
+        a.out_d[q * a.k + lane] = di_dist(best.list);
+    }
     }
 }
 
-template <int TPR, int F, bool EXCL>
-int launch_w(const QueryScanArgs& a, cudaStream_t st)
+// thin cones: a team per 32 probes, as far as the warps go; fat ones: all warps
+int64_t team_of(int64_t P, int64_t warps, bool fat)
 {
-    // enough warps for the chip (some 3600 resident): over thin cones one per query
-    // from 2048 queries up and four from 256; over fat ones, whose queries have more
-    // rows, from 4096 and 608 (1000 queries, 20 cones of 504 rows: four 157, sixteen
-    // 180 us; 300 queries: 139 and 49)
-    if (a.Q >= (a.share ? 4096 : 2048)) query_scan_kernel<TPR, F, EXCL, 1><<<unsigned((a.Q + 3) / 4), 128, 0, st>>>(a);
-    else if (a.Q >= (a.share ? 608 : 256)) query_scan_kernel<TPR, F, EXCL, 4><<<unsigned(a.Q), 128, 0, st>>>(a);
-    else query_scan_kernel<TPR, F, EXCL, 16><<<unsigned(a.Q), 512, 0, st>>>(a);
-    return count_launch();
+    int64_t team = warps;
+    if (!fat)
+        while (team > 1 && warps / team < (P + 31) / 32) team /= 2;
+    return team;
+}
+// thin cones: waves of blocks (32 warps per SM) times a block's rounds of 32 probes
+double rounds(int64_t Q, int64_t P, int64_t W, int num_sms)
+{
+    const int64_t slots = int64_t(num_sms) * 32 / W, team = team_of(P, W, false), teams = W / team;
+    return double((Q + slots - 1) / slots) * double(((P + 31) / 32 + teams - 1) / teams) / double(team);
+}
+
+template <int TPR, int F, bool EXCL, int W, bool LISTED>
+int launch_team(QueryScanArgs a, bool fat, int cluster, int64_t clusters, cudaStream_t st)
+{
+    a.team = int(team_of(a.P_eff, int64_t(W) * cluster, fat));
+    a.cluster = cluster;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(clusters * cluster));
+    cfg.blockDim = dim3(32 * W);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = unsigned(cluster);
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, query_scan_kernel<TPR, F, EXCL, W, LISTED>, a);
+    const int rc = count_launch();
+    if (e != cudaSuccess && !rc) {
+        set_error("per-query scan: launch failed (%s)", cudaGetErrorString(e));
+        return -5;
+    }
+    return rc;
+}
+
+// Enough warps for the chip (some 3600 resident), and more, shorter blocks where a
+// last wave of long ones would be nearly empty.  Measured (us):
+//   thin cones, 1602 probes of 4.5 rows: W = 1 / 4 / 8 / 16 at 700 queries 934 / 383 /
+//   394 / 310, 1268: 955 / 681 / 574 / 488, 2500: 1034 / 1026 / 942 / 846, 5000: 1332 /
+//   1713 / 1678 / 1563; 128 probes of 6 rows, 700: 230 / 126 / 130 / 128, 1500: 242 /
+//   197 / 179 / 190, 2500: 261 / 266 / 263 / 295;
+//   patches (fat, uneven), 20 probes, 500: 184 / 91 / 75 / 75, 1000: 169 / 87 / 78 /
+//   87, 3000: 227 / 124 / 129 / 171, 8000 (40 probes): 325 / 336 / 358 / 476.
+// Over thin cones the number of warps whose blocks need the fewest rounds in all,
+// which orders all of these but those bound by DRAM (795 queries, 260 probes: 165
+// with sixteen warps, 141 with four; 550 probes: 348 with eight, 301 with four).
+// With sixteen, as many blocks, up to eight, as give every SM two (one / two / four /
+// eight blocks: 24 queries, 198 cones of 17 rows of d = 100, 91 / 58 / 46 / 42; 6
+// queries, 7000 thin cones, 210 / 132 / 97 / 72; 135 queries over patches 76 / 56 / 60
+// / 93; 200 queries 48 / 56 / 60 / 83).  A list of queries takes eight: it is as often
+// one query as all.
+template <int TPR, int F, bool EXCL>
+int launch_w(const QueryScanArgs& a, bool fat, int num_sms, cudaStream_t st)
+{
+    if (a.sel) {
+        const int64_t clusters = 2 * int64_t(num_sms) / 8;
+        return launch_team<TPR, F, EXCL, 16, true>(a, fat, 8, clusters < 1 ? 1 : (clusters < a.Q ? clusters : a.Q), st);
+    }
+    if (a.Q >= (fat ? 6144 : (a.P_eff >= 256 ? 3600 : 2048))) {
+        query_scan_kernel<TPR, F, EXCL, 1><<<unsigned((a.Q + 3) / 4), 128, 0, st>>>(a);
+        return count_launch();
+    }
+    int w = fat && a.Q >= 2048 ? 4 : (fat && a.Q >= 608 ? 8 : 16);
+    if (!fat && a.Q >= 256)
+        for (const int v : {8, 4})
+            if (rounds(a.Q, a.P_eff, v, num_sms) <= rounds(a.Q, a.P_eff, w, num_sms)) w = v;
+    if (w == 4) return launch_team<TPR, F, EXCL, 4, false>(a, fat, 1, a.Q, st);
+    if (w == 8) return launch_team<TPR, F, EXCL, 8, false>(a, fat, 1, a.Q, st);
+    int c = 8;
+    while (c > 1 && a.Q * c > 2 * int64_t(num_sms)) c /= 2;
+    return launch_team<TPR, F, EXCL, 16, false>(a, fat, c, a.Q, st);
 }
 
 template <bool EXCL>
-int launch_d(const QueryScanArgs& a, cudaStream_t st)
+int launch_d(const QueryScanArgs& a, bool fat, int num_sms, cudaStream_t st)
 {
     switch (a.d_pad) {
-    case 16: return launch_w<4, 1, EXCL>(a, st);
-    case 32: return launch_w<8, 1, EXCL>(a, st);
-    case 64: return launch_w<16, 1, EXCL>(a, st);
-    case 128: return launch_w<32, 1, EXCL>(a, st);
+    case 16: return launch_w<4, 1, EXCL>(a, fat, num_sms, st);
+    case 32: return launch_w<8, 1, EXCL>(a, fat, num_sms, st);
+    case 64: return launch_w<16, 1, EXCL>(a, fat, num_sms, st);
+    case 128: return launch_w<32, 1, EXCL>(a, fat, num_sms, st);
     }
-    return launch_w<32, 2, EXCL>(a, st);
+    return launch_w<32, 2, EXCL>(a, fat, num_sms, st);
 }
 
 }  // namespace
 
 int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
                      int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
-                     int64_t grid_w, int radius, bool share, int64_t* out_ids, float* out_d, cudaStream_t st)
+                     int64_t grid_w, int radius, bool fat, const uint32_t* sel, int num_sms, int64_t* out_ids,
+                     float* out_d, cudaStream_t st)
 {
     if (Q == 0) return 0;
     QueryScanArgs a{};
-    a.share = share ? 1 : 0;
+    a.sel = sel;
     a.xs = xs;
     a.Y = Y;
     a.offsets = offsets;
@@ -250,7 +333,7 @@ int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* 
     a.NC = NC;
     a.out_ids = out_ids;
     a.out_d = out_d;
-    return query_src ? launch_d<true>(a, st) : launch_d<false>(a, st);
+    return query_src ? launch_d<true>(a, fat, num_sms, st) : launch_d<false>(a, fat, num_sms, st);
 }
 
 }  // namespace osann

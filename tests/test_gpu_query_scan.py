@@ -41,3 +41,47 @@ def test_query_scan_matches_batched(osann, d, L, Q):
             assert np.array_equal(to_np(a[1]).view(np.uint32), to_np(b[1]).view(np.uint32))
     assert idx.status() == 0
     idx.close()
+
+
+@pytest.mark.parametrize("L", [1, 2])
+@pytest.mark.parametrize("Q", [2, 38, 39, 76, 77, 152, 153])
+def test_query_scan_clusters_and_teams(osann, L, Q):
+    """One to eight blocks per query (more than two per SM never), and budgets that
+    leave teams of 1, 2, ... all of a query's warps per 32 probes."""
+    rng = np.random.default_rng(L + Q)
+    N, d = 6007, 48
+    X = rng.standard_normal((N, d)).astype(np.float32)
+    Y = rng.standard_normal((Q, d)).astype(np.float32)
+    idx = osann.Index(to_dev(X), L)
+    Yd = to_dev(Y)
+    for P, k in ((5, 4), (64, 32), (65, 1), (515, 10), (4512, 17)):
+        a = idx.search(Yd, P, k, path="plain")
+        b = idx.search(Yd, P, k, path="batched")
+        assert np.array_equal(to_np(a[0]), to_np(b[0]))
+        assert np.array_equal(to_np(a[1]).view(np.uint32), to_np(b[1]).view(np.uint32))
+    assert idx.status() == 0
+    idx.close()
+
+
+@pytest.mark.parametrize("L", [1, 2])
+@pytest.mark.parametrize("n", [1, 37, 39, 300])
+def test_overflowed_queries(osann, L, n):
+    """n of 500 queries whose survivor lists overflow (2000 equal rows at their
+    distance): the exact scan of the listed queries by clusters in turns."""
+    rng = np.random.default_rng(L + n)
+    d = 32
+    X = rng.standard_normal((20_000, d)).astype(np.float32)
+    X[5000:7000] = X[5000]
+    Y = rng.standard_normal((500, d)).astype(np.float32)
+    Y[::500 // n if n < 500 else 1][:n] = X[5000]
+    idx = osann.Index(to_dev(X), L)
+    Yd = to_dev(Y)
+    idx.screen_stats()
+    for P, k in ((60, 3), (60, 20), (idx.NC, 8)):
+        a = idx.search(Yd, P, k, path="fp16")
+        assert idx.screen_stats()["fallbacks"] >= n
+        b = idx.search(Yd, P, k, path="batched")
+        assert np.array_equal(to_np(a[0]), to_np(b[0]))
+        assert np.array_equal(to_np(a[1]).view(np.uint32), to_np(b[1]).view(np.uint32))
+    assert idx.status() == 0
+    idx.close()
