@@ -41,8 +41,9 @@ extern "C" {
 
 /* Search paths (same results, different schedules). */
 #define OSANN_PATH_AUTO 0    /* the 16-bit screen when enough queries share a cone (per
-                                occupied cone, as counted by a synchronous build), the
-                                fp32 tile scan for d > 128, else plain */
+                                occupied cone, as counted by a synchronous build), over
+                                every row where that is cheaper (thin cones, or k > 1 with
+                                many candidates), the fp32 tile scan for d > 128, else plain */
 #define OSANN_PATH_PLAIN 1   /* one or more warps per query scanning its cones */
 #define OSANN_PATH_BATCHED 2 /* cone-major work list, persistent fp32 tile scan */
 #define OSANN_PATH_BF16 3    /* cone-major work list, bf16 tensor-core screening with a
@@ -427,8 +428,7 @@ int64_t osann_launch_count(void);
 /* Test hook for failure detection (the paper has no counterpart): the clock
  * budget, in SM cycles, of the plain scan's waits for its staged copies
  * (OSANN_PATH_PLAIN, and the exact rescan of the tensor-core paths: staged
- * only while a budget is set).  A wait
- * that runs past it gives up: the kernel lets its copies in flight land
+ * only while a budget is set).  A wait that runs past it gives up: the kernel lets its copies in flight land
  * (under the full budget), writes what it found for the query at hand and
  * empty results (-1, +inf) for its other queries, and sets
  * OSANN_STATUS_TIMEOUT, which the next osann_status reports; the context

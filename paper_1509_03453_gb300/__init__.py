@@ -267,8 +267,8 @@ class Index:
         """Top-k by exact squared distance over the first min(P, N_C)
         probed cones.  Returns (ids int64 [Q,k], sqdists float32 [Q,k]).
         ``group``: queries per work-list item on the batched paths (0 =
-        default); ``layout``: the tensor-core screen's query tiles ("smem",
-        "tmem" or "default"); both change the speed, not the result.
+        default); it changes the speed, not the result.  ``layout`` ("smem",
+        "tmem" or "default") is accepted and changes neither.
         ``clusters`` (ROSANNA+ index): nearest clusters visited, P cones in
         each."""
         torch = _torch()

@@ -2,9 +2,9 @@
 //
 // Validation, device allocation (stream-ordered, through an optional
 // caller-installed allocator), per-device constant tables, workspace layout,
-// the index build and the two search schedules, and stage timing.  Every
-// step of the method runs in the kernels of keys.cu, buckets.cu, probes.cu,
-// scan_plain.cu and scan_batched.cu; this file only sequences them.
+// the index build and the search schedules, and stage timing.  Every step of
+// the method runs in the kernels of keys.cu, buckets.cu, probes.cu, scan_*.cu
+// and tc_*.cu; this file only sequences them.
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
@@ -562,14 +562,23 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
 // Whether screening every row beats the mode that would be taken otherwise.  All
 // in microseconds on this chip, from these measurements:
 //   dense screen: N / 128 row tiles per 128 queries, 64 cycles per 16 columns at
-//   about 0.8 of the tensor rate; 250 for the phases and updates;
-//   seed rows, read at random: 2.4 TB/s (2800 for 10^4 x 1024 rows of 512 bytes,
-//   28 for 4096 x 64 of 256);
+//   about 0.8 of the tensor rate; 60 and 40 per phase; seed rows, read at random, at
+//   2.4 TB/s (2800 for 10^4 x 1024 rows of 512 bytes, 28 for 4096 x 64 of 256); per
+//   query and phase 2.1 ns x k and 7 ps per survivor counted below.
 //   cone by cone, an item (a cone and up to 256 queries) costs its tiles, but at
 //   least DENSE_ITEM_CYCLES however few its rows (5200 measured at d = 128, cones
-//   of 6 rows, 3800 with cones of 25); its work list 10 ps per (query, probe), above
-//   12288 cones (global atomics) 45 ps (5400 for 1.2*10^8); seed and list side by side;
+//   of 6 rows, 3800 with cones of 25), and for full items up to 2.8 times that to
+//   keep k bounds; its work list 10 ps per (query, probe), above 12288 cones (global
+//   atomics) 45 ps (5400 for 1.2*10^8); seed and list side by side.
+//   For k > 4 an item's rows bound the k-th best no better than the seed does,
+//   so that about k M / seed rows survive (M the query's candidates), and past the
+//   list's capacity a query is scanned exactly, 4.5 TB/s: N = 2.5*10^6, d = 64, 1600
+//   cones, k = 10: 155 of 1269 queries (item by item 6.4 ms, dense 0.77), k = 32
+//   1242 (44.5, 1.16 ms).
 //   per-query scan: 6 TB/s of rows.
+// (Over 144 Gaussian searches, N = 4*10^5 .. 2.5*10^6, d = 32 .. 100, Q = 100 .. 4096,
+// P = 50 .. 1600, k = 2 .. 32: by this rule 0.73 of the time without it, the better of
+// both always 0.68.)
 // Only for the set key with a direct table and L <= 4, whose list positions the
 // dense screen recomputes for a survivor's cone.
 constexpr double DENSE_ITEM_CYCLES = 4000.0;
@@ -586,16 +595,19 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
     const double sm_us = ix->num_sms * 2000.0;  // SM cycles per microsecond of the chip
     const double row = 4.0 * ix->d_pad, seed_rate = 2.4e6;
     const double tile = 80.0 * double((ix->d + 15) / 16 + 1);
-    const double dense_us = double((ix->N + 127) / 128) * double((Q + 127) / 128) * tile / sm_us + 250.0 +
-                            double(Q) * 256.0 * row / seed_rate;
     const double probes = double(Q) * double(P_eff);
-    const double rows = rows_per_cone(ix);
+    const double rows = rows_per_cone(ix), M = rows * double(P_eff);
     // A phase holds eight times the rows before it, so it leaves about 8 k N / M
-    // survivors per query (M its candidates; fewer where the probed cones hold
-    // nearer rows than the others): past the list's capacity the exact scan would
-    // have the work.  (2240 by this count, 85 found, on the descriptor search; 8200
-    // and mostly overflows on a two-basis Gaussian one, 2950 us against 2080.)
-    if (8.0 * k * double(ix->N) > 2500.0 * rows * double(P_eff)) return false;
+    // survivors per query (fewer where the probed cones hold nearer rows than the
+    // others): past the list's capacity the exact scan would have the work.  (2240 by
+    // this count, 85 found, on the descriptor search; on Gaussian data none of 4096
+    // queries overflowed at 3200, 2 at 5200, a twelfth at 10300.)
+    const double found = 8.0 * k * double(ix->N) / M;
+    if (found > 3500.0) return false;
+    int phases = 1;
+    for (int64_t n = ix->N; n > 4096; n >>= 3) ++phases;
+    const double dense_us = double((ix->N + 127) / 128) * double((Q + 127) / 128) * tile / sm_us + 60.0 + 40.0 * phases +
+                            double(Q) * 256.0 * row / seed_rate + double(Q) * phases * (7e-6 * found + 2.1e-3 * k);
     double other;
     if (mode == MODE_PLAIN) {
         other = probes * rows * row / 6.0e6 + 20.0;
@@ -603,12 +615,17 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
         const double hit = probes < cones ? probes : cones;  // cones with work
         const double groups = std::ceil(probes / hit / 256.0);
         const double work = 2.0 * std::ceil(rows / 128.0) * tile;
-        const double seed = double(Q) * tc_seed_rows(Q, k, rows * double(P_eff)) * row / seed_rate;
+        const double full = probes / hit / groups / 128.0;  // a query tile's rows in use
+        const double bounds = k <= 1 ? 1.0 : (k <= 2 ? 1.2 : (k <= 4 ? 2.4 : 2.8));
+        const double seeds = tc_seed_rows(Q, k, M);
+        const double seed = double(Q) * seeds * row / seed_rate;
         const double list = ix->NC > 12288 ? 150.0 + probes * 45e-6 : 40.0 + probes * 10e-6;
-        other = hit * groups * (work > DENSE_ITEM_CYCLES ? work : DENSE_ITEM_CYCLES) / sm_us +
-                (seed > list ? seed : list) + 60.0;
+        const double over = k > 4 ? (k * M / seeds - TC_SURV_CAP) / 15000.0 : 0.0;  // queries that overflow
+        other = hit * groups * (work > DENSE_ITEM_CYCLES ? work : DENSE_ITEM_CYCLES) / sm_us *
+                    (1.0 + (bounds - 1.0) * (full < 1.0 ? full : 1.0)) +
+                (seed > list ? seed : list) + 60.0 + double(Q) * M * row / 4.5e6 * (over < 0.0 ? 0.0 : (over < 1.0 ? over : 1.0));
     }
-    return dense_us < 0.8 * other;
+    return dense_us < 0.85 * other;
 }
 
 static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path)
@@ -1478,7 +1495,8 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                     radius, b, reinterpret_cast<uint32_t*>(w + L.ubits),
                                     reinterpret_cast<uint32_t*>(w + L.scnt), reinterpret_cast<uint32_t*>(w + L.surv),
                                     TC_SURV_CAP, ix->status, ix->diag, ix->xs, Y, P_eff, ix->d, ix->d_pad, k,
-                                    ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms);
+                                    ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms,
+                                    tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)));
             }
             if (!rc) {
                 StageScope s(OSANN_STAGE_TC_RERANK, st);

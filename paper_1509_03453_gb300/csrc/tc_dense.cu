@@ -194,9 +194,13 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
         for (int r = lane; r < a.m.dk; r += 32) inv[a.m.qorder[q * a.m.dk + r]] = uint8_t(r);
         __syncwarp();
     }
+    constexpr bool WARP_LIST = KMAX >= 16;  // k above 4: one list per warp, over its lanes
+    WarpTopk wl;
     uint64_t list[KMAX];
     topk_init<KMAX>(list, a.k);
-    if (!a.first && wq == 0) {
+    if (WARP_LIST) {
+        if (!a.first && wq == 0) wl.offer(lane < a.k, lane < a.k ? a.best[q * a.k + lane] : EMPTY_DI, a.k, lane);
+    } else if (!a.first && wq == 0) {
         for (int j = lane; j < a.k; j += 32) {
             const uint64_t v = a.best[q * a.k + j];
             if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
@@ -234,10 +238,10 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
 #pragma unroll
             for (int u = 0; u < DENSE_U; ++u) {
                 const float dist = lane_tree(sq4(xv[u], qv), n4);
-                if (sub == 0 && at[u] < m) {
-                    const uint64_t v = pack_di(dist, ids[at[u]]);
-                    if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
-                }
+                const bool is = sub == 0 && at[u] < m;
+                const uint64_t v = pack_di(dist, is ? ids[at[u]] : 0u);
+                if (WARP_LIST) wl.offer(is, v, a.k, lane);
+                else if (is && v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
             }
         }
         __syncwarp();
@@ -245,7 +249,9 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
     if (W > 1) {
         // the warps' k best, gathered for the first one
         __shared__ uint64_t best_sh[W > 1 ? W * KMAX : 1];
-        for (int j = 0; j < a.k; ++j) {
+        if (WARP_LIST) {
+            if (lane < a.k) best_sh[wq * KMAX + lane] = wl.list;
+        } else for (int j = 0; j < a.k; ++j) {
             const uint64_t head = topk_head<KMAX>(list, a.k);
             const uint64_t b = warp_min_u64(head);
             if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
@@ -254,27 +260,34 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
         __syncthreads();
         if (wq != 0) return;
         topk_init<KMAX>(list, a.k);
-        for (int i = lane; i < W * a.k; i += 32) {
+        if (WARP_LIST) {
+            for (int w = 1; w < W; ++w)
+                wl.offer(lane < a.k, lane < a.k ? best_sh[w * KMAX + lane] : EMPTY_DI, a.k, lane);
+        } else for (int i = lane; i < W * a.k; i += 32) {
             const uint64_t v = best_sh[(i / a.k) * KMAX + i % a.k];
             if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
         }
     }
     if (LC > 0 && lane == 0) atomicAdd(a.diag, (unsigned long long)n);
     float kth = INFINITY;
-    for (int j = 0; j < a.k; ++j) {
+    auto put = [&](int j, uint64_t b) {
+        if (a.last) {
+            const uint32_t id = di_id(b);
+            a.out_ids[q * a.k + j] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
+            a.out_d[q * a.k + j] = di_dist(b);
+        } else {
+            a.best[q * a.k + j] = b;
+        }
+    };
+    if (WARP_LIST) {
+        if (lane < a.k) put(lane, wl.list);
+        kth = di_dist(wl.thr);
+    } else for (int j = 0; j < a.k; ++j) {
         const uint64_t head = topk_head<KMAX>(list, a.k);
         const uint64_t b = warp_min_u64(head);
         if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
         kth = di_dist(b);
-        if (lane == 0) {
-            if (a.last) {
-                const uint32_t id = di_id(b);
-                a.out_ids[q * a.k + j] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
-                a.out_d[q * a.k + j] = kth;
-            } else {
-                a.best[q * a.k + j] = b;
-            }
-        }
+        if (lane == 0) put(j, b);
     }
     if (lane == 0 && !a.last) {
         // the canonical fp32 distance is within 6.6e-7 relative of the exact one
@@ -411,7 +424,8 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
         if (dn.n_items > 0) {
             rc = launch_tc_scan(1, ix.maps, ix.perm, ix.rowstat, w + L.yb, reinterpret_cast<float4*>(w + L.qstat), ix.tcs,
                                 nullptr, 0, 0, b, Ubits, scnt, surv, DENSE_SURV_CAP, ix.status, ix.diag, ix.xs, Y, 1, ix.d,
-                                ix.d_pad, 1, ix.cdot2, ix.Bn, ix.cabs, debug, st, num_sms, &dn);
+                                ix.d_pad, 1, ix.cdot2, ix.Bn, ix.cabs, debug, st, num_sms,
+                                int(seed), &dn);
             if (rc) return rc;
         }
         u.first = j == 0;

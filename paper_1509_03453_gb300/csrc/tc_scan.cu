@@ -30,6 +30,7 @@ namespace osann {
 constexpr int TC_SEED_ILP = 8;  // row groups loaded per iteration
 constexpr int PREP_SMALL = 8;   // warps per query of a small batch
 constexpr int PREP_SMALL_Q = 1024;
+constexpr int PREP_WARP_LIST = 16;  // k above 4: one list per warp, over its lanes
 
 // Rows scanned exactly for a query's initial bound.  A large batch keeps
 // tightening its bounds as items finish, so a short seed suffices (64 rows
@@ -129,6 +130,8 @@ __global__ void __launch_bounds__(128)
         qv[f].w = c + 3 < d ? y[c + 3] : 0.f;
     }
     const int64_t src = a.query_src ? a.query_src[q] : -1;
+    constexpr bool WARP_LIST = KMAX >= PREP_WARP_LIST;
+    WarpTopk wl;
     uint64_t list[KMAX];
     topk_init<KMAX>(list, k);
     int scanned = 0;
@@ -163,17 +166,19 @@ __global__ void __launch_bounds__(128)
                     dc = dc < 0 ? -dc : dc;
                     usable = (dr > dc ? dr : dc) > radius;
                 }
-                if (sub == 0 && usable) {
-                    const uint64_t v = pack_di(dist, rr[u]);
-                    if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
-                }
+                const uint64_t v = pack_di(dist, rr[u]);
+                if (WARP_LIST) wl.offer(sub == 0 && usable, v, k, lane);
+                else if (sub == 0 && usable && v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
             }
             scanned += TC_SEED_ILP * CPP;
         }
     }
     // k-th smallest over the warp: k rounds of warp minimum over the lists
     float U = INFINITY;
-    {
+    if (WARP_LIST) {
+        // the canonical fp32 distance is within 6.6e-7 relative of the exact one
+        if (wl.thr != EMPTY_DI) U = di_dist(wl.thr) * (1.0f + 2e-6f) + 1e-30f;
+    } else {
         float kth = INFINITY;
         int found = 0;
         for (int j = 0; j < k; ++j) {
@@ -224,6 +229,8 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
         qv[f].w = c + 3 < a.d ? y[c + 3] : 0.f;
     }
     const int64_t src = a.query_src ? a.query_src[q] : -1;
+    constexpr bool WARP_LIST = KMAX >= PREP_WARP_LIST;
+    WarpTopk wl;
     uint64_t list[KMAX];
     topk_init<KMAX>(list, a.k);
     // the rows t0 + u * CPP + g (u < TC_SEED_ILP) below `end`, row_of(t) -> row
@@ -258,10 +265,9 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
                 dc = dc < 0 ? -dc : dc;
                 usable = (dr > dc ? dr : dc) > a.radius;
             }
-            if (sub == 0 && usable) {
-                const uint64_t v = pack_di(dist, rr[u]);
-                if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
-            }
+            const uint64_t v = pack_di(dist, rr[u]);
+            if (WARP_LIST) wl.offer(sub == 0 && usable, v, a.k, lane);
+            else if (sub == 0 && usable && v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
         }
     };
     const int step = WPQ * TC_SEED_ILP * CPP;
@@ -317,7 +323,16 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
     // warps' k best, gathered in shared memory
     __shared__ uint64_t best_sh[WPQ * KMAX];
     float U = INFINITY;
-    {
+    if (WARP_LIST) {
+        best_sh[wq * KMAX + lane % KMAX] = EMPTY_DI;
+        __syncwarp();
+        if (lane < a.k) best_sh[wq * KMAX + lane] = wl.list;
+        __syncthreads();
+        if (wq != 0) return;
+        for (int w = 1; w < WPQ; ++w)
+            wl.offer(lane < a.k, best_sh[w * KMAX + lane % KMAX], a.k, lane);
+        if (wl.thr != EMPTY_DI) U = di_dist(wl.thr) * (1.0f + 2e-6f) + 1e-30f;
+    } else {
         float kth = INFINITY;
         int found = 0;
         auto rounds = [&](uint64_t* keep) {
@@ -502,30 +517,34 @@ __global__ void __launch_bounds__(128) tc_rerank_kernel(const float* __restrict_
         }
     }
     const int64_t src = EXCL ? query_src[q] : -1;
+    constexpr bool WARP_LIST = KMAX >= PREP_WARP_LIST;
+    WarpTopk wl;
     uint64_t list[KMAX];
     topk_init<KMAX>(list, k);
     // the candidate's canonical distance from its row chunk xv (this lane's F
-    // float4 of the row), then the top-k update
-    auto consider = [&](uint32_t row, bool valid, const float4 (&xv)[F]) {
+    // float4 of the row)
+    auto distance = [&](const float4 (&xv)[F]) {
         float cpart[F];
 #pragma unroll
         for (int f = 0; f < F; ++f) cpart[f] = sq4(xv[f], qv[f]);
-        const float dist = lane_tree(pair_tree<F>(cpart), TPR);
-        if (valid && sub == 0) {
-            const uint32_t id = __ldg(perm + row);
-            if (EXCL && src >= 0) {
-                const int64_t dr = int64_t(id) / grid_w - src / grid_w;
-                const int64_t dc = int64_t(id) % grid_w - src % grid_w;
-                const int64_t adr = dr < 0 ? -dr : dr, adc = dc < 0 ? -dc : dc;
-                if ((adr > adc ? adr : adc) <= radius) return;
-            }
-            const uint64_t v = pack_di(dist, id);
-            if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
+        return lane_tree(pair_tree<F>(cpart), TPR);
+    };
+    // the top-k update
+    auto consider = [&](uint32_t id, bool valid, float dist) {
+        bool ok = valid && sub == 0;
+        if (EXCL && ok && src >= 0) {
+            const int64_t dr = int64_t(id) / grid_w - src / grid_w;
+            const int64_t dc = int64_t(id) % grid_w - src % grid_w;
+            const int64_t adr = dr < 0 ? -dr : dr, adc = dc < 0 ? -dc : dc;
+            ok = (adr > adc ? adr : adc) > radius;
         }
+        const uint64_t v = pack_di(dist, id);
+        if (WARP_LIST) wl.offer(ok, v, k, lane);
+        else if (ok && v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
     };
     const uint32_t n = surv_cnt[q];
     if (n <= uint32_t(cap)) {
-        // RR_U passes at a time: their survivor ids, then their rows, are all
+        // RR_U passes at a time: their survivor rows, then these rows and ids, are all
         // in flight before the first distance
         for (uint32_t b0 = 0; b0 < n; b0 += RR_U * uint32_t(CPP)) {
             uint32_t rows[RR_U];
@@ -537,14 +556,19 @@ __global__ void __launch_bounds__(128) tc_rerank_kernel(const float* __restrict_
                 rows[u] = valid[u] ? surv[q * cap + i] : 0u;
             }
             float4 xv[RR_U][F];
+            uint32_t ids[RR_U];
 #pragma unroll
             for (int u = 0; u < RR_U; ++u) {
                 const float4* xr = reinterpret_cast<const float4*>(xs + size_t(rows[u]) * d_pad) + sub * F;
 #pragma unroll
                 for (int f = 0; f < F; ++f) xv[u][f] = xr[f];
+                ids[u] = __ldg(perm + rows[u]);
             }
+            float dist[RR_U];
 #pragma unroll
-            for (int u = 0; u < RR_U; ++u) consider(rows[u], valid[u], xv[u]);
+            for (int u = 0; u < RR_U; ++u) dist[u] = distance(xv[u]);
+#pragma unroll
+            for (int u = 0; u < RR_U; ++u) consider(ids[u], valid[u], dist[u]);
         }
         if (lane == 0) atomicAdd(diag, (unsigned long long)n);
     } else {
@@ -552,6 +576,14 @@ __global__ void __launch_bounds__(128) tc_rerank_kernel(const float* __restrict_
         if (lane == 0) {
             atomicAdd(diag + 1, 1ull);
             ovf[1 + atomicAdd(ovf, 1u)] = uint32_t(q);
+        }
+        return;
+    }
+    if (WARP_LIST) {
+        if (lane < k) {
+            const uint32_t id = di_id(wl.list);
+            out_ids[q * k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
+            out_d[q * k + lane] = di_dist(wl.list);
         }
         return;
     }
@@ -667,9 +699,16 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
                    int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
-                   const TcDense* dense)
+                   int seed_rows, const TcDense* dense)
 {
     TcArgs a{};
+    // The k-th best of an item's rows beats the seed's only if the item holds k rows
+    // below the seed's bound, of which it expects k rows / seed rows.  Keeping the k
+    // bounds costs more than all else for k > 4, so items where that has a chance
+    // below about 0.001 (Poisson: k c >= k, c = 0.25 at k = 5, 0.55 at k = 32) don't.
+    // Measured: 6546 queries, k = 32, 182 cones of 95 rows of d = 96: screen 2750 -> 330 us.
+    const double least = k > 4 ? (0.2 + 0.011 * k) * seed_rows : 0.0;
+    a.tighten = uint32_t(least > k ? least : k);
     a.perm = perm;
     a.rowstat = rowstat;
     a.Y16 = static_cast<const uint16_t*>(Y16);

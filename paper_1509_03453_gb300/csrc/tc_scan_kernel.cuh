@@ -1,5 +1,5 @@
-// Tensor-core screening kernel: shared by the launchers of tc_scan.cu
-// (checks off) and tc_scan_debug.cu (checks on).
+// Tensor-core screening kernel: shared by the launchers of tc_scan.cu,
+// tc_scan_excl.cu, tc_dense.cu (checks off) and tc_scan_debug.cu (checks on).
 //
 // Batched candidate scan with 16-bit tensor-core screening and an exact fp32
 // rerank.  The 16-bit operands are bf16 (unit roundoff u = 2^-8) or fp16
@@ -9,11 +9,11 @@
 // scaled units (distances scale by s^2, exactly).  Subnormal fp16 rounding
 // adds an absolute error, covered by the terms Cabs(|x| + |q|).
 //
-// For a work item (cone c, group of up to 128 queries that probe it) the
+// For a work item (cone c, group of up to 256 queries that probe it: two tiles) the
 // squared distances are first estimated on the 5th-generation tensor cores
 // as  d~ = |q|^2 + |x|^2 - 2 q~.x~  (q~, x~ rounded to bf16, products exact,
 // fp32 accumulation in TMEM), M = 128 queries x N = 128 cone rows per MMA
-// group, the cone rows streamed by TMA (2-D tensor map over the bf16 copy of
+// group and query tile, the cone rows streamed by TMA (2-D tensor map over the bf16 copy of
 // the permuted vectors, swizzled K-major tiles).  Each query keeps an upper
 // bound U on its k-th best exact distance; a row survives the screen when
 //     d~ - E(q, x) <= U,   E = 2 c |q| |x| + B (|q|^2 + |x|^2),
@@ -31,7 +31,7 @@
 // a per-query list; the rerank computes their canonical fp32 distance (the
 // same expression as every other path) and selects the top-k, so the result
 // is bit-identical to the fp32 paths.  A query whose list overflows is
-// rescanned in full by the rerank (counted).
+// rescanned in full by the per-query scan (counted).
 #pragma once
 
 #include <cuda.h>
@@ -42,7 +42,7 @@
 
 namespace osann {
 
-constexpr int TC_M = 128;  // queries per item = MMA M
+constexpr int TC_M = 128;  // queries per query tile = MMA M
 constexpr int TC_N = 128;  // cone rows per tile = MMA N = TMEM columns
 
 // 16-bit conversions: PREC 0 = bf16, 1 = fp16 (round to nearest or up)
@@ -105,6 +105,7 @@ struct TcArgs {
     const uint32_t* qlist;    // list entries: query * S (+ position)
     TcDense dense;
     uint32_t* counter;
+    uint32_t tighten;    // items of this many rows or more tighten the bounds
     uint32_t* Ubits;     // per query: upper bound on the k-th best distance (float bits)
     uint32_t* surv_cnt;  // per query
     uint32_t* surv;      // Q x cap rows
@@ -212,6 +213,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     // k = 1 without exclusion: the minimum of a full chunk bounds the best
     // candidate directly, and survivors need only their row
     constexpr bool FAST = KMAX == 1 && !EXCL;
+    // columns read at a time: with a long list of bounds 64 values would spill
+    constexpr int CW = KMAX >= 16 ? 32 : 64;
     constexpr int row_bytes = tc_row_bytes(DP);
     constexpr int kblocks = DP >= 64 ? DP / 64 : 1;
     constexpr int epb = row_bytes / 2;
@@ -567,7 +570,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
 #pragma unroll
             for (int i = 0; i < TC_SBUF; ++i)
-                if (i < nb && pos[i] < uint32_t(a.cap)) a.surv[int64_t(e[i].y) * a.cap + pos[i]] = e[i].x;
+                if (i < nb) {
+                    if (pos[i] < uint32_t(a.cap)) a.surv[int64_t(e[i].y) * a.cap + pos[i]] = e[i].x;
+                    else a.Ubits[e[i].y] = 0;  // overflowed: the exact scan has it, later items keep nothing
+                }
             nb = 0;
         };
         for (uint32_t it = 0;; ++it) {
@@ -593,8 +599,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             float ubl[KMAX];  // k smallest upper bounds seen for this query in this item
 #pragma unroll
             for (int u = 0; u < KMAX; ++u) ubl[u] = INFINITY;
+            const bool tighten = wk.nrows >= a.tighten;
             auto bound = [&](float ub) {  // an upper bound on a candidate's distance
-                if (ub < ubl[KMAX - 1]) {
+                if (ub < cur.U) {
 #pragma unroll
                     for (int u = KMAX - 1; u > 0; --u) {
                         const float pu = ubl[u - 1];
@@ -626,7 +633,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     if (src >= 0 && (dr > dcc ? dr : dcc) <= a.radius) continue;
                     const uint32_t pos = atomicAdd(a.surv_cnt + q, 1u);
                     if (pos < uint32_t(a.cap)) a.surv[q * a.cap + pos] = row;
-                    bound(fmaxf((__uint_as_float(sbuf[i * SW + sr].y) + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
+                    if (tighten) bound(fmaxf((__uint_as_float(sbuf[i * SW + sr].y) + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
                 }
                 nb = 0;
             };
@@ -643,16 +650,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 tc_fence_after();
                 const int y0 = DENSE ? int(dense_row(a.dense, wk.r0, uint32_t(t))) : int(wk.r0) + t * TC_N;
                 const int nvalid = min(TC_N, DENSE ? int(a.dense.N) - y0 : int(wk.nrows) - t * TC_N);
-                for (int c0 = 0; c0 < nvalid; c0 += 64) {
-                    float v[64], m[2];
-                    tmem_ld32x2_min(tl + uint32_t(acc * TC_N + c0), v, m[0], m[1]);
-                    if (c0 + 64 >= nvalid) {
+                for (int c0 = 0; c0 < nvalid; c0 += CW) {
+                    float v[CW], m[CW / 32];
+                    if constexpr (CW == 64) tmem_ld32x2_min(tl + uint32_t(acc * TC_N + c0), v, m[0], m[1]);
+                    else tmem_ld32_min(tl + uint32_t(acc * TC_N + c0), v, m[0]);
+                    if (c0 + CW >= nvalid) {
                         // the accumulator's values are in registers: one arrival per warp
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(&accempty[acc]);
                     }
-                    const float vmin = fminf(m[0], m[1]);
+                    const float vmin = fminf(m[0], m[CW / 32 - 1]);
                     const int lim = nvalid - c0;
                     // columns past the item's rows (the next cone's, in the last
                     // tile) can only lower the minimum: the exact mask below drops them
@@ -667,7 +675,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             }
                         }
 #pragma unroll
-                        for (int h = 0; h < 2; ++h) {
+                        for (int h = 0; h < CW / 32; ++h) {
                             if (m[h] > cur.Uthr) continue;
                             uint32_t mask = 0;
 #pragma unroll
@@ -689,7 +697,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                                     for (int u = 1; u < 32; ++u) val = u == j ? v[32 * h + u] : val;
                                 }
                                 // d~ + E <= D + Uoff (scaled units)
-                                if (!FAST && !EXCL) bound(fmaxf((val + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
+                                if (!FAST && !EXCL && tighten) bound(fmaxf((val + cur.Uoff) * (1.0f + 1e-6f) * inv_sc2, 0.0f));
                                 sbuf[nb * SW + sr] =
                                     make_uint2(uint32_t(y0 + c0 + 32 * h + j), EXCL ? __float_as_uint(val) : qi);
                                 ++nb;
@@ -698,7 +706,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     }
                     if (DEBUG && active) {
                         // folded product against an fp32 evaluation, one column per thread
-                        const int col = lane + 32 * (c0 / 64 % 2);
+                        const int col = CW == 64 ? lane + 32 * (c0 / 64 % 2) : lane;
                         if (col < lim) {
                             const int row = y0 + c0 + col;
                             const float* xr = a.xs + size_t(row) * DP;
@@ -708,7 +716,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             const float4 rs = __ldg(a.rowstat + row);
                             float mine = v[0];
 #pragma unroll
-                            for (int u = 1; u < 64; ++u) mine = u == col ? v[u] : mine;
+                            for (int u = 1; u < CW; ++u) mine = u == col ? v[u] : mine;
                             const float ref = -2.0f * sc2 * dot + sc2 * rs.x - cur.Aq1 * sc * rs.y;
                             const float qnorm = sqrtf(cur.qn2);
                             const float lim2 = a.cdot2 * qnorm * sc * rs.y * 1.001f +
