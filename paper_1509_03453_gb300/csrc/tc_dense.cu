@@ -1,27 +1,27 @@
 // Dense screening: every row of the index against every query on the tensor
 // cores, the survivors evaluated exactly.  Used for linear search (Eq. 1 over all
 // N) and for searches whose cones are so thin that a tensor tile per cone would
-// be padding (a 128-row tile for a cone of six rows): there every row is screened
-// and only survivors in a probed cone count.
+// be padding (a 128-row tile for a cone of six rows), or whose survivor lists would
+// overflow cone by cone (k > 1 and many candidates): there every row is screened and
+// only survivors in a probed cone count.
 //
 // The screen (tc_scan_kernel.cuh) needs, per query, an upper bound U on its k-th
 // best exact distance, and leaves about as many survivors as rows lie below it.
 // So the rows are taken in phases, each seven times as many 128-row tiles as all
 // the ones before it (tile numbers divisible by 8^n, then the rest divisible by
 // 8^(n-1), ...; spread over the index, because neighbouring tiles hold neighbouring
-// cones and a run of them can be all near one query): after a phase the survivors' exact distances are merged into the
-// query's k best and U becomes the exact k-th, so that the next phase leaves about
-// 8 k survivors (times the share of the 16-bit error bound) and the whole search
-// a few hundred, whatever N.  The seed of the first phase is exact too (query
-// prep).  A query whose list overflows all the same (many rows within the error
+// cones and a run of them can be all near one query): after a phase the survivors'
+// exact distances are merged into the query's k best and U becomes the exact k-th, so
+// that the next phase leaves about 8 k N / M survivors (M the candidates: all N rows in
+// linear search), whatever N.  The seed of the first phase is exact too (query prep).  A query whose list overflows all the same (many rows within the error
 // bound of each other), or that is out of the 16-bit range, is left to an exact
 // scan of its own.
 //
 // What bounds it is the tensor core: 2 N Q d_pad (plus the 16 columns of the norm
 // terms) fp16 operations, 0.3 ms for 1000 queries over 2*10^6 rows of d = 128;
 // then the updates, whose chain survivor -> row -> list is latency.  Measured there
-// with k = 10: 0.97 ms (the last phase's screen 0.26 ms, updates 0.08 ms each, seed
-// 0.13 ms); the fp32 tile scan 117.6 ms.
+// with k = 10: 0.75 ms (0.95 with a register list per lane in seed and updates; the
+// last phase's screen 0.26 ms); the fp32 tile scan 117.6 ms.
 #include "osann.h"
 #include "tc_scan_kernel.cuh"
 

@@ -116,3 +116,24 @@ def test_thin_cones_overflow(osann):
     same(idx.search(Yd, 1500, 4), idx.search(Yd, 1500, 4, path="plain"))
     assert idx.status() == 0
     idx.close()
+
+
+@pytest.mark.parametrize("k", [2, 5, 16, 32])
+def test_many_candidates_match_scan(osann, k):
+    """Fat cones, k > 1 and so many candidates that survivor lists would overflow cone
+    by cone: the default path screens every row; the same bits as the per-query scan."""
+    rng = np.random.default_rng(k)
+    N, d, Q, P = 400_003, 32, 301, 40
+    X = rng.standard_normal((N, d)).astype(np.float32)
+    Y = rng.standard_normal((Q, d)).astype(np.float32)
+    idx = osann.Index(to_dev(X), 1)
+    Yd = to_dev(Y)
+    same(idx.search(Yd, P, k, path="fp16"), idx.search(Yd, P, k, path="plain"))
+    over = idx.screen_stats()["fallbacks"]
+    kw = dict(query_src=to_dev(rng.integers(0, N, Q)), grid_w=700, radius=5)
+    for extra in ({}, kw):
+        same(idx.search(Yd, P, k, **extra), idx.search(Yd, P, k, path="plain", **extra))
+    if k == 32:
+        assert over > 0 and idx.screen_stats()["fallbacks"] == 0
+    assert idx.status() == 0
+    idx.close()
