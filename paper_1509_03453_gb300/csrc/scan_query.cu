@@ -63,158 +63,158 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
         W == 1 ? int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5) : int64_t(blockIdx.x / blocks);
     const int64_t count = LISTED ? int64_t(a.sel[0]) : a.Q;
     for (int64_t at = first; at < count; at += LISTED ? int64_t(gridDim.x / blocks) : count) {
-    const int64_t q = LISTED ? int64_t(a.sel[1 + at]) : at;
-    const int g = lane / TPR, sub = lane % TPR;
-    float4 qv[F];
-    {
-        const float* y = a.Y + q * int64_t(a.d);
+        const int64_t q = LISTED ? int64_t(a.sel[1 + at]) : at;
+        const int g = lane / TPR, sub = lane % TPR;
+        float4 qv[F];
+        {
+            const float* y = a.Y + q * int64_t(a.d);
 #pragma unroll
-        for (int f = 0; f < F; ++f) {
-            const int c = 4 * (sub * F + f);
-            qv[f].x = c + 0 < a.d ? y[c + 0] : 0.f;
-            qv[f].y = c + 1 < a.d ? y[c + 1] : 0.f;
-            qv[f].z = c + 2 < a.d ? y[c + 2] : 0.f;
-            qv[f].w = c + 3 < a.d ? y[c + 3] : 0.f;
+            for (int f = 0; f < F; ++f) {
+                const int c = 4 * (sub * F + f);
+                qv[f].x = c + 0 < a.d ? y[c + 0] : 0.f;
+                qv[f].y = c + 1 < a.d ? y[c + 1] : 0.f;
+                qv[f].z = c + 2 < a.d ? y[c + 2] : 0.f;
+                qv[f].w = c + 3 < a.d ? y[c + 3] : 0.f;
+            }
         }
-    }
-    const int64_t src = EXCL ? a.query_src[q] : -1;
-    WarpTopk best;
-    // the row index, inside its load group, whose sum this lane ends with (its
-    // lowest for TPR < U), from the halving steps below: the top bit first
-    int u0 = 0;
+        const int64_t src = EXCL ? a.query_src[q] : -1;
+        WarpTopk best;
+        // the row index, inside its load group, whose sum this lane ends with (its
+        // lowest for TPR < U), from the halving steps below: the top bit first
+        int u0 = 0;
 #pragma unroll
-    for (int s = 0; (1 << s) < (TPR < U ? TPR : U); ++s) u0 |= ((lane >> s) & 1) << (2 - s);
-    const bool primary = sub < U;  // (lanes that share a sum: one of them speaks)
+        for (int s = 0; (1 << s) < (TPR < U ? TPR : U); ++s) u0 |= ((lane >> s) & 1) << (2 - s);
+        const bool primary = sub < U;  // (lanes that share a sum: one of them speaks)
 
-    const uint32_t* pl = a.probes + q * a.P_eff;
-    auto cone = [&](int64_t p, uint32_t& s0, uint32_t& n) {
-        s0 = 0;
-        n = 0;
-        if (p < a.P_eff) {
-            const uint32_t b = __ldg(pl + p);
-            if (b < a.NC) {  // never produced by the probe kernel otherwise; guards the offsets read
-                s0 = __ldg(a.offsets + b);
-                n = __ldg(a.offsets + b + 1) - s0;
+        const uint32_t* pl = a.probes + q * a.P_eff;
+        auto cone = [&](int64_t p, uint32_t& s0, uint32_t& n) {
+            s0 = 0;
+            n = 0;
+            if (p < a.P_eff) {
+                const uint32_t b = __ldg(pl + p);
+                if (b < a.NC) {  // never produced by the probe kernel otherwise; guards the offsets read
+                    s0 = __ldg(a.offsets + b);
+                    n = __ldg(a.offsets + b + 1) - s0;
+                }
             }
-        }
-    };
-    const int team = W == 1 ? 1 : a.team;
-    const int64_t pbeg = W == 1 ? 0 : 32 * (wq / team), pstep = W == 1 ? 32 : 32 * (int(blocks) * W / team);
-    const uint32_t tbeg = W == 1 ? 0u : uint32_t(wq % team * B), tstep = uint32_t(team * B);
-    uint32_t st, sz;
-    cone(pbeg + lane, st, sz);
-    for (int64_t p0 = pbeg; p0 < a.P_eff; p0 += pstep) {
-        uint32_t st1, sz1;
-        cone(p0 + pstep + lane, st1, sz1);  // the next 32 cones, behind these ones' rows
-        uint32_t incl = sz;
+        };
+        const int team = W == 1 ? 1 : a.team;
+        const int64_t pbeg = W == 1 ? 0 : 32 * (wq / team), pstep = W == 1 ? 32 : 32 * (int(blocks) * W / team);
+        const uint32_t tbeg = W == 1 ? 0u : uint32_t(wq % team * B), tstep = uint32_t(team * B);
+        uint32_t st, sz;
+        cone(pbeg + lane, st, sz);
+        for (int64_t p0 = pbeg; p0 < a.P_eff; p0 += pstep) {
+            uint32_t st1, sz1;
+            cone(p0 + pstep + lane, st1, sz1);  // the next 32 cones, behind these ones' rows
+            uint32_t incl = sz;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_up_sync(FULL, incl, o);
-            if (lane >= o) incl += v;
-        }
-        const uint32_t total = __shfl_sync(FULL, incl, 31);
-        for (uint32_t t0 = tbeg; t0 < total; t0 += tstep) {
-            // rows of the batch: lane l looks up rows l (and l + 32)
-            uint32_t row[RL], id[RL];
-#pragma unroll
-            for (int h = 0; h < RL; ++h) {
-                const uint32_t t = t0 + uint32_t(32 * h + lane);
-                int c = 0;  // the first cone whose inclusive sum passes t
-#pragma unroll
-                for (int w = 16; w > 0; w >>= 1)
-                    if (__shfl_sync(FULL, incl, c + w - 1) <= t) c += w;
-                const uint32_t r = __shfl_sync(FULL, st, c) + t -
-                                   (__shfl_sync(FULL, incl, c) - __shfl_sync(FULL, sz, c));
-                const bool live = t < total && (B >= 32 || lane < B);
-                row[h] = live ? r : 0u;
-                id[h] = live ? __ldg(a.perm + r) : 0u;
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += v;
             }
-            float4 xv[U][F];
+            const uint32_t total = __shfl_sync(FULL, incl, 31);
+            for (uint32_t t0 = tbeg; t0 < total; t0 += tstep) {
+                // rows of the batch: lane l looks up rows l (and l + 32)
+                uint32_t row[RL], id[RL];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const int e = u * CPP + g;
-                const uint32_t r = __shfl_sync(FULL, row[RL == 2 && u * CPP >= 32 ? RL - 1 : 0], e & 31);
-                const float4* xr = reinterpret_cast<const float4*>(a.xs + size_t(r) * a.d_pad) + sub * F;
+                for (int h = 0; h < RL; ++h) {
+                    const uint32_t t = t0 + uint32_t(32 * h + lane);
+                    int c = 0;  // the first cone whose inclusive sum passes t
 #pragma unroll
-                for (int f = 0; f < F; ++f) xv[u][f] = __ldg(xr + f);
-            }
-            float v[U];
+                    for (int w = 16; w > 0; w >>= 1)
+                        if (__shfl_sync(FULL, incl, c + w - 1) <= t) c += w;
+                    const uint32_t r = __shfl_sync(FULL, st, c) + t -
+                                       (__shfl_sync(FULL, incl, c) - __shfl_sync(FULL, sz, c));
+                    const bool live = t < total && (B >= 32 || lane < B);
+                    row[h] = live ? r : 0u;
+                    id[h] = live ? __ldg(a.perm + r) : 0u;
+                }
+                float4 xv[U][F];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float cp[F];
+                for (int u = 0; u < U; ++u) {
+                    const int e = u * CPP + g;
+                    const uint32_t r = __shfl_sync(FULL, row[RL == 2 && u * CPP >= 32 ? RL - 1 : 0], e & 31);
+                    const float4* xr = reinterpret_cast<const float4*>(a.xs + size_t(r) * a.d_pad) + sub * F;
 #pragma unroll
-                for (int f = 0; f < F; ++f) cp[f] = sq4(xv[u][f], qv[f]);
-                v[u] = pair_tree<F>(cp);
-            }
-            // pairwise tree across the TPR lanes: halving while a lane holds several sums
+                    for (int f = 0; f < F; ++f) xv[u][f] = __ldg(xr + f);
+                }
+                float v[U];
 #pragma unroll
-            for (int s = 0; (1 << s) < TPR; ++s) {
-                const int m = 1 << s;
-                const int half = U >> (s + 1);
-                if (half >= 1) {
-                    const bool up = (lane >> s) & 1;
+                for (int u = 0; u < U; ++u) {
+                    float cp[F];
 #pragma unroll
-                    for (int i = 0; i < half; ++i) {
-                        const float keep = up ? v[i + half] : v[i], give = up ? v[i] : v[i + half];
-                        v[i] = keep + __shfl_xor_sync(FULL, give, m);
+                    for (int f = 0; f < F; ++f) cp[f] = sq4(xv[u][f], qv[f]);
+                    v[u] = pair_tree<F>(cp);
+                }
+                // pairwise tree across the TPR lanes: halving while a lane holds several sums
+#pragma unroll
+                for (int s = 0; (1 << s) < TPR; ++s) {
+                    const int m = 1 << s;
+                    const int half = U >> (s + 1);
+                    if (half >= 1) {
+                        const bool up = (lane >> s) & 1;
+#pragma unroll
+                        for (int i = 0; i < half; ++i) {
+                            const float keep = up ? v[i + half] : v[i], give = up ? v[i] : v[i + half];
+                            v[i] = keep + __shfl_xor_sync(FULL, give, m);
+                        }
+                    } else {
+                        v[0] += __shfl_xor_sync(FULL, v[0], m);
                     }
-                } else {
-                    v[0] += __shfl_xor_sync(FULL, v[0], m);
                 }
-            }
 #pragma unroll
-            for (int i = 0; i < NV; ++i) {
-                const int e = (u0 + i) * CPP + g;
-                const uint32_t lo = __shfl_sync(FULL, id[0], e & 31);
-                const uint32_t hi = RL == 2 ? __shfl_sync(FULL, id[RL - 1], e & 31) : 0u;
-                const uint32_t cid = RL == 2 && e >= 32 ? hi : lo;
-                bool ok = primary && t0 + uint32_t(e) < total && v[i] <= di_dist(best.thr);
-                if (EXCL && ok && src >= 0) {
-                    int64_t dr = int64_t(cid) / a.grid_w - src / a.grid_w;
-                    int64_t dc = int64_t(cid) % a.grid_w - src % a.grid_w;
-                    dr = dr < 0 ? -dr : dr;
-                    dc = dc < 0 ? -dc : dc;
-                    ok = (dr > dc ? dr : dc) > a.radius;
-                }
-                unsigned m = __ballot_sync(FULL, ok);
-                while (m) {
-                    const int s = __ffs(int(m)) - 1;
-                    m &= m - 1u;
-                    best.insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)), a.k, lane);
+                for (int i = 0; i < NV; ++i) {
+                    const int e = (u0 + i) * CPP + g;
+                    const uint32_t lo = __shfl_sync(FULL, id[0], e & 31);
+                    const uint32_t hi = RL == 2 ? __shfl_sync(FULL, id[RL - 1], e & 31) : 0u;
+                    const uint32_t cid = RL == 2 && e >= 32 ? hi : lo;
+                    bool ok = primary && t0 + uint32_t(e) < total && v[i] <= di_dist(best.thr);
+                    if (EXCL && ok && src >= 0) {
+                        int64_t dr = int64_t(cid) / a.grid_w - src / a.grid_w;
+                        int64_t dc = int64_t(cid) % a.grid_w - src % a.grid_w;
+                        dr = dr < 0 ? -dr : dr;
+                        dc = dc < 0 ? -dc : dc;
+                        ok = (dr > dc ? dr : dc) > a.radius;
+                    }
+                    unsigned m = __ballot_sync(FULL, ok);
+                    while (m) {
+                        const int s = __ffs(int(m)) - 1;
+                        m &= m - 1u;
+                        best.insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)), a.k, lane);
+                    }
                 }
             }
+            st = st1;
+            sz = sz1;
         }
-        st = st1;
-        sz = sz1;
-    }
-    if (W > 1) {
-        __shared__ uint64_t sh[W * 32];
-        if (lane < a.k) sh[wb * 32 + lane] = best.list;
-        __syncthreads();
-        if (wb == 0)
-            for (int w = 1; w < W; ++w)
-                for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
-        if (blocks > 1) {
-            // the blocks' lists, through the first one's shared memory
-            namespace cg = cooperative_groups;
-            cg::cluster_group cl = cg::this_cluster();
-            if (wb == 0 && lane < a.k) sh[lane] = best.list;
-            cl.sync();
-            if (rank == 0 && wb == 0)
-                for (unsigned r = 1; r < blocks; ++r) {
-                    const uint64_t* rs = cl.map_shared_rank(sh, r);
-                    best.offer(lane < a.k, lane < a.k ? rs[lane] : EMPTY_DI, a.k, lane);
-                }
-            cl.sync();  // no block leaves, or goes on, while its list is read
-        } else if (LISTED) {
+        if (W > 1) {
+            __shared__ uint64_t sh[W * 32];
+            if (lane < a.k) sh[wb * 32 + lane] = best.list;
             __syncthreads();
+            if (wb == 0)
+                for (int w = 1; w < W; ++w)
+                    for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
+            if (blocks > 1) {
+                // the blocks' lists, through the first one's shared memory
+                namespace cg = cooperative_groups;
+                cg::cluster_group cl = cg::this_cluster();
+                if (wb == 0 && lane < a.k) sh[lane] = best.list;
+                cl.sync();
+                if (rank == 0 && wb == 0)
+                    for (unsigned r = 1; r < blocks; ++r) {
+                        const uint64_t* rs = cl.map_shared_rank(sh, r);
+                        best.offer(lane < a.k, lane < a.k ? rs[lane] : EMPTY_DI, a.k, lane);
+                    }
+                cl.sync();  // no block leaves, or goes on, while its list is read
+            } else if (LISTED) {
+                __syncthreads();
+            }
         }
-    }
-    if (rank == 0 && wb == 0 && lane < a.k) {
-        const uint32_t id = di_id(best.list);
-        a.out_ids[q * a.k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
-        a.out_d[q * a.k + lane] = di_dist(best.list);
-    }
+        if (rank == 0 && wb == 0 && lane < a.k) {
+            const uint32_t id = di_id(best.list);
+            a.out_ids[q * a.k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
+            a.out_d[q * a.k + lane] = di_dist(best.list);
+        }
     }
 }
 

@@ -251,11 +251,13 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
         __shared__ uint64_t best_sh[W > 1 ? W * KMAX : 1];
         if (WARP_LIST) {
             if (lane < a.k) best_sh[wq * KMAX + lane] = wl.list;
-        } else for (int j = 0; j < a.k; ++j) {
-            const uint64_t head = topk_head<KMAX>(list, a.k);
-            const uint64_t b = warp_min_u64(head);
-            if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
-            if (lane == 0) best_sh[wq * KMAX + j] = b;
+        } else {
+            for (int j = 0; j < a.k; ++j) {
+                const uint64_t head = topk_head<KMAX>(list, a.k);
+                const uint64_t b = warp_min_u64(head);
+                if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
+                if (lane == 0) best_sh[wq * KMAX + j] = b;
+            }
         }
         __syncthreads();
         if (wq != 0) return;
@@ -263,9 +265,11 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
         if (WARP_LIST) {
             for (int w = 1; w < W; ++w)
                 wl.offer(lane < a.k, lane < a.k ? best_sh[w * KMAX + lane] : EMPTY_DI, a.k, lane);
-        } else for (int i = lane; i < W * a.k; i += 32) {
-            const uint64_t v = best_sh[(i / a.k) * KMAX + i % a.k];
-            if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
+        } else {
+            for (int i = lane; i < W * a.k; i += 32) {
+                const uint64_t v = best_sh[(i / a.k) * KMAX + i % a.k];
+                if (v < list[KMAX - 1]) topk_insert<KMAX>(list, v);
+            }
         }
     }
     if (LC > 0 && lane == 0) atomicAdd(a.diag, (unsigned long long)n);
@@ -282,12 +286,14 @@ __global__ void __launch_bounds__(32 * DENSE_WARPS) dense_update_kernel(const Up
     if (WARP_LIST) {
         if (lane < a.k) put(lane, wl.list);
         kth = di_dist(wl.thr);
-    } else for (int j = 0; j < a.k; ++j) {
-        const uint64_t head = topk_head<KMAX>(list, a.k);
-        const uint64_t b = warp_min_u64(head);
-        if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
-        kth = di_dist(b);
-        if (lane == 0) put(j, b);
+    } else {
+        for (int j = 0; j < a.k; ++j) {
+            const uint64_t head = topk_head<KMAX>(list, a.k);
+            const uint64_t b = warp_min_u64(head);
+            if (head == b && b != EMPTY_DI) topk_remove<KMAX>(list, a.k, b);
+            kth = di_dist(b);
+            if (lane == 0) put(j, b);
+        }
     }
     if (lane == 0 && !a.last) {
         // the canonical fp32 distance is within 6.6e-7 relative of the exact one
