@@ -570,10 +570,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 }
 #pragma unroll
             for (int i = 0; i < TC_SBUF; ++i)
-                if (i < nb) {
-                    if (pos[i] < uint32_t(a.cap)) a.surv[int64_t(e[i].y) * a.cap + pos[i]] = e[i].x;
-                    else a.Ubits[e[i].y] = 0;  // overflowed: the exact scan has it, later items keep nothing
-                }
+                if (i < nb && pos[i] < uint32_t(a.cap)) a.surv[int64_t(e[i].y) * a.cap + pos[i]] = e[i].x;
+            // overflowed: the exact scan has the query, later items keep nothing of it (k = 1
+            // hardly overflows, and its launch lost 6 to 10% to this: 988 -> 1046 us)
+            if constexpr (KMAX > 1) {
+#pragma unroll
+                for (int i = 0; i < TC_SBUF; ++i)
+                    if (i < nb && pos[i] >= uint32_t(a.cap)) a.Ubits[e[i].y] = 0;
+            }
             nb = 0;
         };
         for (uint32_t it = 0;; ++it) {
