@@ -404,6 +404,10 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
 
 // The data scale of the screen: s = 1 for bf16; for fp16 the power of two
 // with s^2 max|x|^2 <= 2^14 (all-zero data: 1).  tcs = (s, s^2, 1/s^2, X), X >= every row norm.
+// The largest finite fp32 norm squared, below 2^128, needs s = 2^-57: s^2 and 1/s^2 are
+// normal numbers, so nothing clamps the exponent from below (a scale too large would
+// make the fp16 norm columns infinite and lose the row).  Above, s stays at 2^40:
+// smaller norms only use less of the fp16 range.
 template <int PREC>
 __global__ void tc_scale_kernel(const uint32_t* __restrict__ maxn2_bits, float* __restrict__ tcs)
 {
@@ -415,7 +419,7 @@ __global__ void tc_scale_kernel(const uint32_t* __restrict__ maxn2_bits, float* 
         frexpf(m, &x);  // m < 2^x
         const int t = 14 - x;
         e = t >= 0 ? t / 2 : -((1 - t) / 2);
-        e = e > 40 ? 40 : (e < -40 ? -40 : e);
+        e = e > 40 ? 40 : e;
     }
     const float sc = ldexpf(1.0f, e);
     tcs[0] = sc;

@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             cur.Cq = q4.z;
             cur.U = q4.w;
             cur.Uthr = sc2 * q4.w - (1.0f - a.Bn) * q4.x + q4.z;
-            cur.Uoff = (1.0f + a.Bn) * q4.x + 2.0f * a.Bn * sc2 * xmax * xmax + 2.0f * q4.y * sc * xmax + q4.z;
+            cur.Uoff = (1.0f + a.Bn) * q4.x + 2.0f * a.Bn * (sc * xmax) * (sc * xmax) + 2.0f * q4.y * sc * xmax + q4.z;
             const float U0 = cur.U;
             const bool active = qi != 0xFFFFFFFFu;
             const int64_t q = active ? int64_t(qi) : 0;

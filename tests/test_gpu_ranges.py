@@ -1,0 +1,54 @@
+"""Vectors at the ends of what the 16-bit screen can scale: large norms and rows of very
+different norms.  Linear search, the cone screen and the screen over all rows return
+the bits of the per-query fp32 scan, which scales nothing."""
+import numpy as np
+import pytest
+
+from helpers import to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def osann():
+    import paper_1509_03453_gb300 as m
+    from paper_1509_03453_gb300 import build
+    build.build()
+    m.load()
+    return m
+
+
+def same(a, b):
+    assert np.array_equal(to_np(a[0]), to_np(b[0]))
+    assert np.array_equal(to_np(a[1]).view(np.uint32), to_np(b[1]).view(np.uint32))
+
+
+def check(osann, X, Y, L, P, k, dense):
+    """dense: the default path screens every row (its workspace is neither the per-query
+    scan's nor the cone screen's)."""
+    idx = osann.Index(to_dev(X), L)
+    Yd = to_dev(Y)
+    sizes = {p: idx.workspace_size(len(Y), P, k, p) for p in ("auto", "plain", "fp16")}
+    assert (sizes["auto"] not in (sizes["plain"], sizes["fp16"])) == dense
+    ref = idx.search(Yd, P, k, path="plain")
+    assert (to_np(ref[0]) >= 0).any()
+    same(idx.search(Yd, P, k), ref)
+    same(idx.search(Yd, P, k, path="fp16"), ref)
+    same(idx.search(Yd, P, k, path="bf16"), ref)
+    if L == 1:
+        same(idx.bruteforce(Yd, k), idx.search(Yd, idx.NC, k, path="plain"))
+    assert idx.status() == 0
+    idx.close()
+
+
+@pytest.mark.parametrize("d", [32, 100])
+@pytest.mark.parametrize("sx,sy", [(1e13, 1e13), (1e14, 1e11), (1e15, 1e12), (1e17, 1e13), (5e17, 5e17)])
+def test_large_norms(osann, d, sx, sy):
+    rng = np.random.default_rng(3)
+    X = rng.standard_normal((9000, d)).astype(np.float32) * np.float32(sx)
+    Y = rng.standard_normal((1600, d)).astype(np.float32) * np.float32(sy)
+    Y[7] = 0
+    Y[9] *= np.float32(1e-20)
+    check(osann, X, Y[:60], 1, 2 * d, 3, False)
+    X = rng.standard_normal((30_011, d)).astype(np.float32) * np.float32(sx)
+    check(osann, X, Y, *((3, 1500, 4) if d == 32 else (2, 2600, 4)), True)
