@@ -328,7 +328,7 @@ int index_device(const osann_index* ix) { return ix->device; }
 }  // namespace osann
 
 // Coefficients of the screening bound
-//     E = cdot2 |q||x| + Bn (|q|^2 + |x|^2) + cabs (|q| + |x|):
+//     E = cdot2 |q||x| + Bn (|q|^2 + |x|^2) + cabs (|q| + |x|) + tc_norm_eps:
 // 16-bit rounding of both operands (unit roundoff u = 2^-8 for bf16, 2^-11
 // for fp16) and the fp32 accumulation of d_pad products (taken as
 // d_pad 2^-20, sixteen times the round-to-nearest bound); for Bn the fp32

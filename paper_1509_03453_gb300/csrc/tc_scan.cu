@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128)
         const float qn = sc * sc * s, qnorm = sc * sqrtf(s);
         const float A = (a.cdot2 * qnorm + a.cabs) * (1.0f + 6.1035156e-5f);
         const float Ap = from16<PREC>(to16_ru<PREC>(A));
-        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm);
+        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm + tc_norm_eps(PREC));
         a.Ubits[q] = __float_as_uint(U);
         a.surv_cnt[q] = unscreenable || a.tcs[3] > 3.4e38f ? uint32_t(cap) + 1u : 0u;
     }
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
         const float qn = sc * sc * s, qnorm = sc * sqrtf(s);
         const float A = (a.cdot2 * qnorm + a.cabs) * (1.0f + 6.1035156e-5f);
         const float Ap = from16<PREC>(to16_ru<PREC>(A));
-        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm);
+        a.qstat[q] = make_float4(qn, qnorm, -Ap, a.cabs * qnorm + tc_norm_eps(PREC));
         a.Ubits[q] = __float_as_uint(U);
         a.surv_cnt[q] = unscreenable || a.tcs[3] > 3.4e38f ? uint32_t(a.cap) + 1u : 0u;
     }

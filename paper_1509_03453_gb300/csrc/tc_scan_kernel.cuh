@@ -7,7 +7,8 @@
 // first multiplied by an exact power of two s, chosen from the largest row
 // norm so that |s x|^2 <= 2^14, and all screening quantities are in those
 // scaled units (distances scale by s^2, exactly).  Subnormal fp16 rounding
-// adds an absolute error, covered by the terms Cabs(|x| + |q|).
+// adds an absolute error, covered by the terms Cabs(|x| + |q|) (the vectors) and eps
+// (the norm columns).
 //
 // For a work item (cone c, group of up to 256 queries that probe it: two tiles) the
 // squared distances are first estimated on the 5th-generation tensor cores
@@ -16,7 +17,7 @@
 // group and query tile, the cone rows streamed by TMA (2-D tensor map over the bf16 copy of
 // the permuted vectors, swizzled K-major tiles).  Each query keeps an upper
 // bound U on its k-th best exact distance; a row survives the screen when
-//     d~ - E(q, x) <= U,   E = 2 c |q| |x| + B (|q|^2 + |x|^2),
+//     d~ - E(q, x) <= U,   E = 2 c |q| |x| + B (|q|^2 + |x|^2) + Cabs (|x| + |q|) + eps,
 // where c bounds the 16-bit rounding of both operands plus the fp32
 // accumulation (c = 2u + u^2 + K 2^-20) and B the fp32 error of
 // the norms, of their bf16 hi/lo split and a cushion for the fp32 rounding of
@@ -69,6 +70,12 @@ __device__ __forceinline__ uint16_t to16_exact(int prec, float f)
 {
     return prec == 0 ? __bfloat16_as_ushort(__float2bfloat16_rn(f)) : __half_as_ushort(__float2half_rn(f));
 }
+// Absolute rounding error of a row's folded norm terms, scaled units: the low word of
+// fp16(|x|^2) has a spacing of 2^-24 however small the norm, so the split is off by up
+// to 2^-25 (twice that here); bf16 has fp32's exponent range.  It matters where the
+// scale follows a far larger row: beside a row of norm 10^6, rows of norm 5 lost 1 in
+// 60 of their queries' nearest neighbours without it.
+__host__ __device__ constexpr float tc_norm_eps(int prec) { return prec == 0 ? 7.5e-37f : 5.9604645e-8f; }
 __device__ __forceinline__ uint32_t pack16(uint16_t lo, uint16_t hi) { return uint32_t(lo) | (uint32_t(hi) << 16); }
 
 __host__ __device__ constexpr int tc_row_bytes(int d_pad) { return d_pad >= 64 ? 128 : d_pad * 2; }
@@ -97,7 +104,7 @@ struct TcArgs {
     const uint32_t* perm;
     const float4* rowstat;    // per row: ((1-B)|x|^2, |x|, |x|^2, 0); N + TC_N rows
     const uint16_t* Y16;      // Q x d_pad, 16-bit -2 s y
-    const float4* qstat;      // per query, scaled: (|q|^2, |q|, -A' (16-bit value, A' >= 2c|q| + Cabs), Cabs |q|)
+    const float4* qstat;      // per query, scaled: (|q|^2, |q|, -A' (16-bit value, A' >= 2c|q| + Cabs), Cabs |q| + eps)
     const float* tcs;         // (s, s^2, 1/s^2, X): X bounds every row norm (unscaled)
     const int64_t* query_src;
     const uint4* items;       // (first row, end row, first slot, slot count)
@@ -197,7 +204,7 @@ struct TcQConst {
     float Uthr;  // s^2 U - (1-B)|q|^2 + Cq (scaled)
     float Aq1;   // A' (scaled)
     float U;     // upper bound on the k-th best exact distance (unscaled)
-    float Cq;    // Cabs |q| (scaled)
+    float Cq;    // Cabs |q| + the norm terms' absolute error (scaled)
     float Uoff;  // (1+B)|q|^2 + 2B s^2 X^2 + 2A' s X + Cq, X >= every row norm (scaled)
 };
 
@@ -725,7 +732,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                             const float qnorm = sqrtf(cur.qn2);
                             const float lim2 = a.cdot2 * qnorm * sc * rs.y * 1.001f +
                                                4.0f * a.Bn * (cur.qn2 + sc2 * rs.z) +
-                                               2.0f * a.cabs * (sc * rs.y + qnorm) + 1e-30f;
+                                               2.0f * a.cabs * (sc * rs.y + qnorm) + 2.0f * tc_norm_eps(a.prec) + 1e-30f;
                             atomicAdd(a.diag + 2, 1ull);
                             if (fabsf(mine - ref) > lim2) {
                                 atomicAdd(a.diag + 3, 1ull);

@@ -52,3 +52,25 @@ def test_large_norms(osann, d, sx, sy):
     check(osann, X, Y[:60], 1, 2 * d, 3, False)
     X = rng.standard_normal((30_011, d)).astype(np.float32) * np.float32(sx)
     check(osann, X, Y, *((3, 1500, 4) if d == 32 else (2, 2600, 4)), True)
+
+
+@pytest.mark.parametrize("norm", [3e5, 1e6, 3e6, 1e8])
+def test_one_row_of_large_norm(osann, norm):
+    """The scale follows the largest norm; the others' squares are then around the fp16
+    subnormal spacing, whose rounding the screen's bound has to cover."""
+    rng = np.random.default_rng(4)
+    X = rng.standard_normal((30_011, 32)).astype(np.float32)
+    X[17] *= np.float32(norm / np.linalg.norm(X[17]))
+    Y = rng.standard_normal((1600, 32)).astype(np.float32)
+    Y[7] = 0
+    check(osann, X, Y[:300], 1, 40, 2, False)
+    check(osann, X, Y, 3, 1500, 2, True)
+
+
+@pytest.mark.parametrize("scale", [1e-13, 3e-15, 1e-16])
+def test_small_norms(osann, scale):
+    rng = np.random.default_rng(6)
+    X = rng.standard_normal((30_011, 32)).astype(np.float32) * np.float32(scale)
+    Y = rng.standard_normal((1600, 32)).astype(np.float32) * np.float32(scale)
+    check(osann, X, Y[:300], 1, 40, 2, False)
+    check(osann, X, Y, 3, 1500, 2, True)
