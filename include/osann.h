@@ -272,7 +272,7 @@ int osann_probes(const osann_index *index, const float *d_queries, int64_t Q, in
                  void *d_ws, size_t ws_bytes, void *stream);
 
 /* Workspace bytes that osann_search / osann_search_excl need for (Q, P, k)
- * on `path`. */
+ * on `path`.  The size for a batch serves every smaller one. */
 size_t osann_search_workspace_size(const osann_index *index, int64_t Q, int32_t P, int32_t k, int32_t path);
 
 /* ROSANNA+ search (Sec. 4-B) on an index built with centroids: each query

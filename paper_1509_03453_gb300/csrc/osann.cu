@@ -587,7 +587,7 @@ static double rows_per_cone(const osann_index* ix)
 {
     return double(ix->N) / (ix->occupied > 0 ? double(ix->occupied) : double(ix->NC));
 }
-static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, double cones, int mode)
+static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int mode)
 {
     if (!ix->tc_ready[1] || ix->hashed || ix->K || ix->key_mode != OSANN_KEY_SET || ix->L > 4 || ix->N < 8192 ||
         Q > 65536)
@@ -596,7 +596,7 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
     const double row = 4.0 * ix->d_pad, seed_rate = 2.4e6;
     const double tile = 80.0 * double((ix->d + 15) / 16 + 1);
     const double probes = double(Q) * double(P_eff);
-    const double rows = rows_per_cone(ix), M = rows * double(P_eff);
+    const double rows = rows_per_cone(ix), M = rows * double(P_eff), cones = double(ix->N) / rows;
     // A phase holds eight times the rows before it, so it leaves about 8 k N / M
     // survivors per query (fewer where the probed cones hold nearer rows than the
     // others): past the list's capacity the exact scan would have the work.  (2240 by
@@ -628,7 +628,8 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, d
     return dense_us < 0.85 * other;
 }
 
-static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path)
+// The mode of a path, the dense screen aside (its workspace grows with Q).
+static int cone_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int path)
 {
     if (path == OSANN_PATH_PLAIN) return MODE_PLAIN;
     if (path == OSANN_PATH_BATCHED) return MODE_BATCHED;
@@ -645,9 +646,26 @@ static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
     const double per_cone = double(Q) * double(P_eff) / cones;
     const double per_query = double(P_eff) * double(ix->N) / double(ix->NC);
     const bool big_queries = per_query >= 16384.0;
-    int mode = per_cone >= 16.0 || big_queries ? MODE_BATCHED : MODE_PLAIN;
-    if (ix->tc_ready[1] && (per_cone >= 8.0 || big_queries)) mode = MODE_FP16;
-    return dense_pays(ix, Q, P_eff, k, cones, mode) ? MODE_DENSE : mode;
+    if (ix->tc_ready[1] && (per_cone >= 8.0 || big_queries)) return MODE_FP16;
+    return per_cone >= 16.0 || big_queries ? MODE_BATCHED : MODE_PLAIN;
+}
+static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path)
+{
+    const int mode = cone_mode(ix, Q, P_eff, path);
+    return path == OSANN_PATH_AUTO && dense_pays(ix, Q, P_eff, k, mode) ? MODE_DENSE : mode;
+}
+
+// Bytes of the workspace of a search.  Where the dense screen is chosen they hold the
+// cone-major or per-query form too: whether it pays is not monotone in Q, and a
+// workspace sized for the largest batch serves every smaller one, in one form or the
+// other (search_impl).  (256 more: a size that is neither form's names the dense one.)
+static size_t search_ws_bytes(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path, int group, int Mv = 1)
+{
+    const int mode = choose_mode(ix, Q, P_eff, k, path);
+    const size_t need = ws_layout(ix, Q, P_eff, k, mode, group, Mv).total;
+    if (mode != MODE_DENSE) return need;
+    const size_t other = ws_layout(ix, Q, P_eff, k, cone_mode(ix, Q, P_eff, path), group, Mv).total;
+    return (need > other ? need : other) + 256;
 }
 
 // Rows of an occupied cone, on average, below which a query's warps take cones each
@@ -1259,7 +1277,7 @@ size_t osann_search_workspace_size_group(const osann_index* ix, int64_t Q, int32
     if (!ix || Q < 0 || P < 1 || k < 1 || k > MAX_K) return 0;
     if (path < 0 || path > OSANN_PATH_FP16 || group < 0) return 0;
     const int64_t P_eff = p_eff(ix, P);
-    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, k, path), group).total;
+    return search_ws_bytes(ix, Q, P_eff, k, path, group);
 }
 
 size_t osann_search_clusters_workspace_size(const osann_index* ix, int64_t Q, int32_t M, int32_t P, int32_t k,
@@ -1269,7 +1287,7 @@ size_t osann_search_clusters_workspace_size(const osann_index* ix, int64_t Q, in
     if (path < 0 || path > OSANN_PATH_FP16) return 0;
     const int Mv = clusters_of(ix, M);
     const int64_t P_eff = Mv * p_eff(ix, P);
-    return ws_layout(ix, Q, P_eff, k, choose_mode(ix, Q, P_eff, k, path), 0, Mv).total;
+    return search_ws_bytes(ix, Q, P_eff, k, path, 0, Mv);
 }
 
 size_t osann_search_workspace_size(const osann_index* ix, int64_t Q, int32_t P, int32_t k, int32_t path)
@@ -1399,14 +1417,15 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         return OSANN_ERR_UNSUPPORTED;
     }
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const int mode = choose_mode(ix, Q, P_eff, k, path);
-    const int prec = mode == MODE_FP16 ? 1 : 0;
+    int mode = choose_mode(ix, Q, P_eff, k, path);
+    // a workspace sized for another batch may lack room for the dense screen
+    if (mode == MODE_DENSE && d_ws && ws_bytes < ws_layout(ix, Q, P_eff, k, mode, group, Mv).total)
+        mode = cone_mode(ix, Q, P_eff, path);
     if (tc_mode(mode)) {
-        int trc = ensure_tc(const_cast<osann_index*>(ix), prec, st);
+        int trc = ensure_tc(const_cast<osann_index*>(ix), mode == MODE_FP16 ? 1 : 0, st);
         if (trc) return trc;
     }
-    const bool batched = mode != MODE_PLAIN && mode != MODE_DENSE;
-    const WsLayout L = ws_layout(ix, Q, P_eff, k, mode, group, Mv);
+    WsLayout L = ws_layout(ix, Q, P_eff, k, mode, group, Mv);
     // the query-side steps read neither the rows, nor a second-level table,
     // nor a basis or centroids of the index only with a plain direct table
     SideStream front{};
@@ -1420,6 +1439,12 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
     void* owned = nullptr;
     if (!d_ws) {
         owned = d_ws = dev_alloc(L.total, fst);  // usable on st after the join below
+        if (!d_ws && mode == MODE_DENSE) {
+            // (fp16 operands are there: the dense screen needs them too)
+            mode = cone_mode(ix, Q, P_eff, path);
+            L = ws_layout(ix, Q, P_eff, k, mode, group, Mv);
+            owned = d_ws = dev_alloc(L.total, fst);
+        }
         if (!d_ws) {
             set_error("osann_search: workspace allocation failed (%zu bytes)", L.total);
             return OSANN_ERR_OOM;
@@ -1431,6 +1456,8 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         set_error("osann_search: workspace too small (%zu < %zu)", ws_bytes, L.total);
         return OSANN_ERR_INVALID;
     }
+    const int prec = mode == MODE_FP16 ? 1 : 0;
+    const bool batched = mode != MODE_PLAIN && mode != MODE_DENSE;
     char* w = static_cast<char*>(d_ws);
     // the dense screen needs the first cones only (its seed)
     const int64_t P_front = mode == MODE_DENSE && P_per > DENSE_SEED_CONES ? DENSE_SEED_CONES : P_per;
