@@ -493,7 +493,8 @@ int osann_server_pending(const osann_server *server, int64_t *waiting_queries, i
 /* Autotuner: for every index and batch bucket, time each candidate (path,
  * work-list group size, screen layout) -- plain; batched with the default
  * and 32-query groups; fp16 screening with the default (256), 128- and
- * 64-query groups -- on max_batch rows sampled
+ * 64-query groups; OSANN_PATH_AUTO where that screens every row -- on
+ * max_batch rows sampled
  * from the index itself, reps timed runs each, and keep the fastest.
  * out_choices (nullable) receives (path, group) per (index, bucket);
  * osann_server_choices gives the layouts too.  Call with no request in the

@@ -668,6 +668,13 @@ static size_t search_ws_bytes(const osann_index* ix, int64_t Q, int64_t P_eff, i
     return (need > other ? need : other) + 256;
 }
 
+namespace osann {
+bool index_screens_all(const osann_index* ix, int64_t Q, int P, int k)
+{
+    return choose_mode(ix, Q, p_eff(ix, P), k, OSANN_PATH_AUTO) == MODE_DENSE;
+}
+}  // namespace osann
+
 // Rows of an occupied cone, on average, below which a query's warps take cones each
 // in the per-query scan instead of sharing every cone's rows.
 constexpr double THIN_ROWS = 24.0;

@@ -67,3 +67,25 @@ def test_failed_dense_workspace_takes_the_smaller_form(osann):
         assert rc == 0 and a.calls == 2 and a.live == {}
     same((ids, d2), idx.search(Y, 1500, 1, path="plain"))
     idx.close()
+
+
+@pytest.mark.parametrize("graphs", [True, False])
+def test_tuner_can_choose_the_dense_screen(osann, graphs):
+    """Thin cones and k = 10: screening every row is several times faster than cone by cone,
+    and only the default path does it; batches of all sizes give the per-query scan's bits."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    idx = osann.Index(torch.randn((200_000, 32), generator=g, device="cuda"), 3)
+    Y = torch.randn((2048, 32), generator=g, device="cuda")
+    P, k = 6000, 10
+    srv = osann.Server([idx], P=[P], k=[k], slots=1, max_batch=2048, graphs=graphs)
+    choices = srv.tune(reps=2, queries=[Y])
+    assert choices[0][-1] == ("auto", 0, "default")
+    ref = idx.search(Y, P, k, path="plain")
+    for q in (2048, 1999, 1100, 300, 31, 1):
+        t = srv.submit(0, Y[:q])
+        srv.drain()
+        same(srv.result(t), [r[:q] for r in ref])
+    srv.close()
+    idx.close()
