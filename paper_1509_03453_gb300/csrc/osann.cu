@@ -268,6 +268,8 @@ struct osann_index {
     // asynchronous build); kept for the index's life, so the automatic path
     // choice -- and with it the workspace size -- never changes
     int64_t occupied = 0;
+    // rows of the largest cone when it was last read (-1: never); a rebuild keeps it
+    int64_t largest = -1;
     unsigned __int128 nc_true = 0;
     bool hashed = false;          // second-level table (128-bit cone ids)
     int key_bits = 0;             // significant bits of the 128-bit ids
@@ -678,17 +680,31 @@ bool index_screens_all(const osann_index* ix, int64_t Q, int P, int k)
 // Rows of an occupied cone, on average, below which a query's warps take cones each
 // in the per-query scan instead of sharing every cone's rows.
 constexpr double THIN_ROWS = 24.0;
-// The per-query scan of the probed cones (sel: of the listed queries).  A shortened
+// The per-query scan of the probed cones (sel: of the listed queries).  scratch: Q + 1
+// words (the callers': the query signs, of no use once the lists are made).  A shortened
 // wait budget, a test hook, takes the staged form, whose waits it is for.
 static int exact_scan(const osann_index* ix, const float* Y, int64_t Q, const uint32_t* probes, int64_t P_eff, int k,
-                      const int64_t* src, int64_t grid_w, int radius, const uint32_t* sel, int64_t* ids, float* dists,
-                      cudaStream_t st)
+                      const int64_t* src, int64_t grid_w, int radius, const uint32_t* sel, uint32_t* scratch,
+                      int64_t* ids, float* dists, cudaStream_t st)
 {
     if (plain_wait_budget_set())
         return launch_plain_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff, uint32_t(ix->NC),
                                  k, src, grid_w, radius, sel, ix->num_sms, ids, dists, ix->status, st);
+    // A warp alone reads a row of 512 bytes in 0.18 us, so that one cone of 400 000 rows
+    // among thin ones held a batch of 3000 queries for 98 ms (0.72 with this; a block's
+    // staged scan 12).  Too many rows for it: 92 us of them, 16 average cones, or a warp's
+    // part of the whole batch (of a listed one: nothing is known), whichever is most.  At
+    // half that line image patches (cones of up to 654 rows among 4.5 on average) would be
+    // listed too: 20000 queries, 20 cones, 361 us either way with k = 4, 324 -> 359 with 1.
+    const double rows = rows_per_cone(ix);
+    const double part = sel ? 0.0 : double(Q) * double(P_eff) * rows / (32.0 * ix->num_sms);
+    double most = 65536.0 / ix->d_pad;
+    if (most < 16.0 * rows) most = 16.0 * rows;
+    if (most < part) most = part;
+    const bool even = most >= double(ix->N) || (ix->largest >= 0 && double(ix->largest) <= most);
     return launch_query_scan(ix->xs, ix->offsets, ix->perm, ix->d_pad, Y, ix->d, Q, probes, P_eff, uint32_t(ix->NC), k,
-                             src, grid_w, radius, rows_per_cone(ix) >= THIN_ROWS, sel, ix->num_sms, ids, dists, st);
+                             src, grid_w, radius, rows >= THIN_ROWS, even ? 0xFFFFFFFFu : uint32_t(most), scratch, sel,
+                             ix->num_sms, ids, dists, st);
 }
 
 // Probed cones looked up for the dense screen's seed (it stops at its rows).
@@ -1101,7 +1117,7 @@ static int build_impl(const float* d_data, int64_t N, int32_t d, int32_t L, cons
         return rc;
     }
     cudaMemsetAsync(ix->status, 0, 4, st);
-    ix->max_bucket = host_status[1];
+    ix->max_bucket = ix->largest = host_status[1];
     ix->occupied = host_status[3];
     ix->tc_ready[1] = maps_ok;
     *out = ix;
@@ -1274,7 +1290,10 @@ int osann_status(const osann_index* ix, void* stream, uint32_t* flags)
     if (e != cudaSuccess) return cuda_fail(e, "osann_status");
     *flags = h[0];
     // an index built asynchronously learns its largest cone here
-    if (ix->max_bucket < 0) const_cast<osann_index*>(ix)->max_bucket = h[1];
+    if (ix->max_bucket < 0) {
+        const_cast<osann_index*>(ix)->max_bucket = h[1];
+        const_cast<osann_index*>(ix)->largest = h[1];
+    }
     return OSANN_OK;
 }
 
@@ -1541,7 +1560,8 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                 // queries whose survivor list overflowed: exact scan of their probed cones
                 if (!rc)
                     rc = exact_scan(ix, Y, Q, probes, P_eff, k, src, grid_w, radius,
-                                    reinterpret_cast<const uint32_t*>(w + L.ovf), ids, dists, st);
+                                    reinterpret_cast<const uint32_t*>(w + L.ovf),
+                                    reinterpret_cast<uint32_t*>(w + L.qsign), ids, dists, st);
             }
         } else if (!rc) {
             {
@@ -1576,12 +1596,13 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         if (!rc) {
             if (P_front < P_eff) rc = query_front(ix, Y, Q, P_eff, 1, L, w, false, k, st, left);
             if (!rc)
-                rc = exact_scan(ix, Y, Q, probes, P_eff, k, src, grid_w, radius, left, ids, dists, st);
+                rc = exact_scan(ix, Y, Q, probes, P_eff, k, src, grid_w, radius, left, reinterpret_cast<uint32_t*>(w + L.qsign), ids,
+                                dists, st);
         }
     } else if (!rc) {
         StageScope s(OSANN_STAGE_PLAIN_SCAN, st);
-        rc = exact_scan(ix, Y, Q, reinterpret_cast<uint32_t*>(w + L.probes), P_eff, k, src, grid_w, radius, nullptr, ids,
-                        dists, st);
+        rc = exact_scan(ix, Y, Q, reinterpret_cast<uint32_t*>(w + L.probes), P_eff, k, src, grid_w, radius, nullptr,
+                        reinterpret_cast<uint32_t*>(w + L.qsign), ids, dists, st);
     }
     if (owned) dev_free(owned, L.total, st);
     return rc;
@@ -1652,7 +1673,7 @@ int osann_build_search(const float* d_data, int64_t N, int32_t d, int32_t L, con
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "osann_build_search");
         } else {
-            if (ix->max_bucket < 0) ix->max_bucket = h[1];
+            if (ix->max_bucket < 0) ix->max_bucket = ix->largest = h[1];
             if (h[0] & ST_TIMEOUT) {
                 set_error("osann_build_search: a device wait timed out");
                 rc = OSANN_ERR_TIMEOUT;

@@ -114,11 +114,12 @@ int launch_plain_scan(const float* xs, const uint32_t* offsets, const uint32_t* 
 
 // scan_query.cu: the per-query scan, one to 128 warps per query.  fat: fat cones (a
 // query's warps share their rows instead of taking cones each); sel (nullable): device
-// list [count, q_0, ...] of the queries to scan
+// list [count, q_0, ...] of the queries to scan; warp_rows: rows of a cone that are too many
+// for one warp (0xFFFFFFFF: no cone is that large); scratch: Q + 1 words
 int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
                      int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
-                     int64_t grid_w, int radius, bool fat, const uint32_t* sel, int num_sms, int64_t* out_ids,
-                     float* out_d, cudaStream_t st);
+                     int64_t grid_w, int radius, bool fat, uint32_t warp_rows, uint32_t* scratch, const uint32_t* sel,
+                     int num_sms, int64_t* out_ids, float* out_d, cudaStream_t st);
 
 // scan_batched.cu
 struct BatchedBuffers {

@@ -29,6 +29,7 @@ namespace osann {
 namespace {
 
 constexpr int U = 8;  // row loads in flight per lane
+constexpr uint32_t NONE = 0xFFFFFFFFu;
 
 struct QueryScanArgs {
     const float *xs, *Y;
@@ -43,13 +44,22 @@ struct QueryScanArgs {
     int64_t* out_ids;
     float* out_d;
 };
+// (a parameter of its own: QueryScanArgs, grown by these, made the compiler keep fewer
+// loads in flight in the forms that do not read them, 4 to 6% of their time)
+struct QueryScanBig {
+    uint32_t rows;    // rows of a cone that are too many for a warp (NONE: no cone is that large)
+    uint32_t big;     // and for a team
+    uint32_t* heavy;  // list [count, q_0, ...] of the queries left because of that
+};
 
 // TPR lanes per row, F float4 pieces each; W warps per block.  W = 1: a query per
 // warp, four per block; otherwise a cluster of a.cluster blocks per query, in teams
 // of a.team warps: a team takes 32 cones at a time, its warps those cones' rows by turns.
 // LISTED: the clusters take the queries of a list made on the device by turns.
-template <int TPR, int F, bool EXCL, int W, bool LISTED = false>
-__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const QueryScanArgs a)
+// BIG: a query that meets a cone of more than b.big rows (one may hold half the index)
+// is not answered but put on a list, for a launch in which all its warps share it.
+template <int TPR, int F, bool EXCL, int W, bool BIG, bool LISTED = false>
+__global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const QueryScanArgs a, const QueryScanBig b)
 {
     constexpr int CPP = 32 / TPR;     // rows per load instruction
     constexpr int B = U * CPP;        // rows per batch: 8 .. 64
@@ -57,11 +67,13 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
     constexpr int NV = TPR >= U ? 1 : U / TPR;  // row sums a lane ends with
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wb = W == 1 ? 0 : int(threadIdx.x >> 5);
-    const unsigned blocks = W == 1 ? 1u : unsigned(a.cluster), rank = W == 1 ? 0u : blockIdx.x % blocks;
+    const int64_t count = LISTED ? int64_t(a.sel[0]) : a.Q;
+    // (a long list of queries whose warps share every cone: a block each)
+    const bool alone = LISTED && !BIG && a.team == W * a.cluster && count * 2 >= int64_t(gridDim.x);
+    const unsigned blocks = W == 1 || alone ? 1u : unsigned(a.cluster), rank = W == 1 ? 0u : blockIdx.x % blocks;
     const int wq = int(rank) * W + wb;  // warp of the query
     const int64_t first =
         W == 1 ? int64_t(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5) : int64_t(blockIdx.x / blocks);
-    const int64_t count = LISTED ? int64_t(a.sel[0]) : a.Q;
     for (int64_t at = first; at < count; at += LISTED ? int64_t(gridDim.x / blocks) : count) {
         const int64_t q = LISTED ? int64_t(a.sel[1 + at]) : at;
         const int g = lane / TPR, sub = lane % TPR;
@@ -86,19 +98,24 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
         for (int s = 0; (1 << s) < (TPR < U ? TPR : U); ++s) u0 |= ((lane >> s) & 1) << (2 - s);
         const bool primary = sub < U;  // (lanes that share a sum: one of them speaks)
 
+        bool left = false;
         const uint32_t* pl = a.probes + q * a.P_eff;
         auto cone = [&](int64_t p, uint32_t& s0, uint32_t& n) {
             s0 = 0;
             n = 0;
             if (p < a.P_eff) {
-                const uint32_t b = __ldg(pl + p);
-                if (b < a.NC) {  // never produced by the probe kernel otherwise; guards the offsets read
-                    s0 = __ldg(a.offsets + b);
-                    n = __ldg(a.offsets + b + 1) - s0;
+                const uint32_t c = __ldg(pl + p);
+                if (c < a.NC) {  // never produced by the probe kernel otherwise; guards the offsets read
+                    s0 = __ldg(a.offsets + c);
+                    n = __ldg(a.offsets + c + 1) - s0;
+                    if (BIG && n > b.big) {
+                        left = true;
+                        n = 0;
+                    }
                 }
             }
         };
-        const int team = W == 1 ? 1 : a.team;
+        const int team = W == 1 ? 1 : (alone ? W : a.team);
         const int64_t pbeg = W == 1 ? 0 : 32 * (wq / team), pstep = W == 1 ? 32 : 32 * (int(blocks) * W / team);
         const uint32_t tbeg = W == 1 ? 0u : uint32_t(wq % team * B), tstep = uint32_t(team * B);
         uint32_t st, sz;
@@ -187,10 +204,17 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
             st = st1;
             sz = sz1;
         }
+        if (BIG && W == 1) left = __any_sync(FULL, left);
         if (W > 1) {
             __shared__ uint64_t sh[W * 32];
+            __shared__ int sh_left;
             if (lane < a.k) sh[wb * 32 + lane] = best.list;
-            __syncthreads();
+            if (BIG) {
+                left = __syncthreads_or(left);
+                if (threadIdx.x == 0) sh_left = left;
+            } else {
+                __syncthreads();
+            }
             if (wb == 0)
                 for (int w = 1; w < W; ++w)
                     for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
@@ -204,13 +228,16 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
                     for (unsigned r = 1; r < blocks; ++r) {
                         const uint64_t* rs = cl.map_shared_rank(sh, r);
                         best.offer(lane < a.k, lane < a.k ? rs[lane] : EMPTY_DI, a.k, lane);
+                        if (BIG && *cl.map_shared_rank(&sh_left, r)) left = true;
                     }
                 cl.sync();  // no block leaves, or goes on, while its list is read
             } else if (LISTED) {
                 __syncthreads();
             }
         }
-        if (rank == 0 && wb == 0 && lane < a.k) {
+        if (BIG && left) {
+            if (rank == 0 && wb == 0 && lane == 0) b.heavy[1 + atomicAdd(b.heavy, 1u)] = uint32_t(q);
+        } else if (rank == 0 && wb == 0 && lane < a.k) {
             const uint32_t id = di_id(best.list);
             a.out_ids[q * a.k + lane] = id == 0xFFFFFFFFu ? int64_t(-1) : int64_t(id);
             a.out_d[q * a.k + lane] = di_dist(best.list);
@@ -233,11 +260,12 @@ double rounds(int64_t Q, int64_t P, int64_t W, int num_sms)
     return double((Q + slots - 1) / slots) * double(((P + 31) / 32 + teams - 1) / teams) / double(team);
 }
 
-template <int TPR, int F, bool EXCL, int W, bool LISTED>
-int launch_team(QueryScanArgs a, bool fat, int cluster, int64_t clusters, cudaStream_t st)
+template <int TPR, int F, bool EXCL, int W, bool LISTED = false>
+int launch_team(QueryScanArgs a, QueryScanBig b, bool fat, int cluster, int64_t clusters, cudaStream_t st)
 {
     a.team = int(team_of(a.P_eff, int64_t(W) * cluster, fat));
     a.cluster = cluster;
+    b.big = b.rows < NONE / uint32_t(a.team) ? b.rows * uint32_t(a.team) : NONE;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(unsigned(clusters * cluster));
     cfg.blockDim = dim3(32 * W);
@@ -248,7 +276,8 @@ int launch_team(QueryScanArgs a, bool fat, int cluster, int64_t clusters, cudaSt
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, query_scan_kernel<TPR, F, EXCL, W, LISTED>, a);
+    const cudaError_t e = b.rows != NONE ? cudaLaunchKernelEx(&cfg, query_scan_kernel<TPR, F, EXCL, W, true, LISTED>, a, b)
+                                         : cudaLaunchKernelEx(&cfg, query_scan_kernel<TPR, F, EXCL, W, false, LISTED>, a, b);
     const int rc = count_launch();
     if (e != cudaSuccess && !rc) {
         set_error("per-query scan: launch failed (%s)", cudaGetErrorString(e));
@@ -273,49 +302,74 @@ int launch_team(QueryScanArgs a, bool fat, int cluster, int64_t clusters, cudaSt
 // queries, 7000 thin cones, 210 / 132 / 97 / 72; 135 queries over patches 76 / 56 / 60
 // / 93; 200 queries 48 / 56 / 60 / 83).  A list of queries takes eight: it is as often
 // one query as all.
+//
+// Where a cone may be too large for a warp (b.rows), a launch of eight blocks per query
+// follows for the queries with one (one, two, four, eight blocks: 4000 queries over thin
+// cones of d = 64, some of them with a cone of 400 000 rows, 5744 / 2920 / 1509 / 803; left
+// to their warps 35 600), except behind a form whose every query has sixteen warps on
+// each cone.
 template <int TPR, int F, bool EXCL>
-int launch_w(const QueryScanArgs& a, bool fat, int num_sms, cudaStream_t st)
+int launch_listed(const QueryScanArgs& a, const QueryScanBig& b, bool fat, int num_sms, cudaStream_t st)
 {
-    if (a.sel) {
-        const int64_t clusters = 2 * int64_t(num_sms) / 8;
-        return launch_team<TPR, F, EXCL, 16, true>(a, fat, 8, clusters < 1 ? 1 : (clusters < a.Q ? clusters : a.Q), st);
-    }
-    if (a.Q >= (fat ? 6144 : (a.P_eff >= 256 ? 3600 : 2048))) {
-        query_scan_kernel<TPR, F, EXCL, 1><<<unsigned((a.Q + 3) / 4), 128, 0, st>>>(a);
-        return count_launch();
-    }
-    int w = fat && a.Q >= 2048 ? 4 : (fat && a.Q >= 608 ? 8 : 16);
+    const int64_t n = 2 * int64_t(num_sms) / 8, clusters = n < a.Q ? n : a.Q;
+    return launch_team<TPR, F, EXCL, 16, true>(a, b, fat, 8, clusters < 1 ? 1 : clusters, st);
+}
+template <int TPR, int F, bool EXCL>
+int launch_w(QueryScanArgs a, QueryScanBig b, bool fat, int num_sms, cudaStream_t st)
+{
+    int w = fat && a.Q >= 2048 ? 4 : (fat && a.Q >= 608 ? 8 : 16), c = 8;
     if (!fat && a.Q >= 256)
         for (const int v : {8, 4})
             if (rounds(a.Q, a.P_eff, v, num_sms) <= rounds(a.Q, a.P_eff, w, num_sms)) w = v;
-    if (w == 4) return launch_team<TPR, F, EXCL, 4, false>(a, fat, 1, a.Q, st);
-    if (w == 8) return launch_team<TPR, F, EXCL, 8, false>(a, fat, 1, a.Q, st);
-    int c = 8;
-    while (c > 1 && a.Q * c > 2 * int64_t(num_sms)) c /= 2;
-    return launch_team<TPR, F, EXCL, 16, false>(a, fat, c, a.Q, st);
+    if (a.Q >= (fat ? 6144 : (a.P_eff >= 256 ? 3600 : 2048))) w = 1;
+    if (a.sel) w = 16;
+    else if (w < 16) c = 1;
+    while (!a.sel && c > 1 && a.Q * c > 2 * int64_t(num_sms)) c /= 2;
+    if (team_of(a.P_eff, int64_t(w) * c, fat) >= 16) b.rows = NONE;
+    const bool big = b.rows != NONE;
+    if (big) cudaMemsetAsync(b.heavy, 0, 4, st);
+    int rc;
+    if (a.sel) {
+        rc = launch_listed<TPR, F, EXCL>(a, b, fat, num_sms, st);
+    } else if (w == 1) {
+        b.big = b.rows;
+        const unsigned blocks = unsigned((a.Q + 3) / 4);
+        if (big) query_scan_kernel<TPR, F, EXCL, 1, true><<<blocks, 128, 0, st>>>(a, b);
+        else query_scan_kernel<TPR, F, EXCL, 1, false><<<blocks, 128, 0, st>>>(a, b);
+        rc = count_launch();
+    } else {
+        rc = w == 4 ? launch_team<TPR, F, EXCL, 4>(a, b, fat, 1, a.Q, st)
+             : w == 8 ? launch_team<TPR, F, EXCL, 8>(a, b, fat, 1, a.Q, st)
+                      : launch_team<TPR, F, EXCL, 16>(a, b, fat, c, a.Q, st);
+    }
+    if (rc || !big) return rc;
+    a.sel = b.heavy;
+    b.rows = NONE;
+    return launch_listed<TPR, F, EXCL>(a, b, true, num_sms, st);
 }
 
 template <bool EXCL>
-int launch_d(const QueryScanArgs& a, bool fat, int num_sms, cudaStream_t st)
+int launch_d(const QueryScanArgs& a, const QueryScanBig& b, bool fat, int num_sms, cudaStream_t st)
 {
     switch (a.d_pad) {
-    case 16: return launch_w<4, 1, EXCL>(a, fat, num_sms, st);
-    case 32: return launch_w<8, 1, EXCL>(a, fat, num_sms, st);
-    case 64: return launch_w<16, 1, EXCL>(a, fat, num_sms, st);
-    case 128: return launch_w<32, 1, EXCL>(a, fat, num_sms, st);
+    case 16: return launch_w<4, 1, EXCL>(a, b, fat, num_sms, st);
+    case 32: return launch_w<8, 1, EXCL>(a, b, fat, num_sms, st);
+    case 64: return launch_w<16, 1, EXCL>(a, b, fat, num_sms, st);
+    case 128: return launch_w<32, 1, EXCL>(a, b, fat, num_sms, st);
     }
-    return launch_w<32, 2, EXCL>(a, fat, num_sms, st);
+    return launch_w<32, 2, EXCL>(a, b, fat, num_sms, st);
 }
 
 }  // namespace
 
 int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* perm, int d_pad, const float* Y, int d,
                      int64_t Q, const uint32_t* probes, int64_t P_eff, uint32_t NC, int k, const int64_t* query_src,
-                     int64_t grid_w, int radius, bool fat, const uint32_t* sel, int num_sms, int64_t* out_ids,
-                     float* out_d, cudaStream_t st)
+                     int64_t grid_w, int radius, bool fat, uint32_t warp_rows, uint32_t* scratch, const uint32_t* sel,
+                     int num_sms, int64_t* out_ids, float* out_d, cudaStream_t st)
 {
     if (Q == 0) return 0;
     QueryScanArgs a{};
+    const QueryScanBig b{warp_rows, NONE, scratch};
     a.sel = sel;
     a.xs = xs;
     a.Y = Y;
@@ -333,7 +387,7 @@ int launch_query_scan(const float* xs, const uint32_t* offsets, const uint32_t* 
     a.NC = NC;
     a.out_ids = out_ids;
     a.out_d = out_d;
-    return query_src ? launch_d<true>(a, fat, num_sms, st) : launch_d<false>(a, fat, num_sms, st);
+    return query_src ? launch_d<true>(a, b, fat, num_sms, st) : launch_d<false>(a, b, fat, num_sms, st);
 }
 
 }  // namespace osann
