@@ -19,7 +19,7 @@ namespace osann {
 // (tcs[3] = inf).
 //
 // The rows are read at random, so what bounds the kernel is the latency of the
-// chain list entry -> cone offsets -> rows.  From PREP_SMALL_Q queries up, a warp
+// chain list entry -> cone offsets -> rows.  From prep_small_q queries up, a warp
 // per query hides it behind the other warps and takes a cone at a time.  A small
 // batch leaves the chip idle instead: there, PREP_SMALL warps share a query; 32
 // probes are looked up at once (a lane each), the next 32 while these ones' rows
@@ -29,7 +29,6 @@ namespace osann {
 // one warp each 28, the lookup of 32 cones 36 us.
 constexpr int TC_SEED_ILP = 8;  // row groups loaded per iteration
 constexpr int PREP_SMALL = 8;   // warps per query of a small batch
-constexpr int PREP_SMALL_Q = 1024;
 constexpr int PREP_WARP_LIST = 16;  // k above 4: one list per warp, over its lanes
 
 // Rows scanned exactly for a query's initial bound.  A large batch keeps
@@ -49,6 +48,21 @@ int tc_seed_rows(int64_t Q, int k, double M)
     const double r = k > 4 ? k * M / 64.0 : 0.0, q = Q > 0 ? (262144.0 + double(Q) - 1.0) / double(Q) : 1024.0;
     const double n = r > q ? r : q;
     return n < 64.0 ? 64 : (n > 1024.0 ? 1024 : int(n));
+}
+
+// Queries from which a warp each beats a block each.  The blocks shorten the chain, but
+// keep the chip from the work list beside them, the sooner the less a row's read takes.
+// Whole searches with blocks / warps (us), k = 1: d = 16, 200 / 600 / 1000 queries 90 / 86,
+// 97 / 89, 108 / 93; d = 32, N = 10^6, 300 / 500 / 800: 135 / 136, 132 / 122, 148 / 147; d = 64, N =
+// 4*10^6, 400 / 600 / 1000: 269 / 272, 312 / 259, 412 / 353; d = 50, N = 3.5*10^5, 500 / 700:
+// 157 / 166, 190 / 206; d = 128, 500 / 800 / 1000: 304 / 384, 362 / 386, 369 / 369; fat cones on
+// 16 PCA axes, 997: 432 / 374; thin ones of d = 100, 900: 481 / 541.  k = 10, whose seed is
+// longer: d = 16, 400 / 1000: 166 / 165, 198 / 171; d = 32, 1000: 499 / 520.
+static int prep_small_q(int d_pad, int k, bool fat)
+{
+    if (d_pad <= 16) return k > 4 ? 512 : 128;
+    if (d_pad <= 64 && k <= 4) return d_pad <= 32 ? 448 : 512;
+    return fat ? 900 : 1024;
 }
 
 struct PrepArgs {
@@ -680,7 +694,7 @@ int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, 
     a.Ubits = Ubits;
     a.surv_cnt = surv_cnt;
     // d_pad <= 128: one float4 piece per lane
-    const bool small = Q < PREP_SMALL_Q || !probes;
+    const bool small = Q < prep_small_q(d_pad, k, N >= 128 * int64_t(NC)) || !probes;
 #define OSANN_PREP(PR, KM)                                                                              \
     do {                                                                                                \
         if (small) tc_query_prep_block_kernel<1, PR, KM><<<unsigned(Q), 32 * PREP_SMALL, 0, st>>>(a);   \
