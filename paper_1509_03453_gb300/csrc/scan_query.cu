@@ -296,7 +296,9 @@ int launch_team(QueryScanArgs a, QueryScanBig b, bool fat, int cluster, int64_t 
 //   87, 3000: 227 / 124 / 129 / 171, 8000 (40 probes): 325 / 336 / 358 / 476.
 // Over thin cones the number of warps whose blocks need the fewest rounds in all,
 // which orders all of these but those bound by DRAM (795 queries, 260 probes: 165
-// with sixteen warps, 141 with four; 550 probes: 348 with eight, 301 with four).
+// with sixteen warps, 141 with four; 550 probes: 348 with eight, 301 with four).  A tie goes to
+// the shorter block, with many probes to the longer (900 queries, 1055 probes of 4.6 rows of
+// d = 128: four warps 511, eight 554, sixteen 456; the staged scan 469).
 // With sixteen, as many blocks, up to eight, as give every SM two (one / two / four /
 // eight blocks: 24 queries, 198 cones of 17 rows of d = 100, 91 / 58 / 46 / 42; 6
 // queries, 7000 thin cones, 210 / 132 / 97 / 72; 135 queries over patches 76 / 56 / 60
@@ -319,8 +321,10 @@ int launch_w(QueryScanArgs a, QueryScanBig b, bool fat, int num_sms, cudaStream_
 {
     int w = fat && a.Q >= 2048 ? 4 : (fat && a.Q >= 608 ? 8 : 16), c = 8;
     if (!fat && a.Q >= 256)
-        for (const int v : {8, 4})
-            if (rounds(a.Q, a.P_eff, v, num_sms) <= rounds(a.Q, a.P_eff, w, num_sms)) w = v;
+        for (const int v : {8, 4}) {
+            const double r = rounds(a.Q, a.P_eff, v, num_sms), r0 = rounds(a.Q, a.P_eff, w, num_sms);
+            if (r < r0 || (r == r0 && a.P_eff < 1024)) w = v;
+        }
     if (a.Q >= (fat ? 6144 : (a.P_eff >= 256 ? 3600 : 2048))) w = 1;
     if (a.sel) w = 16;
     else if (w < 16) c = 1;
