@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
                         const int s = __ffs(int(m)) - 1;
                         m &= m - 1u;
                         best.insert(pack_di(__shfl_sync(FULL, v[i], s), __shfl_sync(FULL, cid, s)), a.k, lane);
+                        m &= __ballot_sync(FULL, v[i] <= di_dist(best.thr));
                     }
                 }
             }
@@ -215,9 +216,15 @@ __global__ void __launch_bounds__(W == 1 ? 128 : 32 * W) query_scan_kernel(const
             } else {
                 __syncthreads();
             }
-            if (wb == 0)
-                for (int w = 1; w < W; ++w)
-                    for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
+            if (W < 16) {
+                if (wb == 0)
+                    for (int w = 1; w < W; ++w)
+                        for (int j = 0; j < a.k; ++j) best.insert(sh[w * 32 + j], a.k, lane);
+            } else if (wb == 0) {
+                // many lists: 32 entries at a time
+                for (int i = a.k + lane; i - lane < W * a.k; i += 32)
+                    best.offer(i < W * a.k, i < W * a.k ? sh[i / a.k * 32 + i % a.k] : EMPTY_DI, a.k, lane);
+            }
             if (blocks > 1) {
                 // the blocks' lists, through the first one's shared memory
                 namespace cg = cooperative_groups;
