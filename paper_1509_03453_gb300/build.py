@@ -19,8 +19,8 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(PKG, "_build")
 LIB_PATH = os.path.join(OUT_DIR, "libosann.so")
 SOURCES = ["osann.cu", "keys.cu", "buckets.cu", "probes.cu", "scan_plain.cu", "scan_query.cu", "scan_batched.cu",
-           "static_search.cu", "tc_scan.cu", "tc_scan_debug.cu", "tc_scan_excl.cu", "tc_dense.cu", "server.cu",
-           "shard_merge.cu", "cone_table.cu", "clusters.cu"]
+           "static_search.cu", "tc_scan.cu", "tc_scan_debug.cu", "tc_scan_excl.cu", "tc_scan_uneven.cu",
+           "tc_dense.cu", "server.cu", "shard_merge.cu", "cone_table.cu", "clusters.cu"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

@@ -526,9 +526,12 @@ int launch_gather_rows(const float* X, int64_t N, int d, int d_pad, const uint32
 }
 
 __global__ void max_bucket_kernel(const uint32_t* __restrict__ offsets, int64_t NC, uint32_t* __restrict__ out,
-                                  uint32_t* __restrict__ occ)
+                                  uint32_t* __restrict__ occ, const float4* __restrict__ rowstat, int64_t N,
+                                  float* __restrict__ mean_norm)
 {
     uint32_t m = 0, n = 0;
+    const bool sample = blockIdx.x == 0 && threadIdx.x < 32;
+    float x = sample ? rowstat[int64_t(threadIdx.x) * N / 32].y : 0.0f;
     for (int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; c < NC; c += int64_t(gridDim.x) * blockDim.x) {
         uint32_t s = offsets[c + 1] - offsets[c];
         m = s > m ? s : m;
@@ -542,14 +545,20 @@ __global__ void max_bucket_kernel(const uint32_t* __restrict__ offsets, int64_t 
     }
     if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
     if ((threadIdx.x & 31) == 0 && occ && n) atomicAdd(occ, n);
+    if (sample) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (threadIdx.x == 0) *mean_norm = x / 32.0f;
+    }
 }
 
-int launch_max_bucket(const uint32_t* offsets, int64_t NC, uint32_t* out_max, cudaStream_t st, uint32_t* out_occ)
+int launch_max_bucket(const uint32_t* offsets, int64_t NC, uint32_t* out_max, uint32_t* out_occ, const float4* rowstat,
+                      int64_t N, float* out_mean_norm, cudaStream_t st)
 {
     int64_t blocks = (NC + 255) / 256;
     if (blocks > 1024) blocks = 1024;
     if (blocks < 1) blocks = 1;
-    max_bucket_kernel<<<unsigned(blocks), 256, 0, st>>>(offsets, NC, out_max, out_occ);
+    max_bucket_kernel<<<unsigned(blocks), 256, 0, st>>>(offsets, NC, out_max, out_occ, rowstat, N, out_mean_norm);
     return count_launch();
 }
 

@@ -270,6 +270,8 @@ struct osann_index {
     int64_t occupied = 0;
     // rows of the largest cone when it was last read (-1: never); a rebuild keeps it
     int64_t largest = -1;
+    // whether the largest norm is far above the others, when a synchronous build saw it
+    bool uneven = false;
     unsigned __int128 nc_true = 0;
     bool hashed = false;          // second-level table (128-bit cone ids)
     int key_bits = 0;             // significant bits of the 128-bit ids
@@ -935,7 +937,9 @@ static int enqueue_build(osann_index* ix, const float* d_data, char* temp, float
         rc = launch_gather_rows(d_data, N, d, ix->d_pad, ix->perm, ix->xs, ix->rowstat, ix->Bn,
                                 tc_possible ? ix->tcs + 4 : nullptr, ix->x16[1], ix->xe16[1], st, ix->num_sms);
     }
-    if (!rc) rc = launch_max_bucket(ix->offsets, NC, ix->status + 1, st, ix->status + 3);
+    if (!rc)
+        rc = launch_max_bucket(ix->offsets, NC, ix->status + 1, ix->status + 3, ix->rowstat, N,
+                               reinterpret_cast<float*>(ix->status + 8), st);
     return rc;
 }
 
@@ -1098,9 +1102,9 @@ static int build_impl(const float* d_data, int64_t N, int32_t d, int32_t L, cons
         *out = ix;
         return OSANN_OK;
     }
-    uint32_t host_status[4] = {0, 0, 0, 0};  // flags, largest cone, largest |x|^2, occupied cones
+    uint32_t host_status[9] = {};  // flags, largest cone, largest |x|^2, occupied cones, ..., mean norm of a sample
     if (!rc) {
-        cudaError_t e = cudaMemcpyAsync(host_status, ix->status, 16, cudaMemcpyDeviceToHost, st);
+        cudaError_t e = cudaMemcpyAsync(host_status, ix->status, sizeof(host_status), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = cuda_fail(e, "osann_build");
     }
@@ -1119,6 +1123,10 @@ static int build_impl(const float* d_data, int64_t N, int32_t d, int32_t L, cons
     cudaMemsetAsync(ix->status, 0, 4, st);
     ix->max_bucket = ix->largest = host_status[1];
     ix->occupied = host_status[3];
+    float max2, mean;
+    std::memcpy(&max2, &host_status[2], 4);
+    std::memcpy(&mean, &host_status[8], 4);
+    ix->uneven = std::sqrt(max2) > 4.0f * mean;
     ix->tc_ready[1] = maps_ok;
     *out = ix;
     return OSANN_OK;
@@ -1549,7 +1557,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                     reinterpret_cast<uint32_t*>(w + L.scnt), reinterpret_cast<uint32_t*>(w + L.surv),
                                     TC_SURV_CAP, ix->status, ix->diag, ix->xs, Y, P_eff, ix->d, ix->d_pad, k,
                                     ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms,
-                                    tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)));
+                                    tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)), ix->uneven);
             }
             if (!rc) {
                 StageScope s(OSANN_STAGE_TC_RERANK, st);

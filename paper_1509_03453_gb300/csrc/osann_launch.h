@@ -54,9 +54,10 @@ int launch_gather_rows(const float* X, int64_t N, int d, int d_pad, const uint32
                        float Bn, const float* tcs, uint16_t* x16, uint16_t* xe16, cudaStream_t st,
                        int num_sms);  // tcs, x16, xe16 null: no fp16 operands
 int launch_tc_scale(int prec, const uint32_t* maxn2_bits, float* tcs, cudaStream_t st);
-// out_max: largest cone size (atomicMax); out_occ (nullable): occupied cones (atomicAdd)
-int launch_max_bucket(const uint32_t* offsets, int64_t NC, uint32_t* out_max, cudaStream_t st,
-                      uint32_t* out_occ = nullptr);
+// out_max: largest cone size (atomicMax); out_occ: occupied cones (atomicAdd);
+// out_mean_norm: mean norm of 32 rows spread over the index
+int launch_max_bucket(const uint32_t* offsets, int64_t NC, uint32_t* out_max, uint32_t* out_occ, const float4* rowstat,
+                      int64_t N, float* out_mean_norm, cudaStream_t st);
 
 // cone_table.cu: the second-level table of occupied cones.  From perm
 // (sorted by 128-bit id) and the ids: keys[row] = compact cone, offsets over
@@ -189,13 +190,14 @@ struct TcDense {
     uint32_t N, Q, tiles, chunks, groups, mul, n_items;
     int skip;
 };
+// uneven: the bounds of k > 1 and of exclusion take each row's own norm;
 // dense (non-null): its items instead of b's list, and no tightening of U
 int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float4* rowstat, const void* Y16,
                    const float4* qstat, const float* tcs, const int64_t* query_src, int64_t grid_w, int radius,
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
                    int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
-                   int seed_rows, const TcDense* dense = nullptr);
+                   int seed_rows, bool uneven, const TcDense* dense = nullptr);
 int launch_tc_rerank(const float* xs, int d_pad, const uint32_t* perm, const uint32_t* offsets, uint32_t NC,
                      const float* Y, int d, int64_t Q, const uint32_t* probes, int64_t P_eff, const uint32_t* surv_cnt,
                      const uint32_t* surv, int cap, int k, const int64_t* query_src, int64_t grid_w, int radius,

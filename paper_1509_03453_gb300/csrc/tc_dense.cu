@@ -431,7 +431,7 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
             rc = launch_tc_scan(1, ix.maps, ix.perm, ix.rowstat, w + L.yb, reinterpret_cast<float4*>(w + L.qstat), ix.tcs,
                                 nullptr, 0, 0, b, Ubits, scnt, surv, DENSE_SURV_CAP, ix.status, ix.diag, ix.xs, Y, 1, ix.d,
                                 ix.d_pad, 1, ix.cdot2, ix.Bn, ix.cabs, debug, st, num_sms,
-                                int(seed), &dn);
+                                int(seed), false, &dn);
             if (rc) return rc;
         }
         u.first = j == 0;

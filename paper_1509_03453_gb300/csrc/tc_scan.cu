@@ -717,7 +717,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
                    const BatchedBuffers& b, uint32_t* Ubits, uint32_t* surv_cnt, uint32_t* surv, int cap,
                    uint32_t* status, unsigned long long* diag, const float* xs, const float* Y, int64_t S, int d,
                    int d_pad, int k, float cdot2, float Bn, float cabs, int debug, cudaStream_t st, int num_sms,
-                   int seed_rows, const TcDense* dense)
+                   int seed_rows, bool uneven, const TcDense* dense)
 {
     TcArgs a{};
     // The k-th best of an item's rows beats the seed's only if the item holds k rows
@@ -759,6 +759,7 @@ int launch_tc_scan(int prec, const void* maps, const uint32_t* perm, const float
     a.cabs = cabs;
     const bool excl = query_src != nullptr;
     if (dense) return launch_tc_scan_dense(maps, a, debug != 0, st, num_sms);
+    if (uneven && (excl || k > 1) && !debug) return launch_tc_scan_uneven(maps, a, k, excl, st, num_sms);
     if (excl) return launch_tc_scan_excl(maps, a, k, debug != 0, st, num_sms);
     if (debug) return launch_tc_scan_debug(maps, a, k, st, num_sms);
     return launch_tc_dp<false, false>(maps, a, k, st, num_sms);

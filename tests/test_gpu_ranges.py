@@ -74,3 +74,25 @@ def test_small_norms(osann, scale):
     Y = rng.standard_normal((1600, 32)).astype(np.float32) * np.float32(scale)
     check(osann, X, Y[:300], 1, 40, 2, False)
     check(osann, X, Y, 3, 1500, 2, True)
+
+
+@pytest.mark.parametrize("d,L,N,k", [(64, 1, 11_028, 2), (32, 2, 40_011, 5), (100, 1, 20_003, 32), (16, 1, 20_003, 1)])
+def test_uneven_norms(osann, d, L, N, k):
+    """Norms over a factor of 100 and more: a candidate bounds the k-th best by its own norm
+    (by the largest, most bounds say nothing and four times as many rows survive)."""
+    rng = np.random.default_rng(d)
+    X = (rng.standard_normal((N, d)) * np.exp(1.2 * rng.standard_normal((N, 1)))).astype(np.float32)
+    Q = 8000 if k == 2 else 2000
+    Y = (rng.standard_normal((Q, d)) * np.exp(1.2 * rng.standard_normal((Q, 1)))).astype(np.float32)
+    idx = osann.Index(to_dev(X), L)
+    Yd = to_dev(Y)
+    ex = dict(query_src=to_dev(rng.integers(0, N, Q)), grid_w=141, radius=3)
+    for P in (7, 120):
+        idx.screen_stats()
+        same(idx.search(Yd, P, k, path="fp16"), idx.search(Yd, P, k, path="plain"))
+        if P == 120 and k == 2:
+            assert idx.screen_stats()["survivors"] < 60 * Q
+        same(idx.search(Yd, P, k, path="fp16", **ex), idx.search(Yd, P, k, path="plain", **ex))
+        same(idx.search(Yd, P, k, path="bf16"), idx.search(Yd, P, k, path="plain"))
+    assert idx.status() == 0
+    idx.close()
