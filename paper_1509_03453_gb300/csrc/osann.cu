@@ -272,6 +272,8 @@ struct osann_index {
     int64_t largest = -1;
     // whether the largest norm is far above the others, when a synchronous build saw it
     bool uneven = false;
+    // whether the largest cone is far above the average, likewise
+    bool skewed = false;
     unsigned __int128 nc_true = 0;
     bool hashed = false;          // second-level table (128-bit cone ids)
     int key_bits = 0;             // significant bits of the 128-bit ids
@@ -503,9 +505,12 @@ static int side_stream(int device, cudaStream_t caller, SideStream* out)
 // the tensor-core screen), or `group` when it is in range (1..128 for the
 // screen; 1..group_size for the fp32 tile scan, whose thread layout fixes the
 // most).
-static int item_group(const osann_index* ix, int mode, int group)
+// (k > 4 over skewed cones: one tile.  The items of the largest cone are what the others
+// wait for, and keeping k bounds of many candidates takes most of their time.)
+static int item_group(const osann_index* ix, int mode, int group, int k)
 {
-    if (tc_mode(mode)) return group >= 1 && group <= TC_GROUP ? group : 2 * TC_GROUP;
+    if (tc_mode(mode))
+        return group >= 1 && group <= TC_GROUP ? group : (ix->skewed && k > 4 ? TC_GROUP : 2 * TC_GROUP);
     const int gmax = group_size(ix->d_pad);
     return group >= 1 && group <= gmax ? group : gmax;
 }
@@ -532,7 +537,7 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
     if (mode == MODE_DENSE) {
         w.dense = take(dense_ws_bytes(Q, ix->d_pad, k));
     } else if (mode != MODE_PLAIN) {
-        const int G = item_group(ix, mode, group);
+        const int G = item_group(ix, mode, group, k);
         const int64_t n = Q * P_eff;
         int64_t mi = n / G + ix->NC + 1;
         if (mi > n) mi = n;
@@ -591,6 +596,14 @@ static double rows_per_cone(const osann_index* ix)
 {
     return double(ix->N) / (ix->occupied > 0 ? double(ix->occupied) : double(ix->NC));
 }
+// Rows of the screen's seed.  The average that tc_seed_rows goes by says nothing of the
+// queries that meet a skewed index's large cones: 1024 for k > 4, as long as a query has
+// them.  (N = 31000, d = 128, one cone of 2131 rows among thin ones, k = 32, 4334 queries:
+// 5380 us by the average, 1980 so and with items of one tile; 1590 before the two-tile screen.)
+static int seed_rows(const osann_index* ix, int64_t Q, int64_t P_eff, int k)
+{
+    return ix->skewed && k > 4 ? 1024 : tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix));
+}
 static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int mode)
 {
     if (!ix->tc_ready[1] || ix->hashed || ix->K || ix->key_mode != OSANN_KEY_SET || ix->L > 4 || ix->N < 8192 ||
@@ -621,7 +634,7 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
         const double work = 2.0 * std::ceil(rows / 128.0) * tile;
         const double full = probes / hit / groups / 128.0;  // a query tile's rows in use
         const double bounds = k <= 1 ? 1.0 : (k <= 2 ? 1.2 : (k <= 4 ? 2.4 : 2.8));
-        const double seeds = tc_seed_rows(Q, k, M);
+        const double seeds = seed_rows(ix, Q, P_eff, k);
         const double seed = double(Q) * seeds * row / seed_rate;
         const double list = ix->NC > 12288 ? 150.0 + probes * 45e-6 : 40.0 + probes * 10e-6;
         const double over = k > 4 ? (k * M / seeds - TC_SURV_CAP) / 15000.0 : 0.0;  // queries that overflow
@@ -1127,6 +1140,7 @@ static int build_impl(const float* d_data, int64_t N, int32_t d, int32_t L, cons
     std::memcpy(&max2, &host_status[2], 4);
     std::memcpy(&mean, &host_status[8], 4);
     ix->uneven = std::sqrt(max2) > 4.0f * mean;
+    ix->skewed = host_status[1] >= 1024 && double(host_status[1]) * double(ix->occupied) > 16.0 * double(N);
     ix->tc_ready[1] = maps_ok;
     *out = ix;
     return OSANN_OK;
@@ -1516,7 +1530,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
         b.n_items_dev = b.item_off + ix->NC;
         b.scan_temp = w + L.scan_temp;
         b.max_items = L.max_items;
-        const int G = item_group(ix, mode, group);
+        const int G = item_group(ix, mode, group, k);
         uint64_t* partial = reinterpret_cast<uint64_t*>(w + L.partial);
         const uint32_t* probes = reinterpret_cast<uint32_t*>(w + L.probes);
         // the query constants and seed bounds (tensor-core paths) and the work
@@ -1535,7 +1549,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                           reinterpret_cast<float4*>(w + L.qstat),
                                           reinterpret_cast<uint32_t*>(w + L.ubits),
                                           reinterpret_cast<uint32_t*>(w + L.scnt), side.st,
-                                          tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)));
+                                          seed_rows(ix, Q, P_eff, k));
             }
         }
         if (!rc) {
@@ -1557,7 +1571,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                     reinterpret_cast<uint32_t*>(w + L.scnt), reinterpret_cast<uint32_t*>(w + L.surv),
                                     TC_SURV_CAP, ix->status, ix->diag, ix->xs, Y, P_eff, ix->d, ix->d_pad, k,
                                     ix->cdot2[prec], ix->Bn, ix->cabs[prec], debug_checks(), st, ix->num_sms,
-                                    tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix)), ix->uneven);
+                                    seed_rows(ix, Q, P_eff, k), ix->uneven);
             }
             if (!rc) {
                 StageScope s(OSANN_STAGE_TC_RERANK, st);

@@ -98,3 +98,32 @@ def test_one_warp_does_not_hold_a_batch(osann):
             times.append(a.elapsed_time(b))
         assert min(times) < 25.0, (Q, times)
     idx.close()
+
+
+def test_screen_over_a_large_cone(osann):
+    """k > 4 on the 16-bit screen, one cone of 6000 rows among thin ones: a long seed and
+    items of one query tile (by the average cone a tenth of a seed, and 5 ms)."""
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1241)
+    X = torch.randn((31_318, 128), generator=g, device="cuda")
+    X[:6263] *= 0.2
+    X[:6263, :3] = 5 + 0.3 * X[:6263, :3].abs()
+    Y = torch.randn((4334, 128), generator=g, device="cuda")
+    Y[:433] = X[:433]
+    idx = osann.Index(X, 2)
+    for P, k in ((122, 32), (30, 5)):
+        ref = idx.search(Y, P, k, path="plain")
+        times = []
+        for _ in range(4):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            ids, d2 = idx.search(Y, P, k, path="fp16")
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b))
+        assert torch.equal(ids, ref[0]) and torch.equal(d2.view(torch.int32), ref[1].view(torch.int32))
+        if k == 32:
+            assert min(times) < 3.6, times
+    assert idx.status() == 0
+    idx.close()
