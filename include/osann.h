@@ -426,10 +426,11 @@ int osann_stats_get(int32_t stage, double *total_ms, int64_t *count);
 int64_t osann_launch_count(void);
 
 /* Test hook for failure detection (the paper has no counterpart): the clock
- * budget, in SM cycles, of the plain scan's waits for its staged copies
- * (OSANN_PATH_PLAIN, and the exact rescan of the tensor-core paths: staged
- * only while a budget is set).  A wait that runs past it gives up: the kernel lets its copies in flight land
- * (under the full budget), writes what it found for the query at hand and
+ * budget, in SM cycles, of the staged per-query scan's waits for its copies.
+ * While a budget is set that scan runs on OSANN_PATH_PLAIN, and as the exact
+ * rescan of the tensor-core paths, in place of the unstaged one, with the
+ * same results as long as no wait runs out.  A wait that runs past the budget
+ * gives up: the kernel lets its copies in flight land (under the full budget), writes what it found for the query at hand and
  * empty results (-1, +inf) for its other queries, and sets
  * OSANN_STATUS_TIMEOUT, which the next osann_status reports; the context
  * stays usable.  0 restores the default of about one second, which no

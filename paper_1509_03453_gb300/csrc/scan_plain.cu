@@ -1,7 +1,8 @@
-// Staged per-query candidate scan (Algorithm 1 with one basis), for the few
-// queries that a screen left to an exact scan, on a device list whose length the
-// host does not know (scan_query.cu is the scan of whole batches): for each
-// query, visit its probed cones in order and compute the exact squared
+// Staged per-query candidate scan (Algorithm 1 with one basis): the form that failure
+// detection is tested on.  The scan that searches run (scan_query.cu, of whole batches
+// and of the queries that a screen leaves) stages nothing and so waits for nothing; this
+// one runs instead while osann_debug_wait_budget has set a budget for its waits, and
+// its results are the same.  For each query, visit its probed cones in order and compute the exact squared
 // Euclidean distance (Eq. 1) to every point of every visited cone, keeping
 // the k nearest by (distance, id).  Distances are fp32 direct differences.
 //
@@ -28,6 +29,8 @@
 // named barrier only when a query ends, to merge their lists.  Every wait is
 // bounded; a wait that runs out sets ST_TIMEOUT and every role drops out
 // after letting its copies in flight land.
+#include <atomic>
+
 #include "osann_device.cuh"
 #include "osann_launch.h"
 
@@ -43,10 +46,10 @@ constexpr int PLAIN_BAR = 1;              // named barrier of the consumer warps
 // Clock budget of the stage waits (a test can shorten it through
 // osann_debug_wait_budget to make the waits run out; the drain of copies
 // still in flight after a timeout always uses the full budget).
-static long long g_plain_wait_budget = WAIT_BUDGET_CYCLES;
+static std::atomic<long long> g_plain_wait_budget{WAIT_BUDGET_CYCLES};
 
 void set_plain_wait_budget(long long cycles) { g_plain_wait_budget = cycles > 0 ? cycles : WAIT_BUDGET_CYCLES; }
-bool plain_wait_budget_set() { return g_plain_wait_budget != WAIT_BUDGET_CYCLES; }
+bool plain_wait_budget_set() { return g_plain_wait_budget.load() != WAIT_BUDGET_CYCLES; }
 
 __device__ __forceinline__ bool excluded_pair(uint32_t id, int64_t src, int64_t grid_w, int radius)
 {
@@ -381,7 +384,7 @@ static int launch_plain_t(const float* xs, const uint32_t* offsets, const uint32
     const int64_t g = grid < cap ? grid : cap;
     kern<<<unsigned(g), PLAIN_THREADS, smem, st>>>(xs, offsets, perm, d_pad, Y, d, probes, P_eff, NC, k, query_src,
                                                    grid_w, radius, qlist, Q, out_ids, out_d, status,
-                                                   g_plain_wait_budget);
+                                                   g_plain_wait_budget.load());
     return count_launch();
 }
 
