@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(128)
         s += __shfl_xor_sync(0xffffffffu, s, o);
         amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     }
-    // fp16 holds |v| < 65504; keep 2 |s y| and the norm terms well inside
-    const bool unscreenable = PREC == 1 && (2.f * sc * amax > 16384.f || sc * sc * s > 32768.f);
+    // fp16 holds |v| < 65504: keep 2 |s y| and the norm terms well inside (bf16: and the sums)
+    const bool unscreenable = PREC == 1 ? 2.f * sc * amax > 16384.f || sc * sc * s > 32768.f : sc * sc * s > 1e30f;
 
     // seed rows: TPR lanes per row (canonical distance, as in the rerank)
     const int n4 = d_pad >> 2;
@@ -400,8 +400,8 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
         s += __shfl_xor_sync(0xffffffffu, s, o);
         amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
     }
-    // fp16 holds |v| < 65504; keep 2 |s y| and the norm terms well inside
-    const bool unscreenable = PREC == 1 && (2.f * sc * amax > 16384.f || sc * sc * s > 32768.f);
+    // fp16 holds |v| < 65504: keep 2 |s y| and the norm terms well inside (bf16: and the sums)
+    const bool unscreenable = PREC == 1 ? 2.f * sc * amax > 16384.f || sc * sc * s > 32768.f : sc * sc * s > 1e30f;
     if (lane == 0) {
         // scaled units: |q'| = s |q|; A' = 2c|q'| + Cabs, inflated by 2^-14
         // (16-bit hi/lo split of |x|) and rounded up to the 16-bit format
@@ -416,8 +416,9 @@ __global__ void __launch_bounds__(32 * PREP_SMALL) tc_query_prep_block_kernel(co
 
 // ---------------------------------------------------------------- rows
 
-// The data scale of the screen: s = 1 for bf16; for fp16 the power of two
-// with s^2 max|x|^2 <= 2^14 (all-zero data: 1).  tcs = (s, s^2, 1/s^2, X), X >= every row norm.
+// The data scale of the screen: for fp16 the power of two with s^2 max|x|^2 <= 2^14
+// (all-zero data: 1); for bf16 1, or that with <= 2^64 where the norms are larger (near
+// fp32's limit the norm columns or the sums would overflow and lose rows).  tcs = (s, s^2, 1/s^2, X), X >= every row norm.
 // The largest finite fp32 norm squared, below 2^128, needs s = 2^-57: s^2 and 1/s^2 are
 // normal numbers, so nothing clamps the exponent from below (a scale too large would
 // make the fp16 norm columns infinite and lose the row).  Above, s stays at 2^40:
@@ -428,10 +429,10 @@ __global__ void tc_scale_kernel(const uint32_t* __restrict__ maxn2_bits, float* 
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int e = 0;
     const float m = __uint_as_float(*maxn2_bits);  // +inf: a row's norm passed the fp32 range (nothing is screened)
-    if (PREC == 1 && m > 0.0f && m < INFINITY) {
+    if (m > 0.0f && m < INFINITY) {
         int x;
         frexpf(m, &x);  // m < 2^x
-        const int t = 14 - x;
+        const int t = PREC == 1 ? 14 - x : (x > 64 ? 64 - x : 0);
         e = t >= 0 ? t / 2 : -((1 - t) / 2);
         e = e > 40 ? 40 : e;
     }

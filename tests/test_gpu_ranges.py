@@ -96,3 +96,18 @@ def test_uneven_norms(osann, d, L, N, k):
         same(idx.search(Yd, P, k, path="bf16"), idx.search(Yd, P, k, path="plain"))
     assert idx.status() == 0
     idx.close()
+
+
+@pytest.mark.parametrize("scale,outlier", [(1e14, 3e4), (1e16, 3e2), (3e9, 1.0), (4e9, 1.0), (1e18, 1.0)])
+def test_bf16_near_the_limit(osann, scale, outlier):
+    """bf16 columns hold fp32's range but the sums of the screen do not: norms up to fp32's
+    limit, on both sides of the line from which they are scaled, and queries beyond."""
+    rng = np.random.default_rng(9)
+    X = rng.standard_normal((9000, 32)).astype(np.float32) * np.float32(scale)
+    X[17] *= np.float32(outlier)
+    Y = rng.standard_normal((200, 32)).astype(np.float32) * np.float32(scale)
+    Y[3] *= np.float32(outlier)
+    Y[5:8] *= np.float32(1e6)
+    Y[7] = 0
+    Y[9] *= np.float32(1e-20)
+    check(osann, X, Y, 1, 40, 3, False)
