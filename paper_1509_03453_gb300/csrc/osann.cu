@@ -589,7 +589,8 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
 // P = 50 .. 1600, k = 2 .. 32: by this rule 0.73 of the time without it, the better of
 // both always 0.68.)
 // Only for the set key with a direct table and L <= 4, whose list positions the
-// dense screen recomputes for a survivor's cone.
+// dense screen recomputes for a survivor's cone; and up to 65536 queries, whose lists and
+// constants take 8.6 KB each (0.56 GB).
 constexpr double DENSE_ITEM_CYCLES = 4000.0;
 // rows of an occupied cone (of a cone, while the occupied ones are not counted)
 static double rows_per_cone(const osann_index* ix)
@@ -614,7 +615,7 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
     const double tile = 80.0 * double((ix->d + 15) / 16 + 1);
     const double probes = double(Q) * double(P_eff);
     const double rows = rows_per_cone(ix), M = rows * double(P_eff), cones = double(ix->N) / rows;
-    // A phase holds eight times the rows before it, so it leaves about 8 k N / M
+    // A phase holds seven times the rows before it, so it leaves about 7 k N / M (here 8)
     // survivors per query (fewer where the probed cones hold nearer rows than the
     // others): past the list's capacity the exact scan would have the work.  (2240 by
     // this count, 85 found, on the descriptor search; on Gaussian data none of 4096
@@ -1764,8 +1765,8 @@ int osann_screen_stats(const osann_index* ix, void* stream, int64_t* out4)
     return OSANN_OK;
 }
 
-// Linear search through the fp16 screen from this many rows up (the seed alone
-// reads 512): below, the fp32 tile scan.
+// Linear search through the fp16 screen from this many rows up (two phases, and a seed
+// of 256 rows): below, the fp32 tile scan.
 constexpr int64_t DENSE_MIN_ROWS = 8192;
 // Queries per pass: a query's survivor list and constants take 8 KB.
 constexpr int64_t DENSE_MAX_Q = 16384;
