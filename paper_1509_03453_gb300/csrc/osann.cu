@@ -712,6 +712,8 @@ static int exact_scan(const osann_index* ix, const float* Y, int64_t Q, const ui
     // part of the whole batch (of a listed one: nothing is known), whichever is most.  At
     // half that line image patches (cones of up to 654 rows among 4.5 on average) would be
     // listed too: 20000 queries, 20 cones, 361 us either way with k = 4, 324 -> 359 with 1.
+    // (An asynchronous build's largest cone is unknown until the next osann_status: until
+    // then its scans take the second launch, 4 to 8 us, to be safe.)
     const double rows = rows_per_cone(ix);
     const double part = sel ? 0.0 : double(Q) * double(P_eff) * rows / (32.0 * ix->num_sms);
     double most = 65536.0 / ix->d_pad;
