@@ -272,7 +272,9 @@ struct osann_index {
     int64_t largest = -1;
     // whether the largest norm is far above the others, when a synchronous build saw it
     bool uneven = false;
-    // whether the largest cone is far above the average, likewise
+    // the largest cone's rows over the average one's, likewise (0: not known), and whether it
+    // is far above it
+    double spread = 0.0;
     bool skewed = false;
     unsigned __int128 nc_true = 0;
     bool hashed = false;          // second-level table (128-bit cone ids)
@@ -568,7 +570,7 @@ static WsLayout ws_layout(const osann_index* ix, int64_t Q, int64_t P_eff, int k
     return w;
 }
 
-// Whether screening every row beats the mode that would be taken otherwise.  All
+// The mode, or the dense screen where screening every row beats it.  All
 // in microseconds on this chip, from these measurements:
 //   dense screen: N / 128 row tiles per 128 queries, 64 cycles per 16 columns at
 //   about 0.8 of the tensor rate; 60 and 40 per phase; seed rows, read at random, at
@@ -605,11 +607,11 @@ static int seed_rows(const osann_index* ix, int64_t Q, int64_t P_eff, int k)
 {
     return ix->skewed && k > 4 ? 1024 : tc_seed_rows(Q, k, double(P_eff) * rows_per_cone(ix));
 }
-static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int mode)
+static int with_dense(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int mode)
 {
     if (!ix->tc_ready[1] || ix->hashed || ix->K || ix->key_mode != OSANN_KEY_SET || ix->L > 4 || ix->N < 8192 ||
         Q > 65536)
-        return false;
+        return mode;
     const double sm_us = ix->num_sms * 2000.0;  // SM cycles per microsecond of the chip
     const double row = 4.0 * ix->d_pad, seed_rate = 2.4e6;
     const double tile = 80.0 * double((ix->d + 15) / 16 + 1);
@@ -621,7 +623,7 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
     // this count, 85 found, on the descriptor search; on Gaussian data none of 4096
     // queries overflowed at 3200, 2 at 5200, a twelfth at 10300.)
     const double found = 8.0 * k * double(ix->N) / M;
-    if (found > 3500.0) return false;
+    if (found > 3500.0) return mode;
     int phases = 1;
     for (int64_t n = ix->N; n > 4096; n >>= 3) ++phases;
     const double dense_us = double((ix->N + 127) / 128) * double((Q + 127) / 128) * tile / sm_us + 60.0 + 40.0 * phases +
@@ -643,7 +645,18 @@ static bool dense_pays(const osann_index* ix, int64_t Q, int64_t P_eff, int k, i
                     (1.0 + (bounds - 1.0) * (full < 1.0 ? full : 1.0)) +
                 (seed > list ? seed : list) + 60.0 + double(Q) * M * row / 4.5e6 * (over < 0.0 ? 0.0 : (over < 1.0 ? over : 1.0));
     }
-    return dense_us < 0.85 * other;
+    if (dense_us >= 0.85 * other) return mode;
+    // Where it beats the cone screen the per-query scan may beat both (few candidates per
+    // query; k > 1 or uneven norms, whose lists overflow): half as slow again as its
+    // bandwidth and its warps' rate (0.2 us per 512 bytes, at most 128 warps per query) say,
+    // and by far, since an average says little of one query's cones; not where one cone is
+    // far above it.  (643 Gaussian, descriptor, clustered, skewed and other searches that
+    // screened every row: 73 take the scan, none slower; the worst before, 4012 queries, 332
+    // thin cones of d = 64, norms over a factor of 100, 2510 -> 67 us.)
+    const double warps = 4864.0 / double(Q) < 128.0 ? (Q < 4864 ? 4864.0 / double(Q) : 1.0) : 128.0;
+    const double stream = probes * rows * row / 6.0e6, chain = M * 0.2 * ix->d_pad / 128.0 / warps;
+    const double scan_us = 1.5 * (stream > chain ? stream : chain) + 20.0;
+    return ix->spread > 0.0 && ix->spread <= 16.0 && scan_us < 0.6 * dense_us ? MODE_PLAIN : MODE_DENSE;
 }
 
 // The mode of a path, the dense screen aside (its workspace grows with Q).
@@ -670,20 +683,19 @@ static int cone_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int path)
 static int choose_mode(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path)
 {
     const int mode = cone_mode(ix, Q, P_eff, path);
-    return path == OSANN_PATH_AUTO && dense_pays(ix, Q, P_eff, k, mode) ? MODE_DENSE : mode;
+    return path == OSANN_PATH_AUTO ? with_dense(ix, Q, P_eff, k, mode) : mode;
 }
 
-// Bytes of the workspace of a search.  Where the dense screen is chosen they hold the
-// cone-major or per-query form too: whether it pays is not monotone in Q, and a
+// Bytes of the workspace of a search.  Where the automatic path leaves the mode that goes
+// by queries per cone they hold that one too: which pays is not monotone in Q, and a
 // workspace sized for the largest batch serves every smaller one, in one form or the
-// other (search_impl).  (256 more: a size that is neither form's names the dense one.)
+// other (search_impl).  (256 more: a size that is no other form's names the dense one.)
 static size_t search_ws_bytes(const osann_index* ix, int64_t Q, int64_t P_eff, int k, int path, int group, int Mv = 1)
 {
     const int mode = choose_mode(ix, Q, P_eff, k, path);
     const size_t need = ws_layout(ix, Q, P_eff, k, mode, group, Mv).total;
-    if (mode != MODE_DENSE) return need;
     const size_t other = ws_layout(ix, Q, P_eff, k, cone_mode(ix, Q, P_eff, path), group, Mv).total;
-    return (need > other ? need : other) + 256;
+    return (need > other ? need : other) + (mode == MODE_DENSE ? 256 : 0);
 }
 
 namespace osann {
@@ -1143,7 +1155,8 @@ static int build_impl(const float* d_data, int64_t N, int32_t d, int32_t L, cons
     std::memcpy(&max2, &host_status[2], 4);
     std::memcpy(&mean, &host_status[8], 4);
     ix->uneven = std::sqrt(max2) > 4.0f * mean;
-    ix->skewed = host_status[1] >= 1024 && double(host_status[1]) * double(ix->occupied) > 16.0 * double(N);
+    ix->spread = double(host_status[1]) * double(ix->occupied) / double(N);
+    ix->skewed = host_status[1] >= 1024 && ix->spread > 16.0;
     ix->tc_ready[1] = maps_ok;
     *out = ix;
     return OSANN_OK;

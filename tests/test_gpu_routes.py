@@ -60,3 +60,26 @@ def test_few_rows_per_query_take_the_scan(osann):
     idx = osann.Index(to_dev(rng.standard_normal((30_000, 64)).astype(np.float32)), 3)
     assert route(idx, 500, 20, 4) == "plain" and route(idx, 70_000, 20, 4) != "dense"
     idx.close()
+
+
+@pytest.mark.parametrize("N,d,L,Q,P,k,sigma", [(13_000, 64, 3, 4000, 330, 5, 1.2), (75_000, 128, 3, 5000, 300, 1, 0.0)])
+def test_scan_where_it_beats_both_screens(osann, N, d, L, Q, P, k, sigma):
+    """Few candidates per query over thin cones: neither screen runs (no survivors counted),
+    although enough queries share a cone for one."""
+    rng = np.random.default_rng(d)
+    X = rng.standard_normal((N, d)) * np.exp(sigma * rng.standard_normal((N, 1)))
+    Y = rng.standard_normal((Q, d)) * np.exp(sigma * rng.standard_normal((Q, 1)))
+    if sigma == 0.0:
+        X, Y = np.abs(X), np.abs(Y)
+    idx = osann.Index(to_dev(X.astype(np.float32)), L)
+    Y = to_dev(Y.astype(np.float32))
+    assert Q * P / idx.occupied() > 8
+    idx.screen_stats()
+    got = idx.search(Y, P, k)
+    assert idx.screen_stats()["survivors"] == 0
+    same(got, idx.search(Y, P, k, path="fp16"))
+    for q in (1, 777):  # and a workspace for all of them serves fewer
+        import torch
+        ws = torch.empty(idx.workspace_size(Q, P, k), dtype=torch.uint8, device="cuda")
+        same(idx.search(Y[:q], P, k, workspace=ws), [t[:q] for t in got])
+    idx.close()
