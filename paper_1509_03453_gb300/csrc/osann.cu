@@ -1565,7 +1565,7 @@ static int search_impl(const osann_index* ix, const float* Y, const int64_t* src
                                           reinterpret_cast<float4*>(w + L.qstat),
                                           reinterpret_cast<uint32_t*>(w + L.ubits),
                                           reinterpret_cast<uint32_t*>(w + L.scnt), side.st,
-                                          seed_rows(ix, Q, P_eff, k));
+                                          seed_rows(ix, Q, P_eff, k), ix->rot != nullptr);
             }
         }
         if (!rc) {

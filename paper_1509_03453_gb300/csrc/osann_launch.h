@@ -176,12 +176,12 @@ int launch_tc_rows(int prec, const float* xs, const float4* rowstat, int64_t N, 
                    float* tcs, void* x16, void* xe16, cudaStream_t st, int num_sms);
 // rows of a query's seed, by batch size, k and the candidates M of a query
 int tc_seed_rows(int64_t Q, int k, double M);
-// probes null: the seed is spread over all N rows
+// probes null: the seed is spread over all N rows; rotated: keyed on a basis of its own
 int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, const uint32_t* probes,
                          int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
                          float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
                          int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
-                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows);
+                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows, bool rotated);
 // Work items of a dense phase (linear search, or a search whose cones are screened
 // together): tile chunks x groups of 256 queries.  The phase's 128-row tiles are
 // mul * (0, 1, 2, ...), or with `skip` mul * (the numbers not divisible by 8);

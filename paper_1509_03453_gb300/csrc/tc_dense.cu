@@ -376,7 +376,7 @@ int launch_dense(const DenseIndex& ix, const float* Y, int64_t Q, int k, const i
     int rc = launch_tc_query_prep(1, Y, Q, ix.d, ix.d_pad, member ? member->seed_probes : nullptr,
                                   member ? member->seed_P : 0, ix.N, ix.offsets, ix.NC, ix.xs, k, ix.cdot2, ix.cabs,
                                   ix.tcs, ix.perm, query_src, grid_w, radius, DENSE_SURV_CAP, w + L.yb,
-                                  reinterpret_cast<float4*>(w + L.qstat), Ubits, scnt, st, int(seed));
+                                  reinterpret_cast<float4*>(w + L.qstat), Ubits, scnt, st, int(seed), false);
     if (rc) return rc;
     cudaMemsetAsync(ovf, 0, 4, st);
     cudaMemsetAsync(counter, 0, 4, st);

@@ -51,17 +51,19 @@ int tc_seed_rows(int64_t Q, int k, double M)
 }
 
 // Queries from which a warp each beats a block each.  The blocks shorten the chain, but
-// keep the chip from the work list beside them, the sooner the less a row's read takes.
-// Whole searches with blocks / warps (us), k = 1: d = 16, 200 / 600 / 1000 queries 90 / 86,
-// 97 / 89, 108 / 93; d = 32, N = 10^6, 300 / 500 / 800: 135 / 136, 132 / 122, 148 / 147; d = 64, N =
-// 4*10^6, 400 / 600 / 1000: 269 / 272, 312 / 259, 412 / 353; d = 50, N = 3.5*10^5, 500 / 700:
-// 157 / 166, 190 / 206; d = 128, 500 / 800 / 1000: 304 / 384, 362 / 386, 369 / 369; fat cones on
-// 16 PCA axes, 997: 432 / 374; thin ones of d = 100, 900: 481 / 541.  k = 10, whose seed is
-// longer: d = 16, 400 / 1000: 166 / 165, 198 / 171; d = 32, 1000: 499 / 520.
-static int prep_small_q(int d_pad, int k, bool fat)
+// keep the chip from the work list beside them: the sooner, the less a row's read takes
+// and the more runs beside them (an index on a basis of its own, one of several searched at
+// a time).  Whole searches with blocks / warps (us), k = 1: d = 16, 200 / 600 / 1000 queries
+// 90 / 86, 97 / 89, 108 / 93; d = 50 on two bases, 871: 415 / 315; d = 64 on two, 552: 426 / 384;
+// d = 128, fat cones on 16 PCA axes, 997: 432 / 374.  On the rows' own basis it is even from
+// d = 32 up: d = 32, N = 10^6, 500 / 800: 132 / 122, 148 / 147; d = 50, N = 2.6*10^6, 756: 331 / 338,
+// N = 3.5*10^5, 700: 190 / 206; d = 64, N = 4*10^6, 700: 366 / 318; d = 128, 500 / 1000: 304 / 384,
+// 369 / 369.  k = 10, whose seed is longer: d = 16, 400 / 1000: 166 / 165, 198 / 171.
+static int prep_small_q(int d_pad, int k, bool fat, bool rotated)
 {
     if (d_pad <= 16) return k > 4 ? 512 : 128;
-    if (d_pad <= 64 && k <= 4) return d_pad <= 32 ? 448 : 512;
+    if (!rotated) return 1024;
+    if (d_pad <= 64 && k <= 4) return 512;
     return fat ? 900 : 1024;
 }
 
@@ -666,7 +668,7 @@ int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, 
                          int64_t P_eff, int64_t N, const uint32_t* offsets, uint32_t NC, const float* xs, int k,
                          float cdot2, float cabs, const float* tcs, const uint32_t* perm, const int64_t* query_src,
                          int64_t grid_w, int radius, int cap, void* Y16, float4* qstat, uint32_t* Ubits,
-                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows)
+                         uint32_t* surv_cnt, cudaStream_t st, int seed_rows, bool rotated)
 {
     if (Q == 0) return 0;
     PrepArgs a{};
@@ -695,7 +697,7 @@ int launch_tc_query_prep(int prec, const float* Y, int64_t Q, int d, int d_pad, 
     a.Ubits = Ubits;
     a.surv_cnt = surv_cnt;
     // d_pad <= 128: one float4 piece per lane
-    const bool small = Q < prep_small_q(d_pad, k, N >= 128 * int64_t(NC)) || !probes;
+    const bool small = Q < prep_small_q(d_pad, k, N >= 128 * int64_t(NC), rotated) || !probes;
 #define OSANN_PREP(PR, KM)                                                                              \
     do {                                                                                                \
         if (small) tc_query_prep_block_kernel<1, PR, KM><<<unsigned(Q), 32 * PREP_SMALL, 0, st>>>(a);   \

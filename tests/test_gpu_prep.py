@@ -17,12 +17,17 @@ def osann():
     return m
 
 
-@pytest.mark.parametrize("d,L,k,line", [(12, 2, 1, 128), (16, 2, 10, 512), (32, 2, 4, 448), (50, 2, 1, 512),
-                                        (64, 1, 5, 900), (64, 2, 5, 1024), (100, 1, 1, 900), (128, 2, 2, 1024)])
-def test_both_sides_of_the_line(osann, d, L, k, line):
+@pytest.mark.parametrize("d,L,k,line,rot", [(12, 2, 1, 128, False), (16, 2, 10, 512, False), (32, 2, 4, 1024, False),
+                                            (50, 2, 1, 512, True), (64, 1, 5, 900, True), (64, 2, 5, 1024, True),
+                                            (100, 1, 1, 900, True), (128, 2, 2, 1024, False)])
+def test_both_sides_of_the_line(osann, d, L, k, line, rot):
     rng = np.random.default_rng(d + k)
     N = 40_003
-    idx = osann.Index(to_dev(rng.standard_normal((N, d)).astype(np.float32)), L)
+    kw = {}
+    if rot:
+        q, _ = np.linalg.qr(rng.standard_normal((d, d)))
+        kw = dict(rot=to_dev(q.astype(np.float32)))
+    idx = osann.Index(to_dev(rng.standard_normal((N, d)).astype(np.float32)), L, **kw)
     Y = to_dev(rng.standard_normal((line, d)).astype(np.float32))
     ex = dict(query_src=to_dev(rng.integers(0, N, line)), grid_w=211, radius=3)
     for P, kw in ((3, {}), (60, ex)):
